@@ -42,7 +42,7 @@ HEADLINE = "cfg3_m4096"
 # the kernel sources it was taken on; an entry whose stamp is not the present sources' is
 # ignored (traffic: null)
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.txt")
-KERNEL_SOURCES = ("iso_kernels.cuh", "iso_api.cu", "iso_schedule.cpp", "iso_internal.h")
+KERNEL_SOURCES = ("iso_kernels.cuh", "iso_words.cuh", "iso_api.cu", "iso_schedule.cpp", "iso_words.cpp", "iso_internal.h")
 
 
 def sources_hash() -> str:

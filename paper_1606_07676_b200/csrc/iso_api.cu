@@ -13,6 +13,7 @@
 #include "iso.h"
 #include "iso_internal.h"
 #include "iso_kernels.cuh"
+#include "iso_words.cuh"
 
 using namespace iso;
 
@@ -219,6 +220,44 @@ void fill_fans(const Request &r, const LaunchPlan &L, FanDev *fd)
     }
 }
 
+// Launches of words: the tables, and the CTA shape for them.  24 warps per SM either way; where the
+// whole launch has fewer warps than that, narrow CTAs spread them over more SMs.
+void plan_words(const Request &r, LaunchPlan &L, uintptr_t inter_addr)
+{
+    build_words(r, L, (uintptr_t)r.send, (uintptr_t)r.recv, inter_addr);
+    const long long groups = (r.comm->P + L.tables.rows_sub - 1) / L.tables.rows_sub;
+    const long long entries = (long long)L.tables.entries.size(), warps = groups * entries;
+    L.threads = warps >= 16ll * r.sm_count ? kWordsThreads : (warps >= 4ll * r.sm_count ? 384 : 128);
+    L.grid = std::max<long long>(1, (warps * 32 + L.threads - 1) / L.threads);
+    L.grid = std::min<long long>(L.grid, (long long)r.sm_count * (kWordsThreads / L.threads));
+    L.grid = std::max<long long>(L.grid, (entries * 32 + L.threads - 1) / L.threads);  // every entry has a warp
+    bool mesh = false;
+    for (int k = 0; k < L.n_used; ++k) mesh = mesh || !r.comm->periodic[L.used_dim[k]];
+    const int depth = L.tables.form == 0 && !mesh ? kWordsDepth : kWordsDepthCoded;
+    L.smem = kWordsPadFront + (size_t)depth * L.threads * 16 + kWordsPadBack;
+}
+
+// Offsets of a words launch's tables from `at` in the request's blob; returns their size.
+size_t words_place(LaunchPlan &L, size_t at)
+{
+    L.units_off = at;
+    L.tiny_off = L.units_off + L.tables.loads.size() * sizeof(LoadDev);
+    L.entries_off = L.tiny_off + L.tables.tiny.size() * sizeof(TinyDev);
+    L.fine_off = L.entries_off + L.tables.entries.size() * sizeof(EntryDev);
+    return L.fine_off - at + (L.tables.fine.size() * sizeof(FineDev) + 15) / 16 * 16;
+}
+
+void fill_words(const LaunchPlan &L, unsigned char *blob)
+{
+    auto put = [&](size_t off, const auto &v) {
+        if (!v.empty()) std::memcpy(blob + off, v.data(), v.size() * sizeof(v[0]));
+    };
+    put(L.units_off, L.tables.loads);
+    put(L.tiny_off, L.tables.tiny);
+    put(L.entries_off, L.tables.entries);
+    put(L.fine_off, L.tables.fine);
+}
+
 // Uploads the lowered schedule and allocates the intermediate buffer.
 int materialise(Request &r)
 {
@@ -282,9 +321,15 @@ int materialise(Request &r)
         plans.push_back(&L);
         for (LaunchPlan &S : L.side) plans.push_back(&S);
     }
+    for (LaunchPlan *plan : plans)
+        if (plan->words) plan_words(r, *plan, (uintptr_t)r.d_inter);
     size_t bytes = 0;
     for (LaunchPlan *plan : plans) {
         LaunchPlan &L = *plan;
+        if (L.words) {
+            bytes += words_place(L, bytes);
+            continue;
+        }
         L.parts_off = bytes;
         bytes += L.parts.size() * sizeof(PartDev);
         L.lookup_off = bytes;
@@ -315,6 +360,10 @@ int materialise(Request &r)
     std::vector<unsigned char> blob(bytes ? bytes : 16, 0);
     for (const LaunchPlan *plan : plans) {
         const LaunchPlan &L = *plan;
+        if (L.words) {
+            fill_words(L, blob.data());
+            continue;
+        }
         int used_index[ISO_MAX_DIMS];
         for (int j = 0; j < ISO_MAX_DIMS; ++j) used_index[j] = -1;
         for (int k = 0; k < L.n_used; ++k) used_index[L.used_dim[k]] = k;
@@ -417,6 +466,15 @@ LaunchDev make_launch_args(const Request &r, const LaunchPlan &L)
     a.parts = reinterpret_cast<const PartDev *>(static_cast<unsigned char *>(r.d_blob) + L.parts_off);
     a.lookup = reinterpret_cast<const uint16_t *>(static_cast<unsigned char *>(r.d_blob) + L.lookup_off);
     a.units = reinterpret_cast<const UnitDev *>(static_cast<unsigned char *>(r.d_blob) + L.units_off);
+    if (L.words) {
+        const unsigned char *blob = static_cast<const unsigned char *>(r.d_blob);
+        a.loads = reinterpret_cast<const LoadDev *>(blob + L.units_off);
+        a.tiny = reinterpret_cast<const TinyDev *>(blob + L.tiny_off);
+        a.entries = reinterpret_cast<const EntryDev *>(blob + L.entries_off);
+        a.fine = reinterpret_cast<const FineDev *>(blob + L.fine_off);
+        a.n_entries = (uint32_t)L.tables.entries.size();
+        a.rows_sub = L.tables.rows_sub;
+    }
     a.buf[ISO_BUF_SEND] = const_cast<unsigned char *>(r.send);
     a.buf[ISO_BUF_RECV] = r.recv;
     a.buf[ISO_BUF_INTER] = r.d_inter;
@@ -544,6 +602,12 @@ unsigned grid_for_rows(const LaunchPlan &L, const LaunchDev &a, int share = 1)
 {
     const long long rows = a.row_hi - a.row_lo;
     if (rows >= a.P && share <= 1) return (unsigned)L.grid;
+    if (L.words) {
+        const long long A = L.tables.rows_sub, groups = (a.row_hi + A - 1) / A - a.row_lo / A;
+        const long long full = std::max<long long>(1, L.grid / std::max(1, share));
+        const long long want = std::min<long long>(full, (groups * a.n_entries * 32 + L.threads - 1) / L.threads);
+        return (unsigned)std::max<long long>(want, ((long long)a.n_entries * 32 + L.threads - 1) / L.threads);
+    }
     if (L.kernel == KERNEL_BULK) return (unsigned)((rows + a.tile_procs - 1) / a.tile_procs);
     const long long groups = (rows + L.rows_per_pass - 1) / L.rows_per_pass;
     // `share` launches of this kind run side by side: each takes its part of the CTA slots
@@ -560,12 +624,12 @@ constexpr int kMaxDynamicSmem = 227 * 1024;  // dynamic shared memory a CTA can 
 size_t table_bytes(const LaunchDev &a) { return (size_t)a.tab_iters * a.rows_per_pass * a.tab_stride * sizeof(uint32_t); }
 
 template <typename Kernel>
-cudaError_t launch_kernel(Kernel kernel, const LaunchPlan &L, const LaunchDev &a, cudaStream_t stream, bool dependent)
-{
+cudaError_t launch_kernel(Kernel kernel, const LaunchPlan &L, const LaunchDev &a, cudaStream_t stream, bool dependent, size_t table)
+{   // table: bytes of a coordinate table behind the plan's shared memory
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid_for_rows(L, a, a.grid_share));
     cfg.blockDim = dim3((unsigned)L.threads);
-    cfg.dynamicSmemBytes = L.smem + table_bytes(a);
+    cfg.dynamicSmemBytes = L.smem + table;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     // programmatic dependent launch: the kernel may start while its predecessor in the stream
@@ -579,7 +643,7 @@ cudaError_t launch_kernel(Kernel kernel, const LaunchPlan &L, const LaunchDev &a
 
 // Wide CTAs need more dynamic shared memory than the default limit: opt in once per kernel.
 template <typename Kernel>
-cudaError_t launch_wide(Kernel kernel, const LaunchPlan &L, const LaunchDev &a, cudaStream_t stream, bool dependent)
+cudaError_t launch_wide(Kernel kernel, const LaunchPlan &L, const LaunchDev &a, cudaStream_t stream, bool dependent, size_t table)
 {
     // (device, kernel) pairs that already have the larger limit: the attribute is per device
     static std::vector<std::pair<int, const void *>> opted_in;
@@ -596,7 +660,7 @@ cudaError_t launch_wide(Kernel kernel, const LaunchPlan &L, const LaunchDev &a, 
             opted_in.push_back(key);
         }
     }
-    return launch_kernel(kernel, L, a, stream, dependent);
+    return launch_kernel(kernel, L, a, stream, dependent, table);
 }
 
 // The hybrid kernel: the vector side's threads plus one warp for the bulk side.
@@ -637,9 +701,53 @@ template <int W, int NU, bool MESH, bool COMPACT>
 cudaError_t launch_rows_wide(bool tab, const LaunchPlan &L, const LaunchDev &a, cudaStream_t stream, bool dependent)
 {
     if constexpr (!MESH && (COMPACT || NU <= 2)) {
-        if (tab) return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, true>, L, a, stream, dependent);
+        if (tab) return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, true>, L, a, stream, dependent, table_bytes(a));
     }
-    return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, false>, L, a, stream, dependent);
+    return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, false>, L, a, stream, dependent, 0);
+}
+
+// Launches of words: the coordinate table where it fits beside the rings of the CTAs of an SM.
+template <int FORM, bool MESH, int NU>
+cudaError_t launch_words_nu(const LaunchPlan &L, LaunchDev &a, cudaStream_t stream, bool dependent)
+{
+    const long long A = a.rows_sub, nw = L.threads / 32, grid = grid_for_rows(L, a, a.grid_share);
+    const long long groups = (a.row_hi + A - 1) / A - a.row_lo / A;
+    const long long slots = grid * nw / a.n_entries;
+    const long long iters = (groups + slots - 1) / slots, per_cta = (nw - 1) / a.n_entries + 2;
+    const size_t words = NU <= 1 ? 1 : (NU == 2 ? 2 : (NU <= 4 ? 4 : 8));
+    const size_t table = (size_t)(iters * per_cta * A) * words * sizeof(uint32_t);
+    if (L.n_used > 0 && (L.smem + table + 1024) * (size_t)(kWordsThreads / L.threads) <= 228 * 1024) {
+        a.tab_iters = (uint32_t)iters;
+        a.tab_slots = (uint32_t)per_cta;
+        return launch_wide(iso_gather_words<FORM, MESH, NU, true>, L, a, stream, dependent, table);
+    }
+    return launch_wide(iso_gather_words<FORM, MESH, ISO_MAX_DIMS, false>, L, a, stream, dependent, 0);
+}
+
+template <int FORM, bool MESH>
+cudaError_t launch_words_form(const LaunchPlan &L, LaunchDev &a, cudaStream_t stream, bool dependent)
+{
+    switch (L.n_used) {
+    case 0:
+    case 1: return launch_words_nu<FORM, MESH, 1>(L, a, stream, dependent);
+    case 2: return launch_words_nu<FORM, MESH, 2>(L, a, stream, dependent);
+    case 3: return launch_words_nu<FORM, MESH, 3>(L, a, stream, dependent);
+    case 4: return launch_words_nu<FORM, MESH, 4>(L, a, stream, dependent);
+    default: return launch_words_nu<FORM, MESH, ISO_MAX_DIMS>(L, a, stream, dependent);
+    }
+}
+
+cudaError_t launch_words(const LaunchPlan &L, LaunchDev &a, cudaStream_t stream, bool dependent)
+{
+    if (a.n_entries == 0) return cudaSuccess;
+    const int form = L.tables.form;
+    if (a.mesh_mask)
+        return form == 0   ? launch_words_form<0, true>(L, a, stream, dependent)
+               : form == 1 ? launch_words_form<1, true>(L, a, stream, dependent)
+                           : launch_words_form<2, true>(L, a, stream, dependent);
+    return form == 0   ? launch_words_form<0, false>(L, a, stream, dependent)
+           : form == 1 ? launch_words_form<1, false>(L, a, stream, dependent)
+                       : launch_words_form<2, false>(L, a, stream, dependent);
 }
 
 int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool dependent, long long row_lo = 0,
@@ -664,9 +772,9 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
     if (inter_row_base && a.buf[ISO_BUF_INTER]) a.buf[ISO_BUF_INTER] -= inter_row_base * r.inter_stride;
     cudaError_t e;
     if (L.kernel == KERNEL_BULK) {
-        e = launch_kernel(iso_gather_bulk, L, a, stream, dependent);
+        e = launch_kernel(iso_gather_bulk, L, a, stream, dependent, 0);
     } else if (L.kernel == KERNEL_FAN) {
-        e = launch_wide(iso_fan_rows<kWideDepth>, L, a, stream, dependent);
+        e = launch_wide(iso_fan_rows<kWideDepth>, L, a, stream, dependent, 0);
     } else if (!L.side.empty()) {
         // mixed-width launch with a bulk side: vector warps + one bulk warp per CTA
         LaunchDev sd = make_launch_args(r, L.side[0]);
@@ -691,9 +799,8 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
             : L.n_used == 2 ? (tab ? launch_hybrid(iso_gather_rows_hybrid<kHybridDepth, 2, true>, L, a, sd, smem, stream, dependent)
                                    : launch_hybrid(iso_gather_rows_hybrid<kHybridDepth, 2, false>, L, a, sd, smem, stream, dependent))
                             : launch_hybrid(iso_gather_rows_hybrid<kHybridDepth, 3, false>, L, a, sd, smem, stream, dependent);
-    } else if (L.width > 0 && L.width < 4) {
-        e = L.width == 2 ? launch_kernel(iso_gather_rows_reg<2, 4>, L, a, stream, dependent)
-                         : launch_kernel(iso_gather_rows_reg<1, 4>, L, a, stream, dependent);
+    } else if (L.words) {
+        e = launch_words(L, a, stream, dependent);
     } else {
         // kernels specialised on the number of shifted dimensions; meshes take the general one
         // (with compact unit descriptors: on the dimensions one unit is shifted along)
@@ -705,7 +812,7 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
         // dimension, and on the compact last phase of 16-byte blocks; the one-pass direct
         // schedules, three or more wrap tests per row, are bound by the latency of their
         // scattered loads and gain nothing, so they keep the divisions)
-        if ((L.width == 16 || L.width == 0) && L.threads > 256 && L.n_used > 0 && r.knobs.coord_table &&
+        if (L.threads > 256 && L.n_used > 0 && r.knobs.coord_table &&
             (L.compact || nu <= 2) && !a.mesh_mask) {
             const long long groups = (a.row_hi - a.row_lo + L.rows_per_pass - 1) / L.rows_per_pass;
             const long long grid = grid_for_rows(L, a, a.grid_share) / std::max(1, L.col_split);  // CTAs that share the rows
@@ -715,9 +822,8 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
             if (!tab) a.tab_iters = 0;
         }
 #define ISO_ROWS(W, NU, MESH, COMPACT)                                                                          \
-    e = ((W == 16 || W == 0) && L.threads > 256)                                                                \
-            ? launch_rows_wide<(W == 0 ? 0 : 16), NU, MESH, COMPACT>(tab, L, a, stream, dependent)             \
-            : launch_kernel(iso_gather_rows<W, kVecDepth, NU, MESH, COMPACT>, L, a, stream, dependent)
+    e = L.threads > 256 ? launch_rows_wide<W, NU, MESH, COMPACT>(tab, L, a, stream, dependent)                  \
+                        : launch_kernel(iso_gather_rows<W, kVecDepth, NU, MESH, COMPACT>, L, a, stream, dependent, 0)
 #define ISO_ROWS_W(W)                                                            \
     do {                                                                         \
         if (a.mesh_mask) ISO_ROWS(W, ISO_MAX_DIMS, true, false);                 \
@@ -731,10 +837,7 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
         else if (nu == 3) ISO_ROWS(W, 3, false, false);                          \
         else ISO_ROWS(W, ISO_MAX_DIMS, false, false);                            \
     } while (0)
-        if (L.width == 0) ISO_ROWS_W(0);
-        else if (L.width == 16) ISO_ROWS_W(16);
-        else if (L.width == 8) ISO_ROWS_W(8);
-        else ISO_ROWS_W(4);
+        ISO_ROWS_W(16);
 #undef ISO_ROWS_W
 #undef ISO_ROWS
     }
@@ -2124,6 +2227,11 @@ extern "C" int Iso_neighbor_alltoall_static(int d, const int dims[], int s, cons
     int64_t table_bytes = 0;
     for (LaunchPlan &L : r.launches) {
         if (L.kernel != KERNEL_VEC) return ISO_ERR_STATE;
+        if (L.words) {
+            plan_words(r, L, (uintptr_t)scratch);
+            table_bytes += (int64_t)words_place(L, (size_t)table_bytes);
+            continue;
+        }
         L.units_off = (size_t)table_bytes;
         table_bytes += (int64_t)L.units_per_proc * (int64_t)sizeof(UnitDev);
     }
@@ -2131,7 +2239,10 @@ extern "C" int Iso_neighbor_alltoall_static(int d, const int dims[], int s, cons
 
     // unit tables, built on the host and copied behind the intermediate buffer
     std::vector<unsigned char> blob((size_t)table_bytes, 0);
-    for (const LaunchPlan &L : r.launches) fill_units(r, L, reinterpret_cast<UnitDev *>(blob.data() + L.units_off));
+    for (const LaunchPlan &L : r.launches) {
+        if (L.words) fill_words(L, blob.data());
+        else fill_units(r, L, reinterpret_cast<UnitDev *>(blob.data() + L.units_off));
+    }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     unsigned char *tables = scratch + inter_bytes;
     // The copy reads `blob`, which dies with this call: outside a stream capture the runtime

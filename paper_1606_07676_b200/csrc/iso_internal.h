@@ -78,6 +78,78 @@ constexpr int kWideDepth = 12;      // the same in CTAs of more than 256 threads
 constexpr int kHybridDepth = 6;     // the same for the vector warps of a hybrid launch (most of the shared memory stages bulk copies)
 constexpr size_t kHybridStageBytes = 128 * 1024;  // staging area of the bulk warps of a hybrid launch
 
+// ---- launches of words (iso_words.cuh) ------------------------------------------------------
+// Tables of a launch whose blocks are not made of whole, equally placed 16-byte units.  A chunk is
+// what one warp moves per row (or group of rows): at most 32 aligned 16-byte words to load, and
+// what they are stored as.
+
+// One word to load, by lane.  In a whole or placed chunk (and in form 2) the lane may also store one.
+struct alignas(16) LoadDev {
+    long long src_term;      // rank_delta * source stride + offset of the block (form 0: of the aligned word)
+    uint32_t len;            // bytes of the block (0: this lane loads nothing)
+    int32_t word;            // forms 1, 2: index of this word, counted from the one that holds the block's first byte;
+                             // placed chunk: which bytes of the destination word this lane's word holds
+    int32_t c[ISO_MAX_DIMS]; // shift (non-periodic dimension: check value) along the launch's used dimensions
+    long long dst_term;      // whole or placed chunk: destination offset of the word; form 2: of the block
+    uint8_t src_buf, dst_buf;
+    uint8_t sub;             // which of the rows of the group
+    uint8_t stores;          // whole or placed chunk, form 2: this lane stores a word
+    uint8_t second, third;   // placed chunk: lanes that hold more bytes of the word (this lane itself: none)
+    uint8_t pad[2];
+};
+static_assert(sizeof(LoadDev) == 64, "load descriptors are read as four 16-byte words");
+
+// One aligned 4- or 8-byte word to store, put together from the chunk's loaded bytes.  A place counts
+// from 16 bytes in front of the chunk's first slot, so that it is never negative.
+struct alignas(8) FineDev {
+    uint32_t a;  // place q0 (10 bits) and lane0 (5) of the first block, q1 (10) and lane1 (5) of the second:
+                 // the byte of the block that falls on the word's byte 0, and a lane that loads the block
+    uint32_t b;  // offset in units of 4 bytes behind the chunk's first word (16 bits), bytes from the first (4)
+                 // and from the second block (4); no bytes: no word
+};
+// The same where more than two blocks meet in a 4-byte word: place (10) and lane (5) of every byte.
+struct alignas(16) TinyDev {
+    uint32_t a, b;  // bytes 0 and 1, bytes 2 and 3
+    uint32_t off;   // offset in units of 4 bytes behind the chunk's first word
+    uint32_t mask;
+};
+
+// How a chunk is stored.  WHOLE (form 0): every lane stores the word it has loaded.  PLACED (form 0):
+// likewise, merged where need be with the words of one or two other lanes, every byte having the same
+// place in both.  ONE4, ONE8: 4- or 8-byte words, each out of one block.  TWO: 4-byte words out of one
+// or two blocks.  TINY: likewise, byte by byte.
+enum { CHUNK_WHOLE = 0, CHUNK_PLACED = 1, CHUNK_ONE4 = 2, CHUNK_ONE8 = 3, CHUNK_TWO = 4, CHUNK_TINY = 5 };
+
+// Which warp does what: warp g of the grid works on entry g mod n, of the row groups dealt to it on
+// those with index `turn` mod `turns`.  A chunk that costs more instructions per row has more entries.
+struct alignas(16) EntryDev {
+    uint32_t chunk, turn, turns;
+    uint32_t first;      // index of the chunk's first FineDev or TinyDev (32 per pass)
+    uint8_t passes;      // 32-word passes over its 4- or 8-byte words; placed chunk: most sources of a word
+    uint8_t kind;        // CHUNK_*
+    uint8_t dst_buf;
+    uint8_t pad[5];
+    long long dst_term;  // its first 4- or 8-byte word, from the (aligned down) start of the row group
+};
+static_assert(sizeof(EntryDev) == 32, "entries are read as two 16-byte words");
+
+struct WordTables {
+    int form = 0;          // 0: all alignments the same for every row, 1: worked out per row, 2: likewise, long blocks
+    uint32_t rows_sub = 1; // forms 0, 1: rows described together (a row group)
+    std::vector<LoadDev> loads;     // 32 per chunk
+    std::vector<EntryDev> chunks;   // one per chunk (turn 0 of 1), before they are dealt to warps
+    std::vector<FineDev> fine;
+    std::vector<TinyDev> tiny;
+    std::vector<EntryDev> entries;
+};
+constexpr int64_t kWordsLongBlock = 64;       // mean block length from which form 2 replaces form 1
+constexpr int64_t kWordsMostGroup = 32 << 10; // bytes of a row group that the tables describe at most
+constexpr int kWordsDepth = 16;               // words in flight per lane, as many as fit beside a coordinate table ...
+constexpr int kWordsDepthCoded = 12;          // ... and where the codes of the stages have to fit into 64 bits
+constexpr int kWordsThreads = 768;            // threads of a CTA, one per SM (fewer where a launch is small)
+constexpr int kWordsPasses = 4;               // passes over a chunk's words at most
+constexpr uint32_t kWordsPadFront = 16, kWordsPadBack = 48;  // shared memory around the ring that a shifted read may touch
+
 struct LaunchPlan {
     int kernel = KERNEL_VEC;
     int width = 16;       // bytes per unit (vector kernel; 0: mixed, every piece has its own); chunk bytes (bulk kernel)
@@ -101,9 +173,11 @@ struct LaunchPlan {
     int col_split = 1;     // vector kernel: column chunks of a row longer than a CTA, one CTA per chunk and row (1: none)
     std::vector<LaunchPlan> side;  // mixed-width vector launch: at most one bulk-copy plan for the long bodies of its rows,
                                    // run by one extra warp of the same CTAs
+    bool words = false;           // vector launch whose blocks are not whole, equally placed 16-byte units
+    WordTables tables;            // its tables (build_words)
     std::vector<FanParent> fans;  // KERNEL_FAN: the launch as parents and their destinations (parts: the same copies, one per destination)
     // byte offsets of this launch's tables inside the request's device blob
-    size_t parts_off = 0, lookup_off = 0, units_off = 0;
+    size_t parts_off = 0, lookup_off = 0, units_off = 0, fine_off = 0, tiny_off = 0, entries_off = 0;
 };
 
 // Experiment knobs, read from the environment ONCE, when a request is created, so that a
@@ -208,6 +282,9 @@ int build_schedule(Request &r);
 // Splits parts into aligned pieces, groups them into kernel launches and fills the launch
 // geometry.  `send_addr` / `recv_addr` / `inter_addr` are only used for their alignment.
 int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr_t inter_addr);
+
+// Fills L.tables for the lowered launch L (L.words).  The addresses are only used for their alignment.
+void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t recv_addr, uintptr_t inter_addr);
 
 // Checks the executed parts for hazards: every range inside its buffer, no write to the send
 // buffer, and within a phase no written range overlapping another written or any read range.

@@ -1059,7 +1059,8 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                 // a vector launch holds at most kMaxVecUnits unit positions per process (each
                 // gets a descriptor): cut longer lists, splitting a piece at a unit boundary
                 if (kernel == KERNEL_VEC) {
-                    const int64_t cap = kMaxVecUnits;
+                    // (a launch of words describes 16-byte words whatever the width of its pieces)
+                    const int64_t cap = width == 16 || !longs.empty() ? (int64_t)kMaxVecUnits : (int64_t)1 << 24;
                     std::vector<Piece> cut;
                     std::vector<size_t> bounds(1, 0);
                     int64_t used_units = 0;
@@ -1117,7 +1118,8 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                     {
                         bool torus = true;
                         for (int k = 0; k < L.n_used; ++k) torus = torus && c.periodic[L.used_dim[k]];
-                        L.compact = kernel == KERNEL_VEC && (width >= 4 || width == 0) && L.n_used > 3 && L.max_nnz < L.n_used &&
+                        L.words = kernel == KERNEL_VEC && width != 16 && longs.empty();
+                        L.compact = kernel == KERNEL_VEC && !L.words && L.n_used > 3 && L.max_nnz < L.n_used &&
                                     torus && !r.persistent;  // (the pipelined one-launch kernel does take compact launches)
                     }
                     // geometry
@@ -1125,14 +1127,21 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                     int64_t tp;
                     int64_t grid;
                     uint32_t whole_row_slots = 1;  // rows a CTA would hold if it covered whole rows
-                    if (kernel == KERNEL_VEC) {
-                        // a row slot covers up to 256 unit positions; short rows share a CTA
-                        // 16-byte launches with long rows use CTAs of up to 1024 threads
+                    if (L.words) {
+                        // (tables, thread count and grid: build_words, when the buffers are placed)
+                        int64_t bytes = 0;
+                        for (size_t k = lo; k < hi; ++k) bytes += cls[k].p.len;
+                        const int64_t warps = std::max<int64_t>(1, (bytes + 415) / 416);  // about 26 words of a chunk are useful
+                        L.threads = kWordsThreads;
+                        L.rows_hint = std::max<int64_t>(1, (int64_t)r.sm_count * (kWordsThreads / 32) / warps);
+                        grid = r.sm_count;
+                        tp = 1;
+                    } else if (kernel == KERNEL_VEC) {
                         // 16-byte and mixed launches run in CTAs of up to 1024 threads, one per SM
                         // (measured against four CTAs of 256 threads: 36.1 against 40.3 microseconds
                         // per all-to-all on the 32^3 torus, 161 against 184 on the 8^5 torus);
                         // ISO_VEC_THREADS=256 or 512 selects the narrower shapes
-                        uint32_t max_threads = (width == 16 || width == 0) ? 1024 : 256;
+                        uint32_t max_threads = 1024;
                         if (!longs.empty())  // leave a warp and the staging area to the bulk side
                             max_threads = std::min<uint32_t>((uint32_t)(1024 - side_lanes),
                                                              (uint32_t)((227 * 1024 - side_smem - 16 * 1024) / (kHybridDepth * 16) / 32 * 32));
@@ -1198,7 +1207,7 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                     L.smem = (size_t)L.n_used * (size_t)tp * sizeof(uint32_t);
                     if (kernel == KERNEL_VEC) {
                         const size_t depth = !longs.empty() ? kHybridDepth : (L.threads > 256 ? kWideDepth : kVecDepth);
-                        L.smem = width >= 4 ? depth * L.threads * width : (width == 0 ? depth * L.threads * 16 : 0);
+                        L.smem = L.words ? 0 : depth * L.threads * 16;
                     }
                     if (kernel == KERNEL_BULK)
                         L.smem = (L.smem + 15) / 16 * 16 + (size_t)L.threads * 2 * (size_t)unit + (size_t)L.threads * 2 * 8;

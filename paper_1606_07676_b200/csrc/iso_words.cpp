@@ -1,0 +1,416 @@
+// Tables of the launches that move blocks of any size and placement in aligned 16-byte words
+// (iso_words.cuh): which words a warp loads, which words it stores, and which bytes of the
+// former make up the latter.
+#include <algorithm>
+#include <cstring>
+#include <numeric>
+
+#include "iso_internal.h"
+
+namespace iso {
+
+namespace {
+
+// A run of bytes that is contiguous on both sides (the lowering may have cut it into pieces).
+struct Block {
+    int src_buf, dst_buf;
+    int64_t src_off, dst_off, len;
+    const Part *p;  // shift and check values
+};
+
+std::vector<Block> merged_blocks(const LaunchPlan &L, int d)
+{
+    std::vector<Block> b;
+    for (const LoweredPart &lp : L.parts)
+        b.push_back(Block{lp.p.src_buf, lp.p.dst_buf, lp.p.src_off, lp.p.dst_off, lp.p.len, &lp.p});
+    std::sort(b.begin(), b.end(), [](const Block &x, const Block &y) {
+        return x.dst_buf != y.dst_buf ? x.dst_buf < y.dst_buf : x.dst_off < y.dst_off;
+    });
+    size_t n = 0;
+    for (size_t k = 0; k < b.size(); ++k) {
+        if (n > 0) {
+            Block &a = b[n - 1];
+            if (a.dst_buf == b[k].dst_buf && a.src_buf == b[k].src_buf && a.dst_off + a.len == b[k].dst_off &&
+                a.src_off + a.len == b[k].src_off && std::memcmp(a.p->shift, b[k].p->shift, sizeof(int) * d) == 0 &&
+                std::memcmp(a.p->check, b[k].p->check, sizeof(int) * d) == 0) {
+                a.len += b[k].len;
+                continue;
+            }
+        }
+        b[n++] = b[k];
+    }
+    b.resize(n);
+    return b;
+}
+
+// The places inside a 16-byte word at which a block may start, over all rows.
+struct Placement {
+    int64_t lowest, highest;
+};
+Placement placement(int64_t addr, int64_t stride)
+{
+    const int64_t g = std::gcd<int64_t>(16, stride);
+    const int64_t lowest = addr & (g - 1);  // g is a power of two
+    return Placement{lowest, lowest + 16 - g};
+}
+
+// Deals warps to the chunks in proportion to what a row costs in them, so that all warps of a launch
+// are done at the same time.  The weights are measured, in units of which a row of whole words costs
+// 50: with equal shares the 27-point stencil of faces, edges and corners took 222 microseconds in three
+// phases on a mesh, with these 159.
+void deal(WordTables &T)
+{
+    std::vector<uint32_t> cost;
+    for (const EntryDev &ck : T.chunks) {
+        uint32_t c = 50;
+        if (ck.kind == CHUNK_PLACED) c = 60;
+        if (ck.kind == CHUNK_ONE4 || ck.kind == CHUNK_ONE8) c = 40 + 8u * ck.passes;
+        if (ck.kind == CHUNK_TWO) c = 75 + 45u * ck.passes;
+        if (ck.kind == CHUNK_TINY) c = 75 + 90u * ck.passes;
+        cost.push_back(c);
+    }
+    T.entries.clear();
+    if (cost.empty()) return;
+    const uint32_t least = *std::min_element(cost.begin(), cost.end());
+    const uint32_t greatest = *std::max_element(cost.begin(), cost.end());
+    const uint32_t unit = 4 * greatest <= 5 * least ? greatest : least / 4;  // entries in quarters of the cheapest chunk
+    for (uint32_t k = 0; k < cost.size(); ++k) {
+        const uint32_t turns = std::max<uint32_t>(1, (cost[k] + unit / 2) / unit);
+        for (uint32_t t = 0; t < turns; ++t) {
+            EntryDev e = T.chunks[k];
+            e.chunk = k;
+            e.turn = t;
+            e.turns = turns;
+            T.entries.push_back(e);
+        }
+    }
+    // the entries of one chunk apart from one another, so that the warps that work on a row at the
+    // same time are neighbours
+    std::stable_sort(T.entries.begin(), T.entries.end(), [](const EntryDev &x, const EntryDev &y) {
+        return (uint64_t)x.turn * y.turns < (uint64_t)y.turn * x.turns;
+    });
+}
+
+struct Run { size_t block; uint32_t sub; int64_t x; int begin, n; };  // bytes x .. x+n of a block, at `begin` in a word
+
+// Collects words of 4 or 8 bytes into chunks: one is closed when the next word would need more than 32
+// loads, or be one too many.
+struct FineChunks {
+    WordTables &T;
+    const uint8_t plainest;  // the chunk's kind as long as every word has one block (TWO: two)
+    EntryDev open{};
+    size_t n_loads = 0;
+    size_t last_block = SIZE_MAX, last_slot = 0;  // block (and row) the last loads belong to
+    uint32_t last_sub = 0;
+    int64_t first_k = 0, last_k = 0;
+    struct Word { int64_t at; std::vector<Run> runs; std::vector<std::pair<uint32_t, uint32_t>> places; };  // (place, lane) per run
+    std::vector<Word> words;
+
+    // range(run, k0, k1): the run's words, counted from the one that holds the block's first byte at its
+    // lowest place, which is returned; load(run, k): the descriptor of its word k
+    template <typename Range, typename Load>
+    void add(int buf, int64_t at, const std::vector<Run> &runs, Range range, Load load)
+    {
+        size_t need = 0, lb = last_block;
+        uint32_t ls = last_sub;
+        int64_t lk = last_k;
+        for (const Run &q : runs) {
+            int64_t k0, k1;
+            range(q, k0, k1);
+            const bool same = lb == q.block && ls == q.sub && k0 <= lk + 1;
+            need += (size_t)(same ? std::max<int64_t>(0, k1 - lk) : k1 - k0 + 1);
+            lk = same ? std::max(lk, k1) : k1;
+            lb = q.block;
+            ls = q.sub;
+        }
+        if (words.size() == 32 * kWordsPasses || (!words.empty() && (open.dst_buf != buf || at - words[0].at >= 4 << 16)) ||
+            n_loads + need > 32)
+            close();
+        if (words.empty()) open.kind = plainest;
+        open.dst_buf = (uint8_t)buf;
+        Word w{at, runs, {}};
+        for (const Run &q : runs) {
+            int64_t k0, k1;
+            const int64_t base = range(q, k0, k1);
+            if (last_block != q.block || last_sub != q.sub || k0 > last_k + 1) {
+                last_block = q.block;
+                last_sub = q.sub;
+                last_slot = n_loads;
+                first_k = k0;
+                last_k = k0 - 1;
+            }
+            while (last_k < k1) {
+                T.loads.push_back(load(q, ++last_k));
+                ++n_loads;
+            }
+            w.places.push_back({(uint32_t)(16 + 16 * ((int64_t)last_slot - first_k) + q.x - q.begin + base), (uint32_t)last_slot});
+        }
+        if (runs.size() > 2) open.kind = CHUNK_TINY;
+        words.push_back(w);
+    }
+
+    void close()
+    {
+        if (words.empty()) return;
+        const bool tiny = open.kind == CHUNK_TINY;
+        open.first = (uint32_t)(tiny ? T.tiny.size() : T.fine.size());
+        open.passes = (uint8_t)((words.size() + 31) / 32);
+        open.dst_term = words[0].at;
+        for (const Word &w : words) {
+            FineDev f{};
+            TinyDev t{};
+            uint32_t mask[2] = {0, 0}, byte[4] = {0, 0, 0, 0};
+            for (size_t j = 0; j < w.runs.size(); ++j) {
+                const Run &q = w.runs[j];
+                const uint32_t place = w.places[j].first, lane = w.places[j].second;
+                for (int e = q.begin; e < q.begin + q.n && e < 4; ++e) {
+                    byte[e] = (place + (uint32_t)e) | lane << 10;
+                    t.mask |= 1u << e;
+                    if (j < 2) mask[j] |= 1u << e;
+                }
+                if (j < 2) f.a |= (place | lane << 10) << (15 * j);
+            }
+            t.a = byte[0] | byte[1] << 15;
+            t.b = byte[2] | byte[3] << 15;
+            t.off = (uint32_t)((w.at - words[0].at) / 4);
+            f.b = t.off | mask[0] << 16 | mask[1] << 20;
+            if (tiny) T.tiny.push_back(t);
+            else T.fine.push_back(f);
+        }
+        T.fine.resize((T.fine.size() + 31) / 32 * 32, FineDev{});
+        T.tiny.resize((T.tiny.size() + 31) / 32 * 32, TinyDev{});
+        T.loads.resize((T.loads.size() + 31) / 32 * 32, LoadDev{});
+        T.chunks.push_back(open);
+        open = EntryDev{};
+        words.clear();
+        n_loads = 0;
+        last_block = SIZE_MAX;
+    }
+};
+
+}  // namespace
+
+void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t recv_addr, uintptr_t inter_addr)
+{
+    const Comm &c = *r.comm;
+    const int64_t stride[3] = {r.send_stride, r.recv_stride, r.inter_stride};
+    const int64_t addr[3] = {(int64_t)(send_addr & 15), (int64_t)(recv_addr & 15), (int64_t)(inter_addr & 15)};
+    WordTables &T = L.tables;
+    T = WordTables{};
+    int used_index[ISO_MAX_DIMS];
+    for (int j = 0; j < ISO_MAX_DIMS; ++j) used_index[j] = -1;
+    for (int k = 0; k < L.n_used; ++k) used_index[L.used_dim[k]] = k;
+
+    const std::vector<Block> blocks = merged_blocks(L, c.d);
+    bool fixed = true;             // every stride and base address is a multiple of 16
+    bool by4 = true, by8 = true;   // every address is a multiple of 4, of 8
+    int64_t rows = 1, bytes = 0, words = 0;
+    for (const Block &b : blocks) {
+        for (int q : {b.src_buf, b.dst_buf}) fixed = fixed && stride[q] % 16 == 0 && addr[q] == 0;
+        for (int64_t v : {stride[b.src_buf], stride[b.dst_buf], addr[b.src_buf], addr[b.dst_buf], b.src_off, b.dst_off, b.len}) {
+            by4 = by4 && v % 4 == 0;
+            by8 = by8 && v % 8 == 0;
+        }
+        rows = std::max<int64_t>(rows, 16 / std::gcd<int64_t>(16, stride[b.dst_buf]));
+        bytes += b.len;
+        words += (b.len + 23) / 16;
+    }
+    if (fixed) rows = 1;
+    // Form 1 describes `rows` rows in its tables: worth it where blocks are short (several meet in a
+    // destination word) and the tables stay small.
+    T.form = fixed ? 0 : ((bytes < kWordsLongBlock * (int64_t)blocks.size() && rows * bytes <= kWordsMostGroup) ? 1 : 2);
+    if (T.form == 2) {
+        rows = 1;
+    } else {
+        // Short rows: several of them share a chunk, so that its 32 loads are nearly all used (24 blocks of
+        // 4 bytes are 24 loads, a quarter of the lanes idle) - where enough warps remain, and in form 0,
+        // which knows no incomplete row group, where every slab is whole groups.
+        const int64_t whole = T.form == 1 ? 0 : (c.d >= 2 ? c.rank_stride[0] : c.P);
+        while (rows * words < 96 && rows * 2 * bytes <= kWordsMostGroup && rows < 16 && whole % (rows * 2) == 0 &&
+               c.P * words / 28 >= 4ll * r.sm_count * (kWordsThreads / 32))
+            rows *= 2;
+    }
+    T.rows_sub = (uint32_t)rows;
+    const int64_t grain = by8 ? 8 : 4;  // of the words that are smaller than 16 bytes
+
+    auto describe = [&](const Block &b, uint32_t sub) {
+        LoadDev ld{};
+        long long delta = 0;
+        for (int j = 0; j < c.d; ++j) {
+            const int value = c.periodic[j] ? b.p->shift[j] : b.p->check[j];
+            delta -= (long long)b.p->shift[j] * c.rank_stride[j];
+            if (value) ld.c[used_index[j]] = value;
+        }
+        ld.src_term = delta * stride[b.src_buf] + b.src_off;
+        ld.len = (uint32_t)b.len;
+        ld.dst_term = b.dst_off;
+        ld.src_buf = (uint8_t)b.src_buf;
+        ld.dst_buf = (uint8_t)b.dst_buf;
+        ld.sub = (uint8_t)sub;
+        return ld;
+    };
+
+    if (T.form == 2) {
+        // a group of lanes per block: one per destination word, and one more that only loads
+        for (const Block &b : blocks) {
+            const LoadDev ld = describe(b, 0);
+            const int64_t n = (placement(addr[b.dst_buf] + b.dst_off, stride[b.dst_buf]).highest + b.len + 15) / 16;
+            for (int64_t w0 = 0; w0 < n; w0 += 31) {
+                const size_t lanes = (size_t)std::min<int64_t>(31, n - w0) + 1;
+                if (T.loads.size() % 32 + lanes > 32) T.loads.resize((T.loads.size() + 31) / 32 * 32, LoadDev{});
+                for (size_t k = 0; k < lanes; ++k) {
+                    T.loads.push_back(ld);
+                    T.loads.back().word = (int32_t)(w0 + (int64_t)k);
+                    T.loads.back().stores = k + 1 < lanes;
+                }
+            }
+        }
+        T.loads.resize((T.loads.size() + 31) / 32 * 32, LoadDev{});
+        T.chunks.resize(T.loads.size() / 32, EntryDev{});
+        deal(T);
+        return;
+    }
+
+    // Forms 0 and 1.  In form 0 a destination word of 16 bytes whose bytes have the same place in one to
+    // three source words can go into a placed chunk; everything else is cut into words of 4 or, where
+    // everything is a multiple of 8, of 8 bytes.
+    struct Fine { int buf; int64_t at; std::vector<Run> runs; };
+    struct Placed { int buf; int64_t at; bool full; std::vector<LoadDev> from; std::vector<Run> runs; };
+    std::vector<Fine> fine;
+    std::vector<Placed> placed;
+    size_t lone = 0;        // placed words from one source that come first
+    std::vector<Run> word;  // runs of the pending 16-byte word
+    int word_buf = -1;
+    int64_t word_at = 0;
+    auto cut = [&](int buf, int64_t base, const std::vector<Run> &runs) {
+        for (const Run &q : runs)
+            for (int at = q.begin; at < q.begin + q.n;) {
+                const int64_t w = base + at / grain * grain;
+                const int end = (int)std::min<int64_t>(at / grain * grain + grain, q.begin + q.n);
+                if (fine.empty() || fine.back().buf != buf || fine.back().at != w) fine.push_back(Fine{buf, w, {}});
+                fine.back().runs.push_back(Run{q.block, q.sub, q.x + at - q.begin, (int)(base + at - w), end - at});
+                at = end;
+            }
+    };
+    auto flush = [&]() {
+        if (word.empty()) return;
+        bool in_place = T.form == 0 && word.size() <= 3;  // every byte of the word has the same place in its source word
+        int filled = 0;
+        for (const Run &q : word) {
+            in_place = in_place && ((blocks[q.block].src_off - blocks[q.block].dst_off) & 15) == 0;
+            filled += q.n;
+        }
+        if (in_place) {
+            Placed w{word_buf, word_at, filled == 16, {}, word};
+            for (const Run &q : word) {
+                LoadDev ld = describe(blocks[q.block], q.sub);
+                ld.src_term += q.x - q.begin;
+                ld.dst_term = word_at;
+                ld.word = (int32_t)(((1u << q.n) - 1u) << q.begin);
+                w.from.push_back(ld);
+            }
+            placed.push_back(w);
+        } else {
+            cut(word_buf, word_at, word);
+        }
+        word.clear();
+    };
+    for (size_t lo = 0; lo < blocks.size();) {
+        size_t hi = lo;
+        while (hi < blocks.size() && blocks[hi].dst_buf == blocks[lo].dst_buf) ++hi;
+        const int buf = blocks[lo].dst_buf;
+        for (uint32_t sub = 0; sub < T.rows_sub; ++sub)
+            for (size_t k = lo; k < hi; ++k) {
+                const int64_t at = (int64_t)sub * stride[buf] + addr[buf] + blocks[k].dst_off;
+                for (int64_t p = at; p < at + blocks[k].len;) {
+                    const int64_t w = p / 16 * 16, end = std::min(w + 16, at + blocks[k].len);
+                    if (word_buf != buf || word_at != w) flush();
+                    word_buf = buf;
+                    word_at = w;
+                    word.push_back(Run{k, sub, p - at, (int)(p - w), (int)(end - p)});
+                    p = end;
+                }
+            }
+        flush();
+        lo = hi;
+    }
+
+    // Words that this launch fills only in part are cheaper as smaller words, unless there are next to
+    // none (the end of a row): with them all placed the irregular collective of 4 to 1024 bytes took
+    // 1642 instead of 1387 microseconds.  Where merged words are few, the words that are not get chunks
+    // of their own, which need no merging (and where everything is a multiple of 4 bytes, the few are
+    // cheaper in smaller words: one-pass irregular 735 against 685); where they are many, they stay
+    // with their neighbours (118-byte blocks, one merged word in eight: 88 against 134 microseconds).
+    {
+        size_t merged = 0, partial = 0;
+        for (const Placed &w : placed) {
+            merged += w.from.size() > 1;
+            partial += !w.full;
+        }
+        const bool apart = merged * 12 < placed.size(), keep_partial = partial * 64 <= placed.size();
+        std::vector<Placed> plain, rest;
+        for (Placed &w : placed) {
+            if (!w.full && !keep_partial) cut(w.buf, w.at, w.runs);
+            else if (!apart) rest.push_back(std::move(w));
+            else if (w.full && w.from.size() == 1) plain.push_back(std::move(w));
+            else if (by4) cut(w.buf, w.at, w.runs);
+            else rest.push_back(std::move(w));
+        }
+        lone = plain.size();
+        placed.swap(plain);
+        placed.insert(placed.end(), rest.begin(), rest.end());
+        std::stable_sort(fine.begin(), fine.end(), [](const Fine &x, const Fine &y) { return x.buf != y.buf ? x.buf < y.buf : x.at < y.at; });
+    }
+    // Placed words in address order, so that the two halves of a 32-byte sector belong to one chunk: the
+    // lanes that store first, then those that only load.
+    for (size_t k = 0; k < placed.size();) {
+        const size_t end = k < lone ? lone : placed.size();
+        size_t n = 0, lanes = 0;
+        while (k + n < end && lanes + placed[k + n].from.size() <= 32) lanes += placed[k + n++].from.size();
+        if (k + n < end && n > 1 && placed[k + n].at % 32 != 0 && placed[k + n].at == placed[k + n - 1].at + 16) --n;
+        const size_t base = T.loads.size();
+        T.loads.resize(base + 32, LoadDev{});
+        size_t extra = n;
+        EntryDev ck{};
+        ck.kind = CHUNK_WHOLE;
+        ck.passes = 1;
+        for (size_t e = 0; e < n; ++e) {
+            const Placed &w = placed[k + e];
+            T.loads[base + e] = w.from[0];
+            T.loads[base + e].stores = 1;
+            uint8_t other[2] = {(uint8_t)e, (uint8_t)e};
+            for (size_t q = 1; q < w.from.size(); ++q) {
+                other[q - 1] = (uint8_t)extra;
+                T.loads[base + extra++] = w.from[q];
+            }
+            T.loads[base + e].second = other[0];
+            T.loads[base + e].third = other[1];
+            if (w.from.size() > 1 || !w.full) ck.kind = CHUNK_PLACED;
+            ck.passes = std::max<uint8_t>(ck.passes, (uint8_t)w.from.size());
+        }
+        for (size_t e = n; e < 32; ++e) T.loads[base + e].second = T.loads[base + e].third = (uint8_t)e;
+        T.chunks.push_back(ck);
+        k += n;
+    }
+
+    FineChunks chunks{T, (uint8_t)(by8 ? CHUNK_ONE8 : (by4 ? CHUNK_ONE4 : CHUNK_TWO))};
+    auto range = [&](const Run &q, int64_t &k0, int64_t &k1) -> int64_t {
+        const Block &b = blocks[q.block];
+        const Placement pl = placement(addr[b.src_buf] + b.src_off, stride[b.src_buf]);
+        k0 = (pl.lowest + q.x) / 16;
+        k1 = (pl.highest + q.x + q.n - 1) / 16;
+        return T.form == 0 ? pl.lowest : 0;  // (form 1 adds the row's own place at run time)
+    };
+    auto load = [&](const Run &q, int64_t k) {
+        const Block &b = blocks[q.block];
+        LoadDev ld = describe(b, q.sub);
+        ld.word = (int32_t)k;
+        if (T.form == 0) ld.src_term += k * 16 - ((addr[b.src_buf] + b.src_off) & 15);  // the aligned word itself
+        return ld;
+    };
+    for (const Fine &w : fine) chunks.add(w.buf, w.at, w.runs, range, load);
+    chunks.close();
+    deal(T);
+}
+
+}  // namespace iso
