@@ -231,9 +231,7 @@ void plan_words(const Request &r, LaunchPlan &L, uintptr_t inter_addr)
     L.grid = std::max<long long>(1, (warps * 32 + L.threads - 1) / L.threads);
     L.grid = std::min<long long>(L.grid, (long long)r.sm_count * (kWordsThreads / L.threads));
     L.grid = std::max<long long>(L.grid, (entries * 32 + L.threads - 1) / L.threads);  // every entry has a warp
-    bool mesh = false;
-    for (int k = 0; k < L.n_used; ++k) mesh = mesh || !r.comm->periodic[L.used_dim[k]];
-    const int depth = L.tables.form == 0 && !mesh ? kWordsDepth : kWordsDepthCoded;
+    const int depth = L.tables.form == 0 ? kWordsDepth : kWordsDepthCoded;
     L.smem = kWordsPadFront + (size_t)depth * L.threads * 16 + kWordsPadBack;
 }
 
@@ -742,9 +740,7 @@ cudaError_t launch_words(const LaunchPlan &L, LaunchDev &a, cudaStream_t stream,
     if (a.n_entries == 0) return cudaSuccess;
     const int form = L.tables.form;
     if (a.mesh_mask)
-        return form == 0   ? launch_words_form<0, true>(L, a, stream, dependent)
-               : form == 1 ? launch_words_form<1, true>(L, a, stream, dependent)
-                           : launch_words_form<2, true>(L, a, stream, dependent);
+        return form == 1 ? launch_words_form<1, true>(L, a, stream, dependent) : launch_words_form<2, true>(L, a, stream, dependent);
     return form == 0   ? launch_words_form<0, false>(L, a, stream, dependent)
            : form == 1 ? launch_words_form<1, false>(L, a, stream, dependent)
                        : launch_words_form<2, false>(L, a, stream, dependent);
@@ -812,7 +808,7 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
         // dimension, and on the compact last phase of 16-byte blocks; the one-pass direct
         // schedules, three or more wrap tests per row, are bound by the latency of their
         // scattered loads and gain nothing, so they keep the divisions)
-        if (L.threads > 256 && L.n_used > 0 && r.knobs.coord_table &&
+        if (L.width == 16 && L.threads > 256 && L.n_used > 0 && r.knobs.coord_table &&
             (L.compact || nu <= 2) && !a.mesh_mask) {
             const long long groups = (a.row_hi - a.row_lo + L.rows_per_pass - 1) / L.rows_per_pass;
             const long long grid = grid_for_rows(L, a, a.grid_share) / std::max(1, L.col_split);  // CTAs that share the rows
@@ -822,8 +818,8 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
             if (!tab) a.tab_iters = 0;
         }
 #define ISO_ROWS(W, NU, MESH, COMPACT)                                                                          \
-    e = L.threads > 256 ? launch_rows_wide<W, NU, MESH, COMPACT>(tab, L, a, stream, dependent)                  \
-                        : launch_kernel(iso_gather_rows<W, kVecDepth, NU, MESH, COMPACT>, L, a, stream, dependent, 0)
+    e = (W == 16 && L.threads > 256) ? launch_rows_wide<16, NU, MESH, COMPACT>(tab, L, a, stream, dependent)    \
+                                     : launch_kernel(iso_gather_rows<W, kVecDepth, NU, MESH, COMPACT>, L, a, stream, dependent, 0)
 #define ISO_ROWS_W(W)                                                            \
     do {                                                                         \
         if (a.mesh_mask) ISO_ROWS(W, ISO_MAX_DIMS, true, false);                 \
@@ -837,7 +833,8 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
         else if (nu == 3) ISO_ROWS(W, 3, false, false);                          \
         else ISO_ROWS(W, ISO_MAX_DIMS, false, false);                            \
     } while (0)
-        ISO_ROWS_W(16);
+        if (L.width == 16) ISO_ROWS_W(16);
+        else ISO_ROWS_W(4);
 #undef ISO_ROWS_W
 #undef ISO_ROWS
     }

@@ -85,17 +85,18 @@ constexpr size_t kHybridStageBytes = 128 * 1024;  // staging area of the bulk wa
 
 // One word to load, by lane.  In a whole or placed chunk (and in form 2) the lane may also store one.
 struct alignas(16) LoadDev {
-    long long src_term;      // rank_delta * source stride + offset of the block (form 0: of the aligned word)
+    long long src_term;      // rank_delta * source stride + offset of the block, or (with word 0) of the aligned word itself
+                             // where that is the same place inside its word for all rows
     uint32_t len;            // bytes of the block (0: this lane loads nothing)
-    int32_t word;            // forms 1, 2: index of this word, counted from the one that holds the block's first byte;
-                             // placed chunk: which bytes of the destination word this lane's word holds
+    int32_t word;            // index of this word, counted from the one that holds the byte at src_term
     int32_t c[ISO_MAX_DIMS]; // shift (non-periodic dimension: check value) along the launch's used dimensions
-    long long dst_term;      // whole or placed chunk: destination offset of the word; form 2: of the block
+    long long dst_term;      // whole or placed chunk: the word, from the (aligned down) start of the row group; form 2: offset
+                             // of the block
     uint8_t src_buf, dst_buf;
     uint8_t sub;             // which of the rows of the group
     uint8_t stores;          // whole or placed chunk, form 2: this lane stores a word
     uint8_t second, third;   // placed chunk: lanes that hold more bytes of the word (this lane itself: none)
-    uint8_t pad[2];
+    uint16_t mask;           // placed chunk: which bytes of the destination word this lane's word holds
 };
 static_assert(sizeof(LoadDev) == 64, "load descriptors are read as four 16-byte words");
 
@@ -114,9 +115,9 @@ struct alignas(16) TinyDev {
     uint32_t mask;
 };
 
-// How a chunk is stored.  WHOLE (form 0): every lane stores the word it has loaded.  PLACED (form 0):
-// likewise, merged where need be with the words of one or two other lanes, every byte having the same
-// place in both.  ONE4, ONE8: 4- or 8-byte words, each out of one block.  TWO: 4-byte words out of one
+// How a chunk is stored.  WHOLE: every lane stores the word it has loaded.  PLACED: likewise, merged
+// where need be with the words of one or two other lanes, every byte having the same place in both
+// (for all rows).  ONE4, ONE8: 4- or 8-byte words, each out of one block.  TWO: 4-byte words out of one
 // or two blocks.  TINY: likewise, byte by byte.
 enum { CHUNK_WHOLE = 0, CHUNK_PLACED = 1, CHUNK_ONE4 = 2, CHUNK_ONE8 = 3, CHUNK_TWO = 4, CHUNK_TINY = 5 };
 
@@ -134,7 +135,7 @@ struct alignas(16) EntryDev {
 static_assert(sizeof(EntryDev) == 32, "entries are read as two 16-byte words");
 
 struct WordTables {
-    int form = 0;          // 0: all alignments the same for every row, 1: worked out per row, 2: likewise, long blocks
+    int form = 0;          // 0: all alignments the same for every row, 1: not so, or a mesh, 2: long blocks of any alignment
     uint32_t rows_sub = 1; // forms 0, 1: rows described together (a row group)
     std::vector<LoadDev> loads;     // 32 per chunk
     std::vector<EntryDev> chunks;   // one per chunk (turn 0 of 1), before they are dealt to warps

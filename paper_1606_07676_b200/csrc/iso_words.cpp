@@ -202,11 +202,17 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     for (int k = 0; k < L.n_used; ++k) used_index[L.used_dim[k]] = k;
 
     const std::vector<Block> blocks = merged_blocks(L, c.d);
-    bool fixed = true;             // every stride and base address is a multiple of 16
+    auto at16 = [&](int buf) { return stride[buf] % 16 == 0 && addr[buf] == 0; };  // the same places inside a word for all rows
+    bool fixed = true, dst_fixed = true;  // all buffers, all destinations are like that
     bool by4 = true, by8 = true;   // every address is a multiple of 4, of 8
-    int64_t rows = 1, bytes = 0, words = 0;
+    int64_t rows = 1, bytes = 0, words = 0, moving = 0, moving_bytes = 0;  // moving: blocks that are not, on either side
     for (const Block &b : blocks) {
-        for (int q : {b.src_buf, b.dst_buf}) fixed = fixed && stride[q] % 16 == 0 && addr[q] == 0;
+        dst_fixed = dst_fixed && at16(b.dst_buf);
+        if (!at16(b.src_buf) || !at16(b.dst_buf)) {
+            fixed = false;
+            ++moving;
+            moving_bytes += b.len;
+        }
         for (int64_t v : {stride[b.src_buf], stride[b.dst_buf], addr[b.src_buf], addr[b.dst_buf], b.src_off, b.dst_off, b.len}) {
             by4 = by4 && v % 4 == 0;
             by8 = by8 && v % 8 == 0;
@@ -215,10 +221,13 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         bytes += b.len;
         words += (b.len + 23) / 16;
     }
-    if (fixed) rows = 1;
-    // Form 1 describes `rows` rows in its tables: worth it where blocks are short (several meet in a
-    // destination word) and the tables stay small.
-    T.form = fixed ? 0 : ((bytes < kWordsLongBlock * (int64_t)blocks.size() && rows * bytes <= kWordsMostGroup) ? 1 : 2);
+    bool mesh = false;
+    for (int k = 0; k < L.n_used; ++k) mesh = mesh || !c.periodic[L.used_dim[k]];
+    // Form 1 describes `rows` rows in its tables: worth it where the blocks whose place varies are short
+    // (several meet in a destination word) and the tables stay small.
+    if (dst_fixed) rows = 1;
+    if (fixed) T.form = mesh ? 1 : 0;
+    else T.form = moving_bytes < kWordsLongBlock * moving && rows * bytes <= kWordsMostGroup ? 1 : 2;
     if (T.form == 2) {
         rows = 1;
     } else {
@@ -271,8 +280,8 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         return;
     }
 
-    // Forms 0 and 1.  In form 0 a destination word of 16 bytes whose bytes have the same place in one to
-    // three source words can go into a placed chunk; everything else is cut into words of 4 or, where
+    // Forms 0 and 1.  A destination word of 16 bytes whose bytes have the same place in one to three
+    // source words, for all rows, can go into a placed chunk; everything else is cut into words of 4 or, where
     // everything is a multiple of 8, of 8 bytes.
     struct Fine { int buf; int64_t at; std::vector<Run> runs; };
     struct Placed { int buf; int64_t at; bool full; std::vector<LoadDev> from; std::vector<Run> runs; };
@@ -294,10 +303,10 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     };
     auto flush = [&]() {
         if (word.empty()) return;
-        bool in_place = T.form == 0 && word.size() <= 3;  // every byte of the word has the same place in its source word
+        bool in_place = word.size() <= 3;  // every byte of the word has the same place in its source word
         int filled = 0;
         for (const Run &q : word) {
-            in_place = in_place && ((blocks[q.block].src_off - blocks[q.block].dst_off) & 15) == 0;
+            in_place = in_place && at16(blocks[q.block].src_buf) && ((blocks[q.block].src_off + q.x) & 15) == q.begin;
             filled += q.n;
         }
         if (in_place) {
@@ -306,7 +315,7 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
                 LoadDev ld = describe(blocks[q.block], q.sub);
                 ld.src_term += q.x - q.begin;
                 ld.dst_term = word_at;
-                ld.word = (int32_t)(((1u << q.n) - 1u) << q.begin);
+                ld.mask = (uint16_t)(((1u << q.n) - 1u) << q.begin);
                 w.from.push_back(ld);
             }
             placed.push_back(w);
@@ -366,7 +375,7 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     for (size_t k = 0; k < placed.size();) {
         const size_t end = k < lone ? lone : placed.size();
         size_t n = 0, lanes = 0;
-        while (k + n < end && lanes + placed[k + n].from.size() <= 32) lanes += placed[k + n++].from.size();
+        while (k + n < end && placed[k + n].buf == placed[k].buf && lanes + placed[k + n].from.size() <= 32) lanes += placed[k + n++].from.size();
         if (k + n < end && n > 1 && placed[k + n].at % 32 != 0 && placed[k + n].at == placed[k + n - 1].at + 16) --n;
         const size_t base = T.loads.size();
         T.loads.resize(base + 32, LoadDev{});
@@ -374,6 +383,7 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         EntryDev ck{};
         ck.kind = CHUNK_WHOLE;
         ck.passes = 1;
+        ck.dst_buf = (uint8_t)placed[k].buf;
         for (size_t e = 0; e < n; ++e) {
             const Placed &w = placed[k + e];
             T.loads[base + e] = w.from[0];
@@ -399,13 +409,13 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         const Placement pl = placement(addr[b.src_buf] + b.src_off, stride[b.src_buf]);
         k0 = (pl.lowest + q.x) / 16;
         k1 = (pl.highest + q.x + q.n - 1) / 16;
-        return T.form == 0 ? pl.lowest : 0;  // (form 1 adds the row's own place at run time)
+        return at16(b.src_buf) ? pl.lowest : 0;  // (where it varies the kernel adds the row's own place)
     };
     auto load = [&](const Run &q, int64_t k) {
         const Block &b = blocks[q.block];
         LoadDev ld = describe(b, q.sub);
-        ld.word = (int32_t)k;
-        if (T.form == 0) ld.src_term += k * 16 - ((addr[b.src_buf] + b.src_off) & 15);  // the aligned word itself
+        if (at16(b.src_buf)) ld.src_term += k * 16 - (b.src_off & 15);  // the aligned word itself
+        else ld.word = (int32_t)k;
         return ld;
     };
     for (const Fine &w : fine) chunks.add(w.buf, w.at, w.runs, range, load);

@@ -17,10 +17,11 @@
 // down its rows.
 //
 // FORM says how source and destination are placed against each other:
-//   0  every stride and base address is a multiple of 16: the place of every byte inside its word
-//      is the same for all rows, so shifts and masks come from the tables;
-//   1  anything else, short blocks: the tables describe A consecutive rows (A * stride is a multiple
-//      of 16), and the source's place inside its word is worked out per row;
+//   0  every stride and base address is a multiple of 16 and all dimensions are periodic: the place of
+//      every byte inside its word is the same for all rows, so shifts and masks come from the tables;
+//   1  anything else, short blocks: the tables describe A consecutive rows (A * the destination's stride
+//      is a multiple of 16), and the place of a source whose stride is not one, and whether it exists
+//      at all, is worked out per row (a "code" per word in flight);
 //   2  anything else, long blocks: a group of lanes per block, both alignments worked out per row;
 //      16-byte stores, only the first and the last word of a block in part.
 // An aligned word that holds one byte of a buffer never leaves the buffer's page, so words are
@@ -113,10 +114,11 @@ template <int FORM, bool MESH, int NU, bool TAB>
 __global__ void __launch_bounds__(kWordsThreads, 1) iso_gather_words(const __grid_constant__ LaunchDev L)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    constexpr int DEPTH = FORM == 0 && !MESH ? kWordsDepth : kWordsDepthCoded, R = 2;
+    constexpr int DEPTH = FORM == 0 ? kWordsDepth : kWordsDepthCoded, R = 2;
+    static_assert(FORM != 0 || !MESH, "a mesh needs codes");
     constexpr uint32_t NT = NU <= 1 ? 1 : (NU == 2 ? 2 : (NU <= 4 ? 4 : 8));  // table entries per row
     constexpr uint32_t kNone = 16;                                            // code of a block that has no source
-    constexpr bool coded = FORM != 0 || MESH;
+    constexpr bool coded = FORM != 0;
     constexpr bool GROUPS = FORM != 2;  // the tables may describe several rows
     constexpr int kFew = 4;             // up to so many dimensions their wrap terms are kept in registers
     const uint32_t nthr = blockDim.x, nw = nthr >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
@@ -173,22 +175,22 @@ __global__ void __launch_bounds__(kWordsThreads, 1) iso_gather_words(const __gri
     const unsigned char *src_ld = L.buf[ld.src_buf] + ld.src_term + ((long long)s_first * A + sub) * stride_s;
     const long long src_step = (long long)s_step * A * stride_s;
     const bool loads = ld.len != 0;
-    const bool whole = FORM == 0 && en.kind == CHUNK_WHOLE, placed = FORM == 0 && en.kind == CHUNK_PLACED;
-    const int db = FORM == 2 || whole || placed ? ld.dst_buf : en.dst_buf;
+    const bool whole = FORM != 2 && en.kind == CHUNK_WHOLE, placed = FORM != 2 && en.kind == CHUNK_PLACED;
+    const int db = FORM == 2 ? ld.dst_buf : en.dst_buf;
     const long long group_d = (long long)A * L.buf_stride[db];
     const bool keep = (whole || placed) && L.keep_inter && db == 2;  // ISO_BUF_INTER
     const uint64_t policy = keep ? l2_policy_evict_last() : 0;
-    unsigned char *const base_d = FORM == 2 || whole || placed
-                                      ? L.buf[db] + ld.dst_term
-                                      : reinterpret_cast<unsigned char *>(reinterpret_cast<uintptr_t>(L.buf[db]) & ~(uintptr_t)15) + en.dst_term;
+    unsigned char *const base_d = FORM == 2 ? L.buf[db] + ld.dst_term
+                                            : reinterpret_cast<unsigned char *>(reinterpret_cast<uintptr_t>(L.buf[db]) & ~(uintptr_t)15) +
+                                                  (whole || placed ? ld.dst_term : en.dst_term);
     long long wrap_bytes[NU <= kFew ? NU : 1];
     if (NU <= kFew) {
 #pragma unroll
         for (int e = 0; e < NU; ++e) wrap_bytes[e] = (long long)L.used_wrap[e] * stride_s;
     }
 
-    // Loads this lane's word of row group s into a ring slot.  Returns where in its word the block
-    // starts, or kNone (forms 1, 2, meshes).
+    // Loads this lane's word of row group s into a ring slot.  Returns where in its word the byte at
+    // src_term lies, or kNone (forms 1, 2).
     const uint32_t tab_row = L.tab_slots * A * NT;
     uint32_t tab_at = ((slot - first_slot) * A + sub) * NT + en.turn * tab_row;
     const uint32_t tab_step = en.turns * tab_row;
@@ -240,8 +242,8 @@ __global__ void __launch_bounds__(kWordsThreads, 1) iso_gather_words(const __gri
             }
         if (NU > kFew) src += (long long)wraps * stride_s;
         if (FORM == 0) {
-            if (loads && (!MESH || valid)) cp_async<16>(to, src);
-            return MESH && !valid ? kNone : 0u;
+            if (loads) cp_async<16>(to, src);
+            return 0u;
         }
         const uint32_t mis = (uint32_t)(uintptr_t)src & 15u;
         int w = ld.word;
@@ -253,7 +255,7 @@ __global__ void __launch_bounds__(kWordsThreads, 1) iso_gather_words(const __gri
         return valid ? mis : kNone;
     };
 
-    unsigned long long codes = 0;  // forms 1, 2 and meshes: five bits per stage in flight, the newest lowest
+    unsigned long long codes = 0;  // forms 1 and 2: five bits per stage in flight, the newest lowest
     uint32_t s_ld = s_first;
     const uint32_t stage_bytes = nthr * 16;
     auto load_two = [&](unsigned char *to) {
@@ -314,7 +316,7 @@ __global__ void __launch_bounds__(kWordsThreads, 1) iso_gather_words(const __gri
             for (int i = 0; i < RW; ++i) v[i] = *reinterpret_cast<const uint4 *>(stage + i * stage_bytes);
 #pragma unroll
             for (int i = 0; i < RW; ++i)
-                if (loads && (MESH ? code_of(i) != kNone : s + i * s_step < s_hi)) {
+                if (loads && (coded ? code_of(i) != kNone : s + i * s_step < s_hi)) {
                     if (keep) store_16_hinted(dst + i * dst_step, v[i], policy);
                     else *reinterpret_cast<uint4 *>(dst + i * dst_step) = v[i];
                 }
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(kWordsThreads, 1) iso_gather_words(const __gri
         }
     } else if (placed) {
         // what is stored: this lane's bytes, those of the second and of the third lane
-        const uint32_t m_own = loads ? (uint32_t)ld.word : 0u;
+        const uint32_t m_own = loads ? (uint32_t)ld.mask : 0u;
         uint32_t m_second = __shfl_sync(0xffffffffu, m_own, ld.second), m_third = __shfl_sync(0xffffffffu, m_own, ld.third);
         if (ld.second == lane) m_second = 0;
         if (ld.third == lane) m_third = 0;
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(kWordsThreads, 1) iso_gather_words(const __gri
 #pragma unroll
             for (int i = 0; i < R; ++i) {
                 mask[i] = s + i * s_step < s_hi ? m_own | m_second | m_third : 0u;
-                if (MESH) {
+                if (coded) {
                     const uint32_t code = code_of(i), code2 = __shfl_sync(0xffffffffu, code, ld.second), code3 = __shfl_sync(0xffffffffu, code, ld.third);
                     mask[i] = (code != kNone ? m_own : 0u) | (code2 != kNone ? m_second : 0u) | (code3 != kNone ? m_third : 0u);
                 }
