@@ -220,14 +220,19 @@ void fill_fans(const Request &r, const LaunchPlan &L, FanDev *fd)
     }
 }
 
-// Launches of words: the tables, and the CTA shape for them.  24 warps per SM either way; where the
-// whole launch has fewer warps than that, narrow CTAs spread them over more SMs.
+// Launches of words: the tables, and the CTA shape for them.  24 warps per SM either way: one CTA of
+// 768 threads where a warp has 30 rows and more (irregular 64x64x32 in one pass: 615 microseconds per
+// start against 663 with two CTAs of 384; 777-byte allgather on 31x33x29 264 against 287), else CTAs
+// narrow enough that those of the next launch can start while these drain: two of 384 (one of 768:
+// 13-byte blocks on 257x251 40.6 against 38.9, 24-byte allgather on 32^3 19.9 against 18.9), and three
+// of 256 where a warp has hardly any rows (16^3 with 64-byte blocks: 10.0, 8.9 and 8.7).
 void plan_words(const Request &r, LaunchPlan &L, uintptr_t inter_addr)
 {
     build_words(r, L, (uintptr_t)r.send, (uintptr_t)r.recv, inter_addr);
     const long long groups = (r.comm->P + L.tables.rows_sub - 1) / L.tables.rows_sub;
     const long long entries = (long long)L.tables.entries.size(), warps = groups * entries;
-    L.threads = warps >= 16ll * r.sm_count ? kWordsThreads : (warps >= 4ll * r.sm_count ? 384 : 128);
+    const long long rows = warps / (r.sm_count * (kWordsThreads / 32));  // of a warp
+    L.threads = rows >= 30 ? kWordsThreads : (rows >= 6 ? 384 : 256);
     L.grid = std::max<long long>(1, (warps * 32 + L.threads - 1) / L.threads);
     L.grid = std::min<long long>(L.grid, (long long)r.sm_count * (kWordsThreads / L.threads));
     L.grid = std::max<long long>(L.grid, (entries * 32 + L.threads - 1) / L.threads);  // every entry has a warp

@@ -147,7 +147,8 @@ constexpr int64_t kWordsLongBlock = 64;       // mean block length from which fo
 constexpr int64_t kWordsMostGroup = 32 << 10; // bytes of a row group that the tables describe at most
 constexpr int kWordsDepth = 16;               // words in flight per lane, as many as fit beside a coordinate table ...
 constexpr int kWordsDepthCoded = 12;          // ... and where the codes of the stages have to fit into 64 bits
-constexpr int kWordsThreads = 768;            // threads of a CTA, one per SM (fewer where a launch is small)
+constexpr int kWordsThreads = 768;            // threads per SM, in one to three CTAs
+constexpr int64_t kWordsSmallLaunch = 12 << 20;  // bytes up to which a launch of 16-byte units runs as words
 constexpr int kWordsPasses = 4;               // passes over a chunk's words at most
 constexpr uint32_t kWordsPadFront = 16, kWordsPadBack = 48;  // shared memory around the ring that a shifted read may touch
 

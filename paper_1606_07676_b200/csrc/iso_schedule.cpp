@@ -1123,7 +1123,15 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                         // 256x256, 24 neighbours: 12.3 against 13.9 microseconds, one pass 7.6 against 8.9)
                         bool tiny = width == 4;
                         for (const LoweredPart &lp : L.parts) tiny = tiny && lp.p.len == 4;
-                        L.words = kernel == KERNEL_VEC && width != 16 && longs.empty() && !tiny;
+                        // Small launches of 16-byte units are also better off as words, in narrow CTAs of which
+                        // several fit an SM: a CTA of 1024 threads fills its SM, so the next launch cannot even
+                        // start before this one drains.  Measured per start, wide CTAs against words: 8^3 with 26
+                        // 64-byte blocks 9.4 against 7.2 microseconds, 16^3 12.8 against 8.7 (2.4 MB per launch),
+                        // 60x60 with 24 blocks of 128 bytes 9.0 against 7.7 (9 MB), but 40x40 with 512-byte blocks
+                        // 12.2 against 12.9 (16 MB) and 9^4 with 80 64-byte blocks 30.3 against 33.8 (22 MB).
+                        const bool small = width == 16 && (int64_t)c.P * (int64_t)units * 16 <= kWordsSmallLaunch && !r.persistent &&
+                                           r.wave_request == 0 && r.knobs.vec_threads == 0;
+                        L.words = kernel == KERNEL_VEC && (width != 16 || small) && longs.empty() && !tiny;
                         L.compact = kernel == KERNEL_VEC && !L.words && L.n_used > 3 && L.max_nnz < L.n_used &&
                                     torus && !r.persistent;  // (the pipelined one-launch kernel does take compact launches)
                     }
