@@ -278,7 +278,7 @@ int materialise(Request &r)
     if (sms > 0) r.sm_count = sms;
     {
         // lowered afresh with the request's present settings: the slab plan below reads it
-        int rc0 = lower_schedule(r, (uintptr_t)r.send, (uintptr_t)r.recv, (uintptr_t)r.d_inter);
+        int rc0 = lower_schedule(r, (uintptr_t)r.send, (uintptr_t)r.recv, 0);
         if (rc0 != ISO_SUCCESS) return rc0;
     }
     // pipelined one-launch execution: every launch must be a 16-byte vector launch of at most
@@ -299,7 +299,6 @@ int materialise(Request &r)
         r.wave_ok = ok;
     }
     choose_slab_plan(r);
-    // device tables depend on the alignment of the intermediate buffer: allocate it first
     const int64_t inter_bytes = r.inter_rows * r.inter_stride;
     if (inter_bytes != r.d_inter_bytes) {  // exactly sized, so that the trailing band sits right behind it
         if (r.d_inter_alloc) cudaFree(r.d_inter_alloc);
@@ -315,8 +314,8 @@ int materialise(Request &r)
         ISO_CUDA(cudaMemset(r.d_inter + inter_bytes, kGuardPattern, kGuardBytes));
         }
     }
-    int rc = lower_schedule(r, (uintptr_t)r.send, (uintptr_t)r.recv, (uintptr_t)r.d_inter);
-    if (rc != ISO_SUCCESS) return rc;
+    // (the launches stand: the lowering only looks at the buffer's alignment, and every intermediate
+    // buffer starts on a 256-byte boundary)
 
     // every plan that needs tables: the launches and the bulk sides of hybrid launches
     std::vector<LaunchPlan *> plans;

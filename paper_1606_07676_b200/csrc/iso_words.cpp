@@ -91,46 +91,51 @@ void deal(WordTables &T)
     });
 }
 
-struct Run { size_t block; uint32_t sub; int64_t x; int begin, n; };  // bytes x .. x+n of a block, at `begin` in a word
+struct Run { uint32_t block, sub; int64_t x; int begin, n; };  // bytes x .. x+n of a block, at `begin` in a word
+
+// A destination word and its runs (runs[first] ...).
+struct Word {
+    int64_t at;  // from the (aligned down) start of the row group
+    uint32_t first;
+    uint8_t n, buf;
+    bool in_place, full;  // 16-byte words: could be stored by the lanes that load it; all its bytes are in this launch
+};
 
 // Collects words of 4 or 8 bytes into chunks: one is closed when the next word would need more than 32
 // loads, or be one too many.
 struct FineChunks {
     WordTables &T;
+    const std::vector<Run> &runs;
     const uint8_t plainest;  // the chunk's kind as long as every word has one block (TWO: two)
     EntryDev open{};
-    size_t n_loads = 0;
-    size_t last_block = SIZE_MAX, last_slot = 0;  // block (and row) the last loads belong to
-    uint32_t last_sub = 0;
+    uint32_t n_loads = 0, n_words = 0;
+    uint32_t last_block = UINT32_MAX, last_slot = 0, last_sub = 0;  // what the last loads belong to
     int64_t first_k = 0, last_k = 0;
-    struct Word { int64_t at; std::vector<Run> runs; std::vector<std::pair<uint32_t, uint32_t>> places; };  // (place, lane) per run
-    std::vector<Word> words;
+    Word words[32 * kWordsPasses];
+    std::vector<uint32_t> places;  // place | lane << 10 of every run of the open chunk
 
     // range(run, k0, k1): the run's words, counted from the one that holds the block's first byte at its
     // lowest place, which is returned; load(run, k): the descriptor of its word k
     template <typename Range, typename Load>
-    void add(int buf, int64_t at, const std::vector<Run> &runs, Range range, Load load)
+    void add(const Word &w, Range range, Load load)
     {
-        size_t need = 0, lb = last_block;
-        uint32_t ls = last_sub;
-        int64_t lk = last_k;
-        for (const Run &q : runs) {
-            int64_t k0, k1;
+        uint32_t need = 0, lb = last_block, ls = last_sub;
+        int64_t lk = last_k, k0, k1;
+        for (uint32_t j = w.first; j < w.first + w.n; ++j) {
+            const Run &q = runs[j];
             range(q, k0, k1);
             const bool same = lb == q.block && ls == q.sub && k0 <= lk + 1;
-            need += (size_t)(same ? std::max<int64_t>(0, k1 - lk) : k1 - k0 + 1);
+            need += (uint32_t)(same ? std::max<int64_t>(0, k1 - lk) : k1 - k0 + 1);
             lk = same ? std::max(lk, k1) : k1;
             lb = q.block;
             ls = q.sub;
         }
-        if (words.size() == 32 * kWordsPasses || (!words.empty() && (open.dst_buf != buf || at - words[0].at >= 4 << 16)) ||
-            n_loads + need > 32)
+        if (n_words == 32 * kWordsPasses || (n_words > 0 && (open.dst_buf != w.buf || w.at - words[0].at >= 4 << 16)) || n_loads + need > 32)
             close();
-        if (words.empty()) open.kind = plainest;
-        open.dst_buf = (uint8_t)buf;
-        Word w{at, runs, {}};
-        for (const Run &q : runs) {
-            int64_t k0, k1;
+        if (n_words == 0) open.kind = plainest;
+        open.dst_buf = w.buf;
+        for (uint32_t j = w.first; j < w.first + w.n; ++j) {
+            const Run &q = runs[j];
             const int64_t base = range(q, k0, k1);
             if (last_block != q.block || last_sub != q.sub || k0 > last_k + 1) {
                 last_block = q.block;
@@ -143,32 +148,33 @@ struct FineChunks {
                 T.loads.push_back(load(q, ++last_k));
                 ++n_loads;
             }
-            w.places.push_back({(uint32_t)(16 + 16 * ((int64_t)last_slot - first_k) + q.x - q.begin + base), (uint32_t)last_slot});
+            places.push_back((uint32_t)(16 + 16 * ((int64_t)last_slot - first_k) + q.x - q.begin + base) | last_slot << 10);
         }
-        if (runs.size() > 2) open.kind = CHUNK_TINY;
-        words.push_back(w);
+        if (w.n > 2) open.kind = CHUNK_TINY;
+        words[n_words++] = w;
     }
 
     void close()
     {
-        if (words.empty()) return;
+        if (n_words == 0) return;
         const bool tiny = open.kind == CHUNK_TINY;
         open.first = (uint32_t)(tiny ? T.tiny.size() : T.fine.size());
-        open.passes = (uint8_t)((words.size() + 31) / 32);
+        open.passes = (uint8_t)((n_words + 31) / 32);
         open.dst_term = words[0].at;
-        for (const Word &w : words) {
+        const uint32_t *place = places.data();
+        for (uint32_t k = 0; k < n_words; ++k) {
+            const Word &w = words[k];
             FineDev f{};
             TinyDev t{};
             uint32_t mask[2] = {0, 0}, byte[4] = {0, 0, 0, 0};
-            for (size_t j = 0; j < w.runs.size(); ++j) {
-                const Run &q = w.runs[j];
-                const uint32_t place = w.places[j].first, lane = w.places[j].second;
+            for (uint32_t j = 0; j < w.n; ++j, ++place) {
+                const Run &q = runs[w.first + j];
                 for (int e = q.begin; e < q.begin + q.n && e < 4; ++e) {
-                    byte[e] = (place + (uint32_t)e) | lane << 10;
+                    byte[e] = *place + (uint32_t)e;
                     t.mask |= 1u << e;
                     if (j < 2) mask[j] |= 1u << e;
                 }
-                if (j < 2) f.a |= (place | lane << 10) << (15 * j);
+                if (j < 2) f.a |= *place << (15 * j);
             }
             t.a = byte[0] | byte[1] << 15;
             t.b = byte[2] | byte[3] << 15;
@@ -182,9 +188,9 @@ struct FineChunks {
         T.loads.resize((T.loads.size() + 31) / 32 * 32, LoadDev{});
         T.chunks.push_back(open);
         open = EntryDev{};
-        words.clear();
-        n_loads = 0;
-        last_block = SIZE_MAX;
+        places.clear();
+        n_loads = n_words = 0;
+        last_block = UINT32_MAX;
     }
 };
 
@@ -242,7 +248,9 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     T.rows_sub = (uint32_t)rows;
     const int64_t grain = by8 ? 8 : 4;  // of the words that are smaller than 16 bytes
 
-    auto describe = [&](const Block &b, uint32_t sub) {
+    std::vector<LoadDev> base(blocks.size());  // descriptors without a word
+    for (size_t i = 0; i < blocks.size(); ++i) {
+        const Block &b = blocks[i];
         LoadDev ld{};
         long long delta = 0;
         for (int j = 0; j < c.d; ++j) {
@@ -255,14 +263,14 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         ld.dst_term = b.dst_off;
         ld.src_buf = (uint8_t)b.src_buf;
         ld.dst_buf = (uint8_t)b.dst_buf;
-        ld.sub = (uint8_t)sub;
-        return ld;
-    };
+        base[i] = ld;
+    }
 
     if (T.form == 2) {
         // a group of lanes per block: one per destination word, and one more that only loads
-        for (const Block &b : blocks) {
-            const LoadDev ld = describe(b, 0);
+        for (size_t i = 0; i < blocks.size(); ++i) {
+            const Block &b = blocks[i];
+            const LoadDev &ld = base[i];
             const int64_t n = (placement(addr[b.dst_buf] + b.dst_off, stride[b.dst_buf]).highest + b.len + 15) / 16;
             for (int64_t w0 = 0; w0 < n; w0 += 31) {
                 const size_t lanes = (size_t)std::min<int64_t>(31, n - w0) + 1;
@@ -283,46 +291,26 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     // Forms 0 and 1.  A destination word of 16 bytes whose bytes have the same place in one to three
     // source words, for all rows, can go into a placed chunk; everything else is cut into words of 4 or, where
     // everything is a multiple of 8, of 8 bytes.
-    struct Fine { int buf; int64_t at; std::vector<Run> runs; };
-    struct Placed { int buf; int64_t at; bool full; std::vector<LoadDev> from; std::vector<Run> runs; };
-    std::vector<Fine> fine;
-    std::vector<Placed> placed;
-    size_t lone = 0;        // placed words from one source that come first
-    std::vector<Run> word;  // runs of the pending 16-byte word
-    int word_buf = -1;
-    int64_t word_at = 0;
-    auto cut = [&](int buf, int64_t base, const std::vector<Run> &runs) {
-        for (const Run &q : runs)
-            for (int at = q.begin; at < q.begin + q.n;) {
-                const int64_t w = base + at / grain * grain;
-                const int end = (int)std::min<int64_t>(at / grain * grain + grain, q.begin + q.n);
-                if (fine.empty() || fine.back().buf != buf || fine.back().at != w) fine.push_back(Fine{buf, w, {}});
-                fine.back().runs.push_back(Run{q.block, q.sub, q.x + at - q.begin, (int)(base + at - w), end - at});
-                at = end;
-            }
-    };
-    auto flush = [&]() {
-        if (word.empty()) return;
-        bool in_place = word.size() <= 3;  // every byte of the word has the same place in its source word
+    std::vector<Run> runs;
+    std::vector<Word> words16;
+    runs.reserve((size_t)(rows * words * 2));
+    words16.reserve((size_t)(rows * words * 2));
+    size_t n_in_place = 0, merged = 0, partial = 0;
+    auto finish = [&]() {  // the last of words16 has all its runs
+        if (words16.empty() || words16.back().n) return;
+        Word &w = words16.back();
+        w.n = (uint8_t)(runs.size() - w.first);
+        w.in_place = w.n <= 3;  // every byte of the word has the same place in its source word
         int filled = 0;
-        for (const Run &q : word) {
-            in_place = in_place && at16(blocks[q.block].src_buf) && ((blocks[q.block].src_off + q.x) & 15) == q.begin;
-            filled += q.n;
+        for (size_t j = w.first; j < runs.size(); ++j) {
+            const Block &b = blocks[runs[j].block];
+            w.in_place = w.in_place && at16(b.src_buf) && ((b.src_off + runs[j].x) & 15) == runs[j].begin;
+            filled += runs[j].n;
         }
-        if (in_place) {
-            Placed w{word_buf, word_at, filled == 16, {}, word};
-            for (const Run &q : word) {
-                LoadDev ld = describe(blocks[q.block], q.sub);
-                ld.src_term += q.x - q.begin;
-                ld.dst_term = word_at;
-                ld.mask = (uint16_t)(((1u << q.n) - 1u) << q.begin);
-                w.from.push_back(ld);
-            }
-            placed.push_back(w);
-        } else {
-            cut(word_buf, word_at, word);
-        }
-        word.clear();
+        w.full = filled == 16;
+        n_in_place += w.in_place;
+        merged += w.in_place && w.n > 1;
+        partial += w.in_place && !w.full;
     };
     for (size_t lo = 0; lo < blocks.size();) {
         size_t hi = lo;
@@ -330,19 +318,20 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         const int buf = blocks[lo].dst_buf;
         for (uint32_t sub = 0; sub < T.rows_sub; ++sub)
             for (size_t k = lo; k < hi; ++k) {
-                const int64_t at = (int64_t)sub * stride[buf] + addr[buf] + blocks[k].dst_off;
-                for (int64_t p = at; p < at + blocks[k].len;) {
-                    const int64_t w = p / 16 * 16, end = std::min(w + 16, at + blocks[k].len);
-                    if (word_buf != buf || word_at != w) flush();
-                    word_buf = buf;
-                    word_at = w;
-                    word.push_back(Run{k, sub, p - at, (int)(p - w), (int)(end - p)});
+                const int64_t at = (int64_t)sub * stride[buf] + addr[buf] + blocks[k].dst_off, last = at + blocks[k].len;
+                for (int64_t p = at; p < last;) {
+                    const int64_t w = p / 16 * 16, end = std::min(w + 16, last);
+                    if (words16.empty() || words16.back().buf != buf || words16.back().at != w) {
+                        finish();
+                        words16.push_back(Word{w, (uint32_t)runs.size(), 0, (uint8_t)buf, false, false});
+                    }
+                    runs.push_back(Run{(uint32_t)k, sub, p - at, (int)(p - w), (int)(end - p)});
                     p = end;
                 }
             }
-        flush();
         lo = hi;
     }
+    finish();
 
     // Words that this launch fills only in part are cheaper as smaller words, unless there are next to
     // none (the end of a row): with them all placed the irregular collective of 4 to 1024 bytes took
@@ -350,75 +339,93 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     // of their own, which need no merging (and where everything is a multiple of 4 bytes, the few are
     // cheaper in smaller words: one-pass irregular 735 against 685); where they are many, they stay
     // with their neighbours (118-byte blocks, one merged word in eight: 88 against 134 microseconds).
-    {
-        size_t merged = 0, partial = 0;
-        for (const Placed &w : placed) {
-            merged += w.from.size() > 1;
-            partial += !w.full;
-        }
-        const bool apart = merged * 12 < placed.size(), keep_partial = partial * 64 <= placed.size();
-        std::vector<Placed> plain, rest;
-        for (Placed &w : placed) {
-            if (!w.full && !keep_partial) cut(w.buf, w.at, w.runs);
-            else if (!apart) rest.push_back(std::move(w));
-            else if (w.full && w.from.size() == 1) plain.push_back(std::move(w));
-            else if (by4) cut(w.buf, w.at, w.runs);
-            else rest.push_back(std::move(w));
-        }
-        lone = plain.size();
-        placed.swap(plain);
-        placed.insert(placed.end(), rest.begin(), rest.end());
-        std::stable_sort(fine.begin(), fine.end(), [](const Fine &x, const Fine &y) { return x.buf != y.buf ? x.buf < y.buf : x.at < y.at; });
-    }
-    // Placed words in address order, so that the two halves of a 32-byte sector belong to one chunk: the
-    // lanes that store first, then those that only load.
-    for (size_t k = 0; k < placed.size();) {
-        const size_t end = k < lone ? lone : placed.size();
-        size_t n = 0, lanes = 0;
-        while (k + n < end && placed[k + n].buf == placed[k].buf && lanes + placed[k + n].from.size() <= 32) lanes += placed[k + n++].from.size();
-        if (k + n < end && n > 1 && placed[k + n].at % 32 != 0 && placed[k + n].at == placed[k + n - 1].at + 16) --n;
-        const size_t base = T.loads.size();
-        T.loads.resize(base + 32, LoadDev{});
-        size_t extra = n;
-        EntryDev ck{};
-        ck.kind = CHUNK_WHOLE;
-        ck.passes = 1;
-        ck.dst_buf = (uint8_t)placed[k].buf;
-        for (size_t e = 0; e < n; ++e) {
-            const Placed &w = placed[k + e];
-            T.loads[base + e] = w.from[0];
-            T.loads[base + e].stores = 1;
-            uint8_t other[2] = {(uint8_t)e, (uint8_t)e};
-            for (size_t q = 1; q < w.from.size(); ++q) {
-                other[q - 1] = (uint8_t)extra;
-                T.loads[base + extra++] = w.from[q];
+    const bool apart = merged * 12 < n_in_place, keep_partial = partial * 64 <= n_in_place;
+    std::vector<uint32_t> plain, rest;  // of words16
+    std::vector<Word> fine;
+    std::vector<Run> fine_runs;
+    for (uint32_t i = 0; i < words16.size(); ++i) {
+        const Word &w = words16[i];
+        if (w.in_place && (w.full || keep_partial)) {
+            if (apart && w.full && w.n == 1) {
+                plain.push_back(i);
+                continue;
             }
-            T.loads[base + e].second = other[0];
-            T.loads[base + e].third = other[1];
-            if (w.from.size() > 1 || !w.full) ck.kind = CHUNK_PLACED;
-            ck.passes = std::max<uint8_t>(ck.passes, (uint8_t)w.from.size());
+            if (!apart || !by4) {
+                rest.push_back(i);
+                continue;
+            }
         }
-        for (size_t e = n; e < 32; ++e) T.loads[base + e].second = T.loads[base + e].third = (uint8_t)e;
-        T.chunks.push_back(ck);
-        k += n;
+        for (uint32_t j = w.first; j < w.first + w.n; ++j) {
+            const Run &q = runs[j];
+            for (int at = q.begin; at < q.begin + q.n;) {
+                const int start = (int)(at / grain * grain), end = std::min(start + (int)grain, q.begin + q.n);
+                if (fine.empty() || fine.back().buf != w.buf || fine.back().at != w.at + start)
+                    fine.push_back(Word{w.at + start, (uint32_t)fine_runs.size(), 0, w.buf, false, false});
+                ++fine.back().n;
+                fine_runs.push_back(Run{q.block, q.sub, q.x + at - q.begin, at - start, end - at});
+                at = end;
+            }
+        }
     }
 
-    FineChunks chunks{T, (uint8_t)(by8 ? CHUNK_ONE8 : (by4 ? CHUNK_ONE4 : CHUNK_TWO))};
+    // Placed words in address order, so that the two halves of a 32-byte sector belong to one chunk: the
+    // lanes that store first, then those that only load.
+    for (const std::vector<uint32_t> *list : {&plain, &rest})
+        for (size_t k = 0; k < list->size();) {
+            auto word = [&](size_t i) -> const Word & { return words16[(*list)[i]]; };
+            size_t n = 0, lanes = 0;
+            while (k + n < list->size() && word(k + n).buf == word(k).buf && lanes + word(k + n).n <= 32) lanes += word(k + n++).n;
+            if (k + n < list->size() && n > 1 && word(k + n).at % 32 != 0 && word(k + n).at == word(k + n - 1).at + 16) --n;
+            const size_t first = T.loads.size();
+            T.loads.resize(first + 32, LoadDev{});
+            for (size_t e = 0; e < 32; ++e) T.loads[first + e].second = T.loads[first + e].third = (uint8_t)e;
+            size_t extra = n;
+            EntryDev ck{};
+            ck.kind = CHUNK_WHOLE;
+            ck.passes = 1;
+            ck.dst_buf = word(k).buf;
+            for (size_t e = 0; e < n; ++e) {
+                const Word &w = word(k + e);
+                for (uint32_t j = 0; j < w.n; ++j) {
+                    const Run &q = runs[w.first + j];
+                    const size_t lane = j == 0 ? e : extra++;
+                    const uint8_t second = T.loads[first + lane].second, third = T.loads[first + lane].third;
+                    LoadDev &ld = T.loads[first + lane];
+                    ld = base[q.block];
+                    ld.sub = (uint8_t)q.sub;
+                    ld.src_term += q.x - q.begin;
+                    ld.dst_term = w.at;
+                    ld.mask = (uint16_t)(((1u << q.n) - 1u) << q.begin);
+                    ld.second = second;
+                    ld.third = third;
+                    ld.stores = j == 0;
+                    if (j == 1) T.loads[first + e].second = (uint8_t)lane;
+                    if (j == 2) T.loads[first + e].third = (uint8_t)lane;
+                }
+                if (w.n > 1 || !w.full) ck.kind = CHUNK_PLACED;
+                ck.passes = std::max(ck.passes, w.n);
+            }
+            T.chunks.push_back(ck);
+            k += n;
+        }
+
+    FineChunks chunks{T, fine_runs, (uint8_t)(by8 ? CHUNK_ONE8 : (by4 ? CHUNK_ONE4 : CHUNK_TWO))};
+    std::vector<Placement> places(blocks.size());
+    for (size_t i = 0; i < blocks.size(); ++i) places[i] = placement(addr[blocks[i].src_buf] + blocks[i].src_off, stride[blocks[i].src_buf]);
     auto range = [&](const Run &q, int64_t &k0, int64_t &k1) -> int64_t {
-        const Block &b = blocks[q.block];
-        const Placement pl = placement(addr[b.src_buf] + b.src_off, stride[b.src_buf]);
+        const Placement &pl = places[q.block];
         k0 = (pl.lowest + q.x) / 16;
         k1 = (pl.highest + q.x + q.n - 1) / 16;
-        return at16(b.src_buf) ? pl.lowest : 0;  // (where it varies the kernel adds the row's own place)
+        return at16(blocks[q.block].src_buf) ? pl.lowest : 0;  // (where it varies the kernel adds the row's own place)
     };
     auto load = [&](const Run &q, int64_t k) {
-        const Block &b = blocks[q.block];
-        LoadDev ld = describe(b, q.sub);
-        if (at16(b.src_buf)) ld.src_term += k * 16 - (b.src_off & 15);  // the aligned word itself
+        LoadDev ld = base[q.block];
+        ld.sub = (uint8_t)q.sub;
+        if (at16(blocks[q.block].src_buf)) ld.src_term += k * 16 - (blocks[q.block].src_off & 15);  // the aligned word itself
         else ld.word = (int32_t)k;
         return ld;
     };
-    for (const Fine &w : fine) chunks.add(w.buf, w.at, w.runs, range, load);
+    for (const Word &w : fine) chunks.add(w, range, load);
     chunks.close();
     deal(T);
 }
