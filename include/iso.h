@@ -272,7 +272,9 @@ int Iso_request_set_slabs(Iso_request request, int slabs);
  * the CTA slots and with its own one-slab part of the intermediate buffer: the start and
  * the drain of one chain's short kernels are covered by the other chains.  The number of
  * slabs is rounded to a multiple of n; the launches are then replayed from a captured
- * graph (see Iso_request_set_graph).  1 (default) turns it off; at most 8.  Ignored where
+ * graph (see Iso_request_set_graph).  1 turns it off; at most 8.  Until this is called the
+ * library runs two chains (without a graph, on a second stream of its own beside the
+ * caller's) where it chooses the slabs itself and there are four or more.  Ignored where
  * slab execution is (see there).  The result never depends on it.
  */
 int Iso_request_set_chains(Iso_request request, int chains);

@@ -52,6 +52,10 @@ void release_device(Request &r)
     if (r.d_err) cudaFree(r.d_err);
     for (void *st : r.host_streams) cudaStreamDestroy(static_cast<cudaStream_t>(st));
     r.host_streams.clear();
+    for (void *st : r.chain_streams) cudaStreamDestroy(static_cast<cudaStream_t>(st));
+    r.chain_streams.clear();
+    for (void *e : r.chain_events) cudaEventDestroy(static_cast<cudaEvent_t>(e));
+    r.chain_events.clear();
     for (void *e : r.slab_events) cudaEventDestroy(static_cast<cudaEvent_t>(e));
     for (void *e : r.host_timing) cudaEventDestroy(static_cast<cudaEvent_t>(e));
     r.host_timing.clear();
@@ -1091,7 +1095,17 @@ void choose_slab_plan(Request &r)
         want = 1;
         while (want < target && c.P / (want * 2) >= 6 * rows_per_pass) want *= 2;
     }
-    int chains = std::max(1, r.chains_request);
+    // Left to the library, four slabs and more run as two chains of slabs half that size (as long as that
+    // leaves 512 processes to a slab): the ramp and the drain of one chain's launches are covered by the
+    // other.  Measured in microseconds per start: 2 KB blocks on 256x256 1546 -> 1417, 512 bytes 374 ->
+    // 358, 48^3 with 26 blocks of 128 bytes 247 -> 228, Moore r=3 542 -> 530, 16^4 283 -> 280, irregular
+    // 64x64x32 1389 -> 1324 (from a graph another 2 % faster, but the first start then takes up to 6 ms
+    // longer); two slabs made four (8^5 torus) lost, 155 -> 162, as did two chains without halving the
+    // slabs (shells, one plane of dimension 0 each: 2.65 -> 2.75 ms).
+    const bool two = r.chains_request == 0 && r.knobs.chains < 0 && r.slab_request == 0 && r.knobs.slabs < 0 && want >= 4 &&
+                     want * 2 <= c.dims[0] && c.P / (want * 2) >= 512;
+    if (two) want *= 2;
+    int chains = two ? 2 : std::max(1, r.chains_request);
     if (r.knobs.chains >= 0) chains = std::max(1, std::min(8, r.knobs.chains));
     if (chains > 1) want = std::max(want, chains) / chains * chains;
     if (want < 2) return;
@@ -1106,13 +1120,13 @@ void choose_slab_plan(Request &r)
     if (chains > 1 && slabs.size() % chains == 0) {
         // slabs side by side: every chain has its own one-slab part of the intermediate buffer
         r.chains = chains;
-        r.use_graph = true;
+        if (!two) r.use_graph = true;
         rows *= chains;
     }
     // a start of very many launches is replayed from a graph unless the environment says otherwise
     // (4 KB blocks on the 256x256 torus, 256 launches per start: 3.16 -> 3.10 ms; at 96 launches
     // per start and below replay measured no gain)
-    if (r.knobs.graph < 0 && r.slab_plan.size() * r.launches.size() >= 128) r.use_graph = true;
+    if (!two && r.knobs.graph < 0 && r.slab_plan.size() * r.launches.size() >= 128) r.use_graph = true;
     // the pipelined host-buffer path cuts dimension 0 into slabs of its own (plan_slabs)
     std::vector<SlabPlan> host;
     plan_slabs(r, host);
@@ -1125,10 +1139,28 @@ int check_handle(Iso_request request)
     return request && request->comm ? ISO_SUCCESS : ISO_ERR_ARG;
 }
 
-// Captures the launches of one Iso_Start into a graph.  With r.chains > 1 the slabs are
-// dealt to that many chains, which run side by side: chain k takes the slabs k, k + chains,
-// ..., a 1/chains share of the CTA slots and its own part of the intermediate buffer, so
-// that the ramp and the drain of one chain's kernels are covered by the other chains.
+// Enqueues the slabs as r.chains chains on the streams st (the caller forks and joins them): chain k takes
+// the slabs k, k + chains, ..., a 1/chains share of the CTA slots and its own part of the intermediate
+// buffer, so that the ramp and the drain of one chain's kernels are covered by the other chains.
+int enqueue_chains(Request &r, const std::vector<cudaStream_t> &st, bool use_pdl)
+{
+    const size_t n = st.size();
+    long long slab_rows = 0;
+    for (const auto &w : r.slab_plan) slab_rows = std::max(slab_rows, w.second - w.first);
+    for (size_t i = 0; i < r.slab_plan.size(); ++i) {
+        const size_t k = i % n;
+        const auto &w = r.slab_plan[i];
+        bool first = i < n;  // nothing of this chain precedes it in its stream
+        for (const LaunchPlan &L : r.launches) {
+            int rc = launch_one(r, L, st[k], use_pdl && !first, w.first, w.second, w.first - (long long)k * slab_rows, (int)n);
+            first = false;
+            if (rc != ISO_SUCCESS) return rc;
+        }
+    }
+    return ISO_SUCCESS;
+}
+
+// Captures the launches of one Iso_Start into a graph.
 int build_graph(Request &r, bool use_pdl)
 {
     const int n = std::max(1, r.chains);
@@ -1150,18 +1182,7 @@ int build_graph(Request &r, bool use_pdl)
     }
     if (e == cudaSuccess) {
         if (r.slab_plan.size() > 1) {
-            long long slab_rows = 0;
-            for (const auto &w : r.slab_plan) slab_rows = std::max(slab_rows, w.second - w.first);
-            for (size_t i = 0; i < r.slab_plan.size() && rc == ISO_SUCCESS; ++i) {
-                const int k = (int)(i % (size_t)n);
-                const auto &w = r.slab_plan[i];
-                bool first = i < (size_t)n;  // nothing of this chain precedes it in its stream
-                for (const LaunchPlan &L : r.launches) {
-                    rc = launch_one(r, L, st[k], use_pdl && !first, w.first, w.second, w.first - (long long)k * slab_rows, n);
-                    first = false;
-                    if (rc != ISO_SUCCESS) break;
-                }
-            }
+            rc = enqueue_chains(r, st, use_pdl);
         } else {
             bool first = true;
             for (const LaunchPlan &L : r.launches) {
@@ -1455,7 +1476,7 @@ int Iso_request_get_execution(Iso_request request, int *slabs, int *chains, int 
     if (check_handle(request)) return ISO_ERR_ARG;
     const Request &r = *request;
     if (slabs) *slabs = r.dirty ? r.slab_request : (int)std::max<size_t>(1, r.slab_plan.size());
-    if (chains) *chains = r.dirty ? r.chains_request : r.chains;
+    if (chains) *chains = r.dirty ? std::max(1, r.chains_request) : r.chains;
     if (graph) *graph = r.dirty ? (r.graph_request ? 1 : 0) : (r.use_graph ? 1 : 0);
     return ISO_SUCCESS;
 }
@@ -1787,6 +1808,36 @@ int Iso_Start(Iso_request request, void *cuda_stream)
             if (rc != ISO_SUCCESS) return rc;
         }
         ISO_CUDA(cudaGraphLaunch(static_cast<cudaGraphExec_t>(r.graph_exec), stream));
+        r.last_stream = cuda_stream;
+        r.started = true;
+        return ISO_SUCCESS;
+    }
+    if (r.slab_plan.size() > 1 && r.chains > 1) {
+        // two or more chains of slabs: the first on the caller's stream, the others beside it
+        std::vector<cudaStream_t> st(1, stream);
+        while (r.chain_streams.size() + 1 < (size_t)r.chains) {
+            cudaStream_t s;
+            ISO_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+            r.chain_streams.push_back(s);
+        }
+        while (r.chain_events.size() < (size_t)r.chains) {
+            cudaEvent_t e;
+            ISO_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            r.chain_events.push_back(e);
+        }
+        auto event = [&](int k) { return static_cast<cudaEvent_t>(r.chain_events[k]); };
+        ISO_CUDA(cudaEventRecord(event(0), stream));
+        for (int k = 1; k < r.chains; ++k) {
+            st.push_back(static_cast<cudaStream_t>(r.chain_streams[k - 1]));
+            ISO_CUDA(cudaStreamWaitEvent(st[k], event(0), 0));
+        }
+        int rc = enqueue_chains(r, st, use_pdl);
+        // the caller's stream waits for the other chains whatever happened
+        for (int k = 1; k < r.chains; ++k) {
+            ISO_CUDA(cudaEventRecord(event(k), st[k]));
+            ISO_CUDA(cudaStreamWaitEvent(stream, event(k), 0));
+        }
+        if (rc != ISO_SUCCESS) return rc;
         r.last_stream = cuda_stream;
         r.started = true;
         return ISO_SUCCESS;
