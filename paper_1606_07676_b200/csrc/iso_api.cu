@@ -850,6 +850,8 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
     return ISO_SUCCESS;
 }
 
+constexpr int64_t kHostSlabBytes = 3 << 19;  // bytes of a slab of the pipelined host-buffer path at least
+
 // Slabs of the leading dimension for the pipelined host-buffer path.
 struct SlabPlan {
     long long row_lo, row_hi;
@@ -882,7 +884,11 @@ void plan_slabs(const Request &r, std::vector<SlabPlan> &slabs, int want = 0)
     // default: up to 32 slabs.  The last slabs to arrive (a slab and the neighbours it reads
     // from) can only run and travel back after the final upload, so the tail of the pipeline
     // is about three slabs long: a quarter of the transfer time with 8 slabs, a tenth with 32.
-    int n = std::min(p0, 32);
+    // Small transfers take fewer: a slab costs its launches and two copies, 7 microseconds each at least
+    // (8^3 with 26 16-byte blocks, 213 KB each way, in 8 slabs 159 microseconds, in one 56; 1.7 MB in 10
+    // slabs 216, in one 111; 3.8 MB in 32 slabs 426, in 3 210; 6.8 MB in 16 slabs 352, in 4 to 6 320).
+    const int64_t bytes = c.P * std::max(r.send_stride, r.recv_stride);
+    int n = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(p0, 32), bytes / kHostSlabBytes));
     if (want > 0) {
         n = std::min(p0, want);
     } else if (r.knobs.host_slabs >= 0) {
