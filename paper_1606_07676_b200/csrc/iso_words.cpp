@@ -238,11 +238,13 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         rows = 1;
     } else {
         // Short rows: several of them share a chunk, so that its 32 loads are nearly all used (24 blocks of
-        // 4 bytes are 24 loads, a quarter of the lanes idle) - where enough warps remain, and in form 0,
-        // which knows no incomplete row group, where every slab is whole groups.
+        // 4 bytes are 24 loads, a quarter of the lanes idle) - as long as three warps per SM remain, and in
+        // form 0, which knows no incomplete row group, where every slab is whole groups.  (Asking for 96
+        // warps per SM instead: allgather of 24-byte blocks on 32^3 19.0 against 14.7 microseconds per start,
+        // 8-byte blocks on 300x290 13.5 against 8.4, 12-byte blocks on 100x90 6.1 against 4.8.)
         const int64_t whole = T.form == 1 ? 0 : (c.d >= 2 ? c.rank_stride[0] : c.P);
         while (rows * words < 96 && rows * 2 * bytes <= kWordsMostGroup && rows < 16 && whole % (rows * 2) == 0 &&
-               c.P * words / 28 >= 4ll * r.sm_count * (kWordsThreads / 32))
+               c.P * words / 28 >= 3ll * r.sm_count)
             rows *= 2;
     }
     T.rows_sub = (uint32_t)rows;
