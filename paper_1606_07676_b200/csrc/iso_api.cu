@@ -443,11 +443,15 @@ int materialise(Request &r)
         }
     }
     ISO_CUDA(cudaMemcpy(r.d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice));
-    if (!r.d_err) {
+    // the error flag, only where a kernel may raise it: the vector kernels wait for nothing, and reading the
+    // flag back would cost every Iso_wait a copy (8 microseconds)
+    r.reports = single || wave_n > 0;
+    for (const LaunchPlan *plan : plans) r.reports = r.reports || plan->kernel == KERNEL_BULK;
+    if (r.reports && !r.d_err) {
         ISO_CUDA(cudaMalloc((void **)&r.d_err, sizeof(int)));
         ISO_CUDA(cudaMemset(r.d_err, 0, sizeof(int)));
     }
-    if (!r.h_err) {
+    if (r.reports && !r.h_err) {
         ISO_CUDA(cudaMallocHost((void **)&r.h_err, sizeof(int)));
         *r.h_err = 0;
     }
@@ -1959,11 +1963,11 @@ int Iso_wait(Iso_request request)
     Request &r = *request;
     if (!r.started) return ISO_SUCCESS;
     cudaStream_t stream = static_cast<cudaStream_t>(r.last_stream);
-    if (r.d_err && r.h_err) {
+    if (r.reports) {
         ISO_CUDA(cudaMemcpyAsync(r.h_err, r.d_err, sizeof(int), cudaMemcpyDeviceToHost, stream));
     }
     ISO_CUDA(cudaStreamSynchronize(stream));
-    if (r.h_err && *r.h_err) {
+    if (r.reports && *r.h_err) {
         *r.h_err = 0;
         ISO_CUDA(cudaMemsetAsync(r.d_err, 0, sizeof(int), stream));
         if (r.d_counter) {

@@ -236,6 +236,7 @@ struct Request {
     unsigned char *d_inter_alloc = nullptr;  // the allocation: guard band, buffer, guard band
     int64_t d_inter_bytes = 0;
     int *d_err = nullptr;
+    bool reports = false;  // the plan has kernels that may raise the error flag (bulk copies, waits on other CTAs)
     unsigned long long *d_counter = nullptr;  // grid-barrier arrivals (one-launch execution)
     unsigned long long epoch = 0;             // counter value at the next launch
     int multi_grid = 0;                       // > 0: one-launch execution with this grid
