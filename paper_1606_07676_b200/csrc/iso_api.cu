@@ -511,6 +511,7 @@ LaunchDev make_launch_args(const Request &r, const LaunchPlan &L)
     // against 547; with few slabs the kept lines crowd out the streamed ones: 8 slabs (16^4 torus)
     // 284 against 281, 2 slabs (8^5 torus) 158 against 155, no slabs (32^3 torus) 38.6 against 37.1.
     a.keep_inter = (r.knobs.l2_keep && r.slab_plan.size() >= 16) ? 1u : 0u;
+    a.reverse = (uint32_t)(L.phase & 1);
     a.n_used = L.n_used;
     a.mesh_mask = 0;
     a.grid_share = 1;

@@ -77,6 +77,7 @@ struct LaunchDev {
     uint32_t tab_stride;     // coordinate table: 32-bit words per row (4 or 8)
     uint32_t side_offset;    // hybrid kernel, bulk side: byte offset of its staging area in shared memory
     uint32_t col_split;      // vector kernel: column chunks the CTAs are dealt to (0 or 1: a CTA covers whole rows)
+    uint32_t reverse;        // sender-side kernel: rows are visited from the last to the first
     uint32_t keep_inter;     // vector kernel, 16-byte units: stores into the intermediate buffer ask the L2 to evict them last
     const LoadDev *loads;    // launches of words: 32 per chunk
     const FineDev *fine;
@@ -536,10 +537,15 @@ __global__ void __launch_bounds__(1024, 1) iso_fan_rows(const __grid_constant__ 
         unsigned char *const B0 = L.buf[db0] + dt0, *const B1 = L.buf[db1] + dt1;
         unsigned char *const B2 = L.buf[db2] + dt2, *const B3 = L.buf[db3] + dt3;
         const long long s0 = L.buf_stride[db0], s1 = L.buf_stride[db1], s2 = L.buf_stride[db2], s3 = L.buf_stride[db3];
-        const long long src_step = rstep * stride_s;
+        // Every other phase goes through the rows backwards: it then begins with the parent blocks that the
+        // phase before it has just written, while they are still in the L2 (80 neighbours on 16^4: 96.8 ->
+        // 94.0 microseconds per start).
+        const bool reverse = L.reverse != 0;
+        const long long mirror = L.row_lo + L.row_hi - 1;
+        const long long src_step = (reverse ? -rstep : rstep) * stride_s;
 
         long long r_ld = r0;
-        const unsigned char *src_ld = L.buf[sb] + src_term + r0 * stride_s;
+        const unsigned char *src_ld = L.buf[sb] + src_term + (reverse ? mirror - r0 : r0) * stride_s;
 #pragma unroll
         for (int i = 0; i < DEPTH; ++i) {
             if (r_ld < r_end) {
@@ -550,7 +556,8 @@ __global__ void __launch_bounds__(1024, 1) iso_fan_rows(const __grid_constant__ 
             cp_async_commit();
         }
         uint4 *slot = ring;
-        for (long long r = r0; r < r_end; r += rstep) {
+        for (long long k = r0; k < r_end; k += rstep) {
+            const long long r = reverse ? mirror - k : k;
             cp_async_wait<DEPTH - 1>();
             const uint4 v = *slot;
             const uint32_t t = fastdiv(L.div_rstride[0], (uint32_t)r);
