@@ -149,6 +149,7 @@ constexpr int kWordsDepth = 16;               // words in flight per lane, as ma
 constexpr int kWordsDepthCoded = 12;          // ... and where the codes of the stages have to fit into 64 bits
 constexpr int kWordsThreads = 768;            // threads per SM, in one to three CTAs
 constexpr int64_t kWordsSmallLaunch = 12 << 20;  // bytes up to which a launch of 16-byte units runs as words
+constexpr int64_t kWordsScattered = 96 << 20;    // bytes from which one with scattered loads does
 constexpr int kWordsPasses = 4;               // passes over a chunk's words at most
 constexpr uint32_t kWordsPadFront = 16, kWordsPadBack = 48;  // shared memory around the ring that a shifted read may touch
 

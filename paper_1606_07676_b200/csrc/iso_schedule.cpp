@@ -1129,8 +1129,23 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                         // 64-byte blocks 9.4 against 7.2 microseconds, 16^3 12.8 against 8.7 (2.4 MB per launch),
                         // 60x60 with 24 blocks of 128 bytes 9.0 against 7.7 (9 MB), but 40x40 with 512-byte blocks
                         // 12.2 against 12.9 (16 MB) and 9^4 with 80 64-byte blocks 30.3 against 33.8 (22 MB).
-                        const bool small = width == 16 && (int64_t)c.P * (int64_t)units * 16 <= kWordsSmallLaunch && !r.persistent &&
-                                           r.wave_request == 0 && r.knobs.vec_threads == 0;
+                        // So are launches in which a block moves along three dimensions and more, whose scattered
+                        // loads gain from warps that run independently of one another: allgathers (64-byte
+                        // blocks in one pass, 16^4 125 against 79 microseconds, 32^3 16.7 against 15.2), and
+                        // all-to-alls from 96 MB of blocks of 64 bytes (64^3 184 against 150, 48^3 74.6 against
+                        // 67.5; 32^3, 54 MB, 20.4 against 22.4; 32-byte blocks on 64^3 73.7 against 78.9) or in
+                        // more dimensions (8^5 with 16-byte blocks 65 against 58), as long as a row fits a
+                        // CTA (1396 neighbours 1340 against 1391); and meshes.
+                        int64_t min_len = INT64_MAX;
+                        bool mesh_launch = false;
+                        for (const LoweredPart &lp : L.parts) min_len = std::min(min_len, lp.p.len);
+                        for (int k = 0; k < L.n_used; ++k) mesh_launch = mesh_launch || !c.periodic[L.used_dim[k]];
+                        const bool scattered = mesh_launch ||
+                                               (L.n_used >= 3 && (r.kind == ISO_KIND_ALLGATHER ||
+                                                                  ((int64_t)c.P * (int64_t)units * 16 >= kWordsScattered && units <= 1024 &&
+                                                                   (L.n_used > 3 || min_len >= 64))));
+                        const bool small = width == 16 && ((int64_t)c.P * (int64_t)units * 16 <= kWordsSmallLaunch || scattered) &&
+                                           !r.persistent && r.wave_request == 0 && r.knobs.vec_threads == 0;
                         L.words = kernel == KERNEL_VEC && (width != 16 || small) && longs.empty() && !tiny;
                         L.compact = kernel == KERNEL_VEC && !L.words && L.n_used > 3 && L.max_nnz < L.n_used &&
                                     torus && !r.persistent;  // (the pipelined one-launch kernel does take compact launches)

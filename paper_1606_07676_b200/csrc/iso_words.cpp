@@ -241,9 +241,14 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         // 4 bytes are 24 loads, a quarter of the lanes idle) - as long as three warps per SM remain, and in
         // form 0, which knows no incomplete row group, where every slab is whole groups.  (Asking for 96
         // warps per SM instead: allgather of 24-byte blocks on 32^3 19.0 against 14.7 microseconds per start,
-        // 8-byte blocks on 300x290 13.5 against 8.4, 12-byte blocks on 100x90 6.1 against 4.8.)
+        // 8-byte blocks on 300x290 13.5 against 8.4, 12-byte blocks on 100x90 6.1 against 4.8; 26 64-byte
+        // blocks, 104 words, one row to a group instead of four: 64^3 in one pass 168 against 150.)
         const int64_t whole = T.form == 1 ? 0 : (c.d >= 2 ? c.rank_stride[0] : c.P);
-        while (rows * words < 96 && rows * 2 * bytes <= kWordsMostGroup && rows < 16 && whole % (rows * 2) == 0 &&
+        auto uneven = [&]() {  // too few words, or a last chunk of which a good part is idle
+            const int64_t n = rows * words;
+            return n < 96 || ((n + 31) / 32 * 32 - n) * 100 > 7 * n;
+        };
+        while (uneven() && rows * 2 * bytes <= kWordsMostGroup && rows < 16 && whole % (rows * 2) == 0 &&
                c.P * words / 28 >= 3ll * r.sm_count)
             rows *= 2;
     }
