@@ -711,6 +711,9 @@ cudaError_t launch_hybrid(Kernel kernel, const LaunchPlan &L, const LaunchDev &a
 template <int W, int NU, bool MESH, bool COMPACT>
 cudaError_t launch_rows_wide(bool tab, const LaunchPlan &L, const LaunchDev &a, cudaStream_t stream, bool dependent)
 {
+    if constexpr (W == 16 && !MESH && !COMPACT && NU >= 1 && NU <= 2) {
+        if (tab && a.keep_inter) return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, true, true>, L, a, stream, dependent, table_bytes(a));
+    }
     if constexpr (!MESH && (COMPACT || NU <= 2)) {
         if (tab) return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, true>, L, a, stream, dependent, table_bytes(a));
     }

@@ -315,7 +315,14 @@ __device__ __forceinline__ UnitRegs load_unit(const LaunchDev &L, uint32_t u)
 // then reads its row's entry with one shared-memory load.  The direct schedule, three wrap
 // tests per row, spent 110 instructions per 16-byte unit and ran at 70 % issue utilisation
 // with the integer-multiply pipe as the top stall; the table removes that arithmetic.
-template <int W, int DEPTH, int NU, bool MESH, bool COMPACT, bool TAB = false>
+//
+// HINT: the launch may be part of a slab execution with many slabs, whose stores into the intermediate
+// buffer ask the L2 to evict them last.  A variant of its own because the policy's registers cost the
+// launches that never use it 2 to 4 %: 32^3 with 26 64-byte blocks 37.3 against 35.8 microseconds per
+// start, 8^5 with 16-byte blocks 155.2 against 151.8.  (Marking the loads from the send buffers and the
+// stores into the receive buffers evict_first as well: Moore r=3 529 -> 513, but shells 2654 -> 2697 and
+// 16^4 281 -> 285.)
+template <int W, int DEPTH, int NU, bool MESH, bool COMPACT, bool TAB = false, bool HINT = false>
 __device__ __forceinline__ void gather_rows_body(const LaunchDev &L, unsigned char *ring_base, bool dependent_launch,
                                                  uint32_t cta, uint32_t n_cta, const uint32_t nthr)
 {   // nthr: threads of the CTA that run this body (all of them, except in the hybrid kernel)
@@ -378,7 +385,7 @@ __device__ __forceinline__ void gather_rows_body(const LaunchDev &L, unsigned ch
 #pragma unroll
         for (int e = 0; e < NU; ++e) wrap_bytes[e] = (long long)L.used_wrap[dim_of(e)] * R.stride_s;
         const long long src_step = rstep * R.stride_s, dst_step = rstep * R.stride_d;
-        const bool keep = W == 16 && L.keep_inter && R.to_inter;
+        const bool keep = W == 16 && HINT && L.keep_inter && R.to_inter;
         const uint64_t policy = keep ? l2_policy_evict_last() : 0;
 
         // `row`: the row's entry of the coordinate table (TAB), unused otherwise
@@ -466,11 +473,11 @@ __global__ void __launch_bounds__(256, 4) iso_gather_rows(const __grid_constant_
 // The same body in CTAs of up to 1024 threads, for launches whose payload per process has
 // more than 256 unit positions: one CTA then covers up to 16 KB of a row at a time, so rows
 // are still visited one after the other instead of in 4 KB columns.
-template <int W, int DEPTH, int NU, bool MESH, bool COMPACT, bool TAB>
+template <int W, int DEPTH, int NU, bool MESH, bool COMPACT, bool TAB, bool HINT = false>
 __global__ void __launch_bounds__(1024, 1) iso_gather_rows_wide(const __grid_constant__ LaunchDev L)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    gather_rows_body<W, DEPTH, NU, MESH, COMPACT, TAB>(L, smem_raw, true, blockIdx.x, gridDim.x, blockDim.x);
+    gather_rows_body<W, DEPTH, NU, MESH, COMPACT, TAB, HINT>(L, smem_raw, true, blockIdx.x, gridDim.x, blockDim.x);
 }
 
 // Sender-side form of an allgather phase.  In the prefix-trie schedule (Section III-B) a node's

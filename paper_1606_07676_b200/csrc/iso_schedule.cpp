@@ -1128,7 +1128,8 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                         // start before this one drains.  Measured per start, wide CTAs against words: 8^3 with 26
                         // 64-byte blocks 9.4 against 7.2 microseconds, 16^3 12.8 against 8.7 (2.4 MB per launch),
                         // 60x60 with 24 blocks of 128 bytes 9.0 against 7.7 (9 MB), but 40x40 with 512-byte blocks
-                        // 12.2 against 12.9 (16 MB) and 9^4 with 80 64-byte blocks 30.3 against 33.8 (22 MB).
+                        // 12.2 against 12.9 (16 MB), 9^4 with 80 64-byte blocks 30.3 against 33.8 (22 MB) and, with
+                        // rows longer than a CTA, 8x6x10 with 342 64-byte blocks 12.7 against 13.6.
                         // So are launches in which a block moves along three dimensions and more, whose scattered
                         // loads gain from warps that run independently of one another: allgathers (64-byte
                         // blocks in one pass, 16^4 125 against 79 microseconds, 32^3 16.7 against 15.2), and
@@ -1144,7 +1145,7 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                                                (L.n_used >= 3 && (r.kind == ISO_KIND_ALLGATHER ||
                                                                   ((int64_t)c.P * (int64_t)units * 16 >= kWordsScattered && units <= 1024 &&
                                                                    (L.n_used > 3 || min_len >= 64))));
-                        const bool small = width == 16 && ((int64_t)c.P * (int64_t)units * 16 <= kWordsSmallLaunch || scattered) &&
+                        const bool small = width == 16 && (((int64_t)c.P * (int64_t)units * 16 <= kWordsSmallLaunch && units <= 1024) || scattered) &&
                                            !r.persistent && r.wave_request == 0 && r.knobs.vec_threads == 0;
                         L.words = kernel == KERNEL_VEC && (width != 16 || small) && longs.empty() && !tiny;
                         L.compact = kernel == KERNEL_VEC && !L.words && L.n_used > 3 && L.max_nnz < L.n_used &&
