@@ -54,6 +54,13 @@ def test_block_sizes(m, call):
     _compare(wl.Workload("w", call, (5, 9, 4), wl.moore(3, 1), m, seed=m + 2), periodic=[0, 1, 0])
 
 
+@pytest.mark.parametrize("m", [113, 242, 252, 260, 371])
+def test_blocks_over_two_chunks(m):
+    # long blocks whose lanes do not fill a chunk of 32: they go on in the next one
+    _compare(wl.Workload("w", "alltoall", (6, 5, 7), wl.moore(3, 1), m, seed=m), lead=(m % 16, 3))
+    _compare(wl.Workload("w", "allgather", (13, 11), wl.moore(2, 2), m, seed=m + 1), periodic=[0, 1])
+
+
 @pytest.mark.parametrize("seed", range(6))
 def test_irregular_sizes(seed):
     rng = np.random.default_rng(seed)
