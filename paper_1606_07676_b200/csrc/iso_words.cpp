@@ -57,7 +57,7 @@ Placement placement(int64_t addr, int64_t stride)
 // Deals warps to the chunks in proportion to what a row costs in them, so that all warps of a launch
 // are done at the same time.  The weights are measured, in units of which a row of whole words costs
 // 50: with equal shares the 27-point stencil of faces, edges and corners took 222 microseconds in three
-// phases on a mesh, with these 159.
+// phases on a mesh, with these 166.
 // (Placed chunks at 60, so that they got as many warps as whole ones: those warps finished last, 32^3 with
 // blocks of 1024, 32 and 1 bytes in one pass 103.7 against 87.7 microseconds, the same on a mesh 169.0
 // against 166.2, 64x64x32 with 30 blocks of 4 to 1024 bytes 1334 against 1316; anything from 70 to 100 is
