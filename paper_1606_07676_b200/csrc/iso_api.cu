@@ -2291,15 +2291,21 @@ extern "C" int Iso_neighbor_alltoall_static(int d, const int dims[], int s, cons
     rc = lower_schedule(r, (uintptr_t)r.send, (uintptr_t)r.recv, (uintptr_t)scratch);
     if (rc != ISO_SUCCESS) return rc;
     int64_t table_bytes = 0;
-    for (LaunchPlan &L : r.launches) {
-        if (L.kernel != KERNEL_VEC) return ISO_ERR_STATE;
-        if (L.words) {
-            plan_words(r, L, (uintptr_t)scratch);
-            table_bytes += (int64_t)words_place(L, (size_t)table_bytes);
-            continue;
+    for (bool again = true; again;) {
+        table_bytes = 0;
+        for (LaunchPlan &L : r.launches) {
+            if (L.kernel != KERNEL_VEC) return ISO_ERR_STATE;
+            if (L.words) {
+                plan_words(r, L, (uintptr_t)scratch);
+                table_bytes += (int64_t)words_place(L, (size_t)table_bytes);
+                continue;
+            }
+            L.units_off = (size_t)table_bytes;
+            table_bytes += (int64_t)L.units_per_proc * (int64_t)sizeof(UnitDev);
         }
-        L.units_off = (size_t)table_bytes;
-        table_bytes += (int64_t)L.units_per_proc * (int64_t)sizeof(UnitDev);
+        // tables that describe 16 rows may not fit where those of one row do
+        again = inter_bytes + table_bytes > (int64_t)ISO_STATIC_SCRATCH_BYTES && !r.lean_tables;
+        if (again) r.lean_tables = true;
     }
     if (inter_bytes + table_bytes > (int64_t)ISO_STATIC_SCRATCH_BYTES) return ISO_ERR_TOO_LARGE;
 

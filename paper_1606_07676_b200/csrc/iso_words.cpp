@@ -237,10 +237,10 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     // (several meet in a destination word) and the tables stay small.
     if (dst_fixed) rows = 1;
     if (fixed) T.form = mesh ? 1 : 0;
-    else T.form = moving_bytes < kWordsLongBlock * moving && rows * bytes <= kWordsMostGroup ? 1 : 2;
+    else T.form = moving_bytes < kWordsLongBlock * moving && rows * bytes <= kWordsMostGroup && (rows == 1 || !r.lean_tables) ? 1 : 2;
     if (T.form == 2) {
         rows = 1;
-    } else {
+    } else if (!r.lean_tables) {
         // Short rows: several of them share a chunk, so that its 32 loads are nearly all used (24 blocks of
         // 4 bytes are 24 loads, a quarter of the lanes idle) - as long as three warps per SM remain, and in
         // form 0, which knows no incomplete row group, where every slab is whole groups.  (Asking for 96

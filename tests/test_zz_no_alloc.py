@@ -34,7 +34,8 @@ def _cases():
     odd = np.array([[0, 0, 0], [1, 0, -1], [1, 0, -1], [-5, 3, 2], [0, 1, 0], [2, 2, 2]], np.int32)  # zero vector, a repeat, |c| >= p
     return [((8, 8, 8), wl.moore(3, 1), 64, 11), ((12, 10), wl.moore(2, 2), 24, 12),
             ((7, 5), wl.moore(2, 1), 1, 13), ((6, 4, 3), wl.moore(3, 1), 2, 14), ((9, 11), wl.moore(2, 2), 20, 15),
-            ((3, 1, 2), odd, 16, 16), ((2, 2), wl.moore(2, 1), 48, 17), ((5, 4, 3, 2), wl.moore(4, 1), 8, 18)]
+            ((3, 1, 2), odd, 16, 16), ((2, 2), wl.moore(2, 1), 48, 17), ((5, 4, 3, 2), wl.moore(4, 1), 8, 18),
+            ((5, 5, 4, 3), wl.moore(4, 3)[:2001], 1, 19)]  # word tables of 16 rows would not fit into the scratch area
 
 
 def test_static_entry_point_matches_the_oracle_twice_in_a_row():
