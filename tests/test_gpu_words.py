@@ -77,3 +77,10 @@ def test_many_rows_and_slabs(m):
     _compare(wl.Workload("w", "alltoall", (61, 257), wl.moore(2, 2), m, seed=m))
     _compare(wl.Workload("w", "alltoall", (61, 257), wl.moore(2, 1), m, seed=m), slabs=7)
     _compare(wl.Workload("w", "alltoall", (96, 512), wl.moore(2, 1), m, seed=m), slabs=3)
+
+
+@pytest.mark.parametrize("dims,offs,m", [((1300001,), wl.positive_octant(1, 1), 17), ((811, 803), wl.positive_octant(2, 1)[:1], 9),
+                                         ((61, 53, 59), wl.moore(3, 3), 3), ((31, 30, 29), wl.moore(3, 3), 48), ((15, 14, 16, 17), wl.moore(4, 1), 20)])
+def test_coordinates_without_a_table(dims, offs, m):
+    # launches whose table of coordinates does not fit beside the rings: every lane divides
+    _compare(wl.Workload("w", "allgather", dims, offs, m, seed=m))
