@@ -815,6 +815,9 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
                             : launch_hybrid(iso_gather_rows_hybrid<kHybridDepth, 3, false>, L, a, sd, smem, stream, dependent);
     } else if (L.words) {
         e = launch_words(L, a, stream, dependent);
+    } else if (L.width > 0 && L.width < 4) {
+        e = L.width == 2 ? launch_kernel(iso_gather_rows_reg<2, 4>, L, a, stream, dependent, 0)
+                         : launch_kernel(iso_gather_rows_reg<1, 4>, L, a, stream, dependent, 0);
     } else {
         // kernels specialised on the number of shifted dimensions; meshes take the general one
         // (with compact unit descriptors: on the dimensions one unit is shifted along)
@@ -826,7 +829,7 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
         // dimension, and on the compact last phase of 16-byte blocks; the one-pass direct
         // schedules, three or more wrap tests per row, are bound by the latency of their
         // scattered loads and gain nothing, so they keep the divisions)
-        if (L.width == 16 && L.threads > 256 && L.n_used > 0 && r.knobs.coord_table &&
+        if ((L.width == 16 || L.width == 0) && L.threads > 256 && L.n_used > 0 && r.knobs.coord_table &&
             (L.compact || nu <= 2) && !a.mesh_mask) {
             const long long groups = (a.row_hi - a.row_lo + L.rows_per_pass - 1) / L.rows_per_pass;
             const long long grid = grid_for_rows(L, a, a.grid_share) / std::max(1, L.col_split);  // CTAs that share the rows
@@ -836,8 +839,9 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
             if (!tab) a.tab_iters = 0;
         }
 #define ISO_ROWS(W, NU, MESH, COMPACT)                                                                          \
-    e = (W == 16 && L.threads > 256) ? launch_rows_wide<16, NU, MESH, COMPACT>(tab, L, a, stream, dependent)    \
-                                     : launch_kernel(iso_gather_rows<W, kVecDepth, NU, MESH, COMPACT>, L, a, stream, dependent, 0)
+    e = ((W == 16 || W == 0) && L.threads > 256)                                                                \
+            ? launch_rows_wide<(W == 0 ? 0 : 16), NU, MESH, COMPACT>(tab, L, a, stream, dependent)             \
+            : launch_kernel(iso_gather_rows<W, kVecDepth, NU, MESH, COMPACT>, L, a, stream, dependent, 0)
 #define ISO_ROWS_W(W)                                                            \
     do {                                                                         \
         if (a.mesh_mask) ISO_ROWS(W, ISO_MAX_DIMS, true, false);                 \
@@ -851,7 +855,9 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
         else if (nu == 3) ISO_ROWS(W, 3, false, false);                          \
         else ISO_ROWS(W, ISO_MAX_DIMS, false, false);                            \
     } while (0)
-        if (L.width == 16) ISO_ROWS_W(16);
+        if (L.width == 0) ISO_ROWS_W(0);
+        else if (L.width == 16) ISO_ROWS_W(16);
+        else if (L.width == 8) ISO_ROWS_W(8);
         else ISO_ROWS_W(4);
 #undef ISO_ROWS_W
 #undef ISO_ROWS

@@ -207,6 +207,7 @@ struct Knobs {
     bool coord_table = true;  // ISO_COORD_TABLE=0: row coordinates by division in every thread
     bool l2_keep = true;      // ISO_L2_KEEP=0: no eviction-priority hint on stores into the intermediate buffer
     int ag_order = -1;        // ISO_AG_ORDER=0/1: allgather visits the dimensions first-to-last / last-to-first
+    int words = -1;           // ISO_WORDS: 0 = no launches of words, 1 = wherever they can be (-1: chosen by the library)
 };
 Knobs read_knobs();
 

@@ -738,6 +738,57 @@ __global__ void __launch_bounds__(1024, 1) iso_gather_rows_wave(const __grid_con
     }
 }
 
+// Same ownership scheme with the data held in registers, for 1- and 2-byte units (cp.async
+// moves at least 4 bytes): UNROLL independent loads in flight before the first store.
+template <int W, int UNROLL>
+__global__ void __launch_bounds__(256) iso_gather_rows_reg(const __grid_constant__ LaunchDev L)
+{
+    using V = typename VecOf<W>::type;
+    const uint32_t CU = L.chunk_units, U = L.units_per_proc;
+    const int G = (int)L.rows_per_pass;
+    const int g = (int)(threadIdx.x / CU);
+    const uint32_t ul = threadIdx.x - (uint32_t)g * CU;
+    grid_dependency_wait();
+    grid_launch_dependents();
+    const long long r0 = L.row_lo + (long long)G * blockIdx.x + g;
+    if (g >= G || r0 >= L.row_hi) return;
+    const long long rstep = (long long)G * gridDim.x;
+
+    for (uint32_t u = ul; u < U; u += CU) {
+        const UnitRegs R = load_unit(L, u);
+        for (long long rb = r0; rb < L.row_hi; rb += rstep * UNROLL) {
+            V val[UNROLL];
+            V *dst[UNROLL];
+#pragma unroll
+            for (int k = 0; k < UNROLL; ++k) {
+                const long long r = rb + k * rstep;
+                dst[k] = nullptr;
+                if (r < L.row_hi) {
+                    long long wrap = 0;
+                    bool valid = true;
+                    for (int e = 0; e < L.n_used; ++e) {
+                        const uint32_t t = fastdiv(L.div_rstride[e], (uint32_t)r);
+                        const int x = (int)(t - fastdiv(L.div_size[e], t) * L.used_size[e]);
+                        if ((L.mesh_mask >> e) & 1) {
+                            const int y = x - R.c[e];
+                            valid = valid && y >= 0 && y < (int)L.used_size[e];
+                        } else if (x < R.c[e]) {
+                            wrap += L.used_wrap[e];
+                        }
+                    }
+                    if (valid) {
+                        val[k] = *reinterpret_cast<const V *>(R.A + (r + wrap) * R.stride_s);
+                        dst[k] = reinterpret_cast<V *>(R.B + r * R.stride_d);
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < UNROLL; ++k)
+                if (dst[k]) *dst[k] = val[k];
+        }
+    }
+}
+
 // Does nothing: a chain of these measures what a kernel launch costs on the stream
 // (with and without programmatic dependent launch), the floor under every short phase.
 __global__ void iso_empty_kernel(int)

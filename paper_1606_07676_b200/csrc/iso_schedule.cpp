@@ -66,6 +66,7 @@ Knobs read_knobs()
     k.col_split = num("ISO_COL_SPLIT", 1) != 0;
     k.ag_order = num("ISO_AG_ORDER", -1);
     k.l2_keep = num("ISO_L2_KEEP", 1) != 0;
+    k.words = (int)num("ISO_WORDS", -1);
     return k;
 }
 
@@ -742,6 +743,86 @@ int common_alignment(std::initializer_list<int64_t> xs)
     return a;
 }
 
+// What a launch is made of, for the choice between words and units.
+struct LaunchShape {
+    int n_used = 0;      // shifted dimensions
+    bool torus = true;   // all of them periodic
+    int64_t blocks = 0, bytes = 0, units = 0, words = 0;  // per process
+    int64_t lanes = 0;   // that the blocks take where each has a group of lanes to itself (build_words, form 2)
+    int64_t longest = 0, shortest = INT64_MAX;            // block lengths
+    int64_t short_bytes = 0;  // in blocks of less than 4 bytes
+    int64_t moving = 0;  // blocks whose place inside a 16-byte word changes from row to row
+    int64_t apart = 0;   // others whose place in the source's words is not the one in the destination's
+    int64_t from_send = 0;    // bytes read from the send buffer
+};
+
+// Launches that move in units although they could move as words.  Words pay for whole 16-byte loads, for lanes
+// without work where a row has few words, and for putting words together; units pay for a load and a store
+// per unit, a division per dimension and row, and badly for rows longer than a CTA and more than two dimensions.
+// Microseconds per start, units against words:
+bool better_in_units(const Request &r, int width, const LaunchShape &s)
+{
+    const Comm &c = *r.comm;
+    if (!s.torus || s.blocks == 0) return false;  // (meshes: 1.4 to 4 times slower in units)
+    const int64_t mean = s.bytes / s.blocks;
+    // rows the grid holds at a time (four CTAs of 256 threads per SM)
+    const int64_t at_once = (int64_t)r.sm_count * 4 * std::max<int64_t>(1, 256 / std::max<int64_t>(1, s.units));
+    // 4-byte blocks and nothing else: a word would be a 16-byte load for every 4 bytes, and those loads do
+    // not share sectors through the L1 (256x256, 24 neighbours 12.3 against 13.9, one pass 7.6 against 8.9).
+    if (width == 4 && s.longest == 4 && s.shortest == 4) return true;
+    // Likewise blocks of one 8-, 2- or 1-byte unit that an allgather reads from send buffers which hold nothing else: 8
+    // bytes, 63 neighbours on 35x34x33 in one pass 14.9 against 24.7; 1 byte, 342 on 15x14x16 10.8 against 85; 2 bytes, 22
+    // on 14544 4.4 against 7.1, but, along four dimensions, 15 on 16x12x13x14 8.1 against 6.5.
+    if (s.longest == width && s.shortest == width && r.kind == ISO_KIND_ALLGATHER && s.from_send == s.bytes && (width == 8 || s.n_used <= 3))
+        return true;
+    // Multiples of 8 bytes whose places change from row to row, or are others in the source than in the destination:
+    // launches that keep the grid busy.  Along one dimension: 88 bytes, 2 neighbours on 187299 11 against 40 and 1 on 8276
+    // 3.1 against 4.5; 120 bytes, 15 on 212x205 60 against 79; 504 bytes, 3 on 114x103 14.2 against 16.4; 24 bytes, 12 on 89060
+    // 9.1 against 12.6 (allgather; all-to-all, 63 on 40x26x38 130 against 120); but with fewer rows (1112 bytes, 7 on 2172)
+    // 10.5 against 9.2, with longer blocks (872 bytes, 5 on 115576) 234 against 194, and an allgather's phase of 714 units per
+    // row (136 bytes, 48 on 385x229) 272 against 246.  Along two: 88 bytes, 15 neighbours on 169x176 19.3 against 26.4, but 24
+    // bytes, 8 on 350x200 7.7 against 7.3 and 568 bytes, 8 on 128x128 32 against 30.  Along three: 312 bytes, 7 on 39x38x33 61
+    // against 49.  Nor rows of more than a CTA in slabs, whose
+    // launches are short (232 bytes, 63 on 31x32x30 535 against 485; but 248 bytes, 7 on 60x68x59 291 against 361).
+    const bool slabs = s.units > 256 && r.kind != ISO_KIND_ALLGATHER && r.inter_stride > 0 && c.P * s.bytes >= (int64_t)96 << 20;
+    if (width == 8 && !slabs && (s.moving == s.blocks || (s.moving == 0 && 4 * s.apart >= s.blocks && s.units <= 640 && mean >= 64))) {
+        if (s.longest == 8) return s.n_used <= 2 && c.P >= 5 * at_once;
+        if (mean < 64) return s.n_used <= 1 && (mean >= 32 || r.kind == ISO_KIND_ALLGATHER) && c.P >= 12 * at_once;
+        if (s.n_used <= 1) return mean <= 820 && 2 * c.P >= at_once * (s.units <= 128 ? 1 : (s.units <= 512 ? 7 : 16));
+        return s.n_used == 2 && mean <= 400 && c.P >= (s.units <= 128 ? 5 : 10) * at_once;
+    }
+    // Multiples of 4 bytes, likewise, along one dimension, where groups of lanes leave much of a chunk of 32 idle: 68 bytes,
+    // 2 neighbours on 151916 13 against 33, 6 on 112145 27 against 47; 100 bytes, 3 on 233x264 17.6 against 28.6; at 70 % (92
+    // bytes, 4 blocks a phase, 39x31x40) 38 against 36.  Of 12 bytes: 12 neighbours on 277867 21.7 against 28.5.
+    if (width == 4 && s.moving == s.blocks && s.n_used <= 1) {
+        if (mean >= 64) return s.bytes * 10 <= (s.lanes + 31) / 32 * 512 * 6 && c.P >= 3 * at_once;
+        return mean <= 12 && c.P >= 12 * at_once;
+    }
+    // Blocks of a byte or two between longer ones in one pass: a 16-byte load for each.  49 and 7 bytes to some, 1 byte to most of
+    // 342 neighbours on 13x11x10 5.4 against 7.1, 100 and 10 bytes, 38x46x37 178 against 230.
+    if (width == 0 && s.n_used == 3) return 5 * s.short_bytes >= s.bytes && s.longest > 4;
+    // And along two where hops of two dimensions are composed (and in the phases of such a schedule along one): 26 stencil blocks
+    // of 961, 31 and 1 bytes on 26x19x18 43 against 56, of 441, 21 and 1 bytes on 40x27x48 104 against 125.
+    if (width == 0 && (s.n_used == 2 || (s.n_used == 1 && r.fusion >= 2 && r.alg == ISO_ALG_COMBINING))) return s.short_bytes > 0;
+    return false;
+}
+
+// Short rows whose words could share a chunk of 32 loads only if the planes of dimension 0 (or, in one
+// dimension, the processes) divided into groups of rows, and do not (build_words, form 0): units once the launch
+// is long.  16 bytes, 2 neighbours on 145571 3.9 against 9.6; 40 bytes, 2 on 117495 6.1 against 10.9; but 72 bytes, 6 on
+// 43779 8.5 against 6.9, 20 bytes, 8 on 120x177 4.8 against 4.2 and, short, 16 bytes, 7 on 20x15x11 9.4 against 8.1.
+// With blocks of a byte or two among them, which take a pass over the bytes of every word, rows up to twice
+// as long: 144, 12 and 1 bytes, 26 on 31x57x53 55 against 86, 81, 9 and 1 bytes, 7 on 24x35x21 14.3 against 20.6; but 26 of
+// 196, 14 and 1 bytes on 23x25x19 21 against 21.
+bool rows_do_not_group(const Request &r, int width, const LaunchShape &s)
+{
+    const Comm &c = *r.comm;
+    const int64_t whole = c.d >= 2 ? c.rank_stride[0] : c.P;
+    int64_t group = 1;
+    while (group < 16 && whole % (group * 2) == 0) group *= 2;
+    return s.torus && s.moving == 0 && s.words * group <= (width == 0 ? (s.short_bytes > 0 ? 64 : 12) : 8) && c.P * s.words >= 100000;
+}
+
 }  // namespace
 
 // Whether the schedule can run slab by slab (see plan_slabs in iso_api.cu): every part that
@@ -894,7 +975,8 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
         if (r.knobs.mixed >= 0) allow_mixed = allow_mixed && r.knobs.mixed != 0;
         // split every part into pieces that share one alignment class
         // cls: width class of the launch (0: mixed widths); base: alignment of the rows it touches
-        struct Piece { Part p; int kernel; int width; int cls; int base; };
+        // (block: length of the part it is cut from; first: no piece of that part precedes it)
+        struct Piece { Part p; int kernel; int width; int cls; int base; int64_t block; bool first; };
         std::vector<Piece> pieces;
         for (size_t k = begin; k < end; ++k) {
             const Part &p = r.parts[k];
@@ -910,6 +992,8 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                 q.kernel = (q.width == 16 && r.bulk_threshold > 0 && len >= r.bulk_threshold) ? KERNEL_BULK : KERNEL_VEC;
                 q.cls = q.width;
                 q.base = base;
+                q.block = p.len;
+                q.first = rel == 0;
                 pieces.push_back(q);
             };
             const bool co_aligned = base == 16 && ((p.src_off - p.dst_off) & 15) == 0;
@@ -1056,11 +1140,38 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                 // bulk copy through shared memory occupies its stage for several microseconds)
                 const size_t side_lanes = kHybridStageBytes / (2 * (size_t)side_chunk);
                 const size_t side_smem = longs.empty() ? 0 : side_lanes * 2 * (size_t)side_chunk + side_lanes * 2 * 8;
+                // Launches that are not made of 16-byte units move as words (iso_gather_words) unless they are
+                // better off in units; those that are, move in units unless they are better off as words (below)
+                bool may_words = kernel == KERNEL_VEC && longs.empty() && r.knobs.words != 0;
+                if (may_words && r.knobs.words != 1) {
+                    LaunchShape s;
+                    bool used[ISO_MAX_DIMS] = {false};
+                    for (const Piece &q : cls) {
+                        s.bytes += q.p.len;
+                        s.units += q.p.len / q.width;
+                        if (q.p.src_buf == ISO_BUF_SEND) s.from_send += q.p.len;
+                        for (int j = 0; j < c.d; ++j) used[j] = used[j] || q.p.shift[j] || q.p.check[j];
+                        if (!q.first) continue;
+                        ++s.blocks;
+                        s.words += (q.block + 23) / 16;
+                        s.lanes += (16 - q.width + q.block + 15) / 16 + 1;
+                        s.longest = std::max(s.longest, q.block);
+                        s.shortest = std::min(s.shortest, q.block);
+                        if (q.block < 4) s.short_bytes += q.block;
+                        if (q.base < 16) ++s.moving;
+                        else if ((q.p.src_off - q.p.dst_off) & 15) ++s.apart;
+                    }
+                    for (int j = 0; j < c.d; ++j)
+                        if (used[j]) { ++s.n_used; s.torus = s.torus && c.periodic[j]; }
+                    if (width >= 8 || width == 0) may_words = !rows_do_not_group(r, width, s);
+                    if (width != 16) may_words = may_words && !better_in_units(r, width, s);
+                }
+                const bool narrow_words = may_words && width != 16;
                 // a vector launch holds at most kMaxVecUnits unit positions per process (each
                 // gets a descriptor): cut longer lists, splitting a piece at a unit boundary
                 if (kernel == KERNEL_VEC) {
                     // (a launch of words describes 16-byte words whatever the width of its pieces)
-                    const int64_t cap = width == 16 || !longs.empty() ? (int64_t)kMaxVecUnits : (int64_t)1 << 24;
+                    const int64_t cap = narrow_words ? (int64_t)1 << 24 : (int64_t)kMaxVecUnits;
                     std::vector<Piece> cut;
                     std::vector<size_t> bounds(1, 0);
                     int64_t used_units = 0;
@@ -1118,12 +1229,7 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                     {
                         bool torus = true;
                         for (int k = 0; k < L.n_used; ++k) torus = torus && c.periodic[L.used_dim[k]];
-                        // (launches of 4-byte blocks and nothing else stay with 4-byte units: a word would be a
-                        // 16-byte load for every 4 bytes, and those loads do not share sectors through the L1.
-                        // 256x256, 24 neighbours: 12.3 against 13.9 microseconds, one pass 7.6 against 8.9)
-                        bool tiny = width == 4;
-                        for (const LoweredPart &lp : L.parts) tiny = tiny && lp.p.len == 4;
-                        // Small launches of 16-byte units are also better off as words, in narrow CTAs of which
+                        // Small launches of 16-byte units are better off as words, in narrow CTAs of which
                         // several fit an SM: a CTA of 1024 threads fills its SM, so the next launch cannot even
                         // start before this one drains.  Measured per start, wide CTAs against words: 8^3 with 26
                         // 64-byte blocks 9.4 against 7.2 microseconds, 16^3 12.8 against 8.7 (2.4 MB per launch),
@@ -1132,7 +1238,9 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                         // rows longer than a CTA, 8x6x10 with 342 64-byte blocks 12.7 against 13.6.
                         // So are launches in which a block moves along three dimensions and more, whose scattered
                         // loads gain from warps that run independently of one another: allgathers (64-byte
-                        // blocks in one pass, 16^4 125 against 79 microseconds, 32^3 16.7 against 15.2), and
+                        // blocks in one pass, 16^4 125 against 79 microseconds, 32^3 16.7 against 15.2; in three dimensions not
+                        // short blocks of 100000 processes and more: 96 bytes to 26 neighbours on 71x61x66 162 against 185, 32
+                        // bytes to 25 on 37x67x59 32 against 42, but 128 bytes to 26 on 71x57x41 123 against 114), and
                         // all-to-alls from 96 MB of blocks of 64 bytes (64^3 184 against 150, 48^3 74.6 against
                         // 67.5; 32^3, 54 MB, 20.4 against 22.4; 32-byte blocks on 64^3 73.7 against 78.9) or in
                         // more dimensions (8^5 with 16-byte blocks 65 against 58), as long as a row fits a
@@ -1142,13 +1250,14 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                         for (const LoweredPart &lp : L.parts) min_len = std::min(min_len, lp.p.len);
                         for (int k = 0; k < L.n_used; ++k) mesh_launch = mesh_launch || !c.periodic[L.used_dim[k]];
                         const bool scattered = mesh_launch ||
-                                               (L.n_used >= 3 && (r.kind == ISO_KIND_ALLGATHER ||
-                                                                  ((int64_t)c.P * (int64_t)units * 16 >= kWordsScattered && units <= 1024 &&
+                                               (L.n_used >= 3 && ((r.kind == ISO_KIND_ALLGATHER && (L.n_used > 3 || c.P < 100000 || min_len >= 128)) ||
+                                                                  (r.kind != ISO_KIND_ALLGATHER && (int64_t)c.P * (int64_t)units * 16 >= kWordsScattered && units <= 1024 &&
                                                                    (L.n_used > 3 || min_len >= 64))));
-                        const bool small = width == 16 && (((int64_t)c.P * (int64_t)units * 16 <= kWordsSmallLaunch && units <= 1024) || scattered) &&
+                        const bool small = may_words && width == 16 &&
+                                           (((int64_t)c.P * (int64_t)units * 16 <= kWordsSmallLaunch && units <= 1024) || scattered || r.knobs.words == 1) &&
                                            !r.persistent && r.wave_request == 0 && r.knobs.vec_threads == 0;
-                        L.words = kernel == KERNEL_VEC && (width != 16 || small) && longs.empty() && !tiny;
-                        L.compact = kernel == KERNEL_VEC && !L.words && L.n_used > 3 && L.max_nnz < L.n_used &&
+                        L.words = narrow_words || small;
+                        L.compact = kernel == KERNEL_VEC && !L.words && (width >= 4 || width == 0) && L.n_used > 3 && L.max_nnz < L.n_used &&
                                     torus && !r.persistent;  // (the pipelined one-launch kernel does take compact launches)
                     }
                     // geometry
@@ -1170,7 +1279,7 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                         // (measured against four CTAs of 256 threads: 36.1 against 40.3 microseconds
                         // per all-to-all on the 32^3 torus, 161 against 184 on the 8^5 torus);
                         // ISO_VEC_THREADS=256 or 512 selects the narrower shapes
-                        uint32_t max_threads = width == 4 ? 256 : 1024;
+                        uint32_t max_threads = width == 16 || width == 0 ? 1024 : 256;
                         if (!longs.empty())  // leave a warp and the staging area to the bulk side
                             max_threads = std::min<uint32_t>((uint32_t)(1024 - side_lanes),
                                                              (uint32_t)((227 * 1024 - side_smem - 16 * 1024) / (kHybridDepth * 16) / 32 * 32));
@@ -1236,7 +1345,7 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                     L.smem = (size_t)L.n_used * (size_t)tp * sizeof(uint32_t);
                     if (kernel == KERNEL_VEC) {
                         const size_t depth = !longs.empty() ? kHybridDepth : (L.threads > 256 ? kWideDepth : kVecDepth);
-                        L.smem = L.words ? 0 : depth * L.threads * (width == 4 ? 4 : 16);
+                        L.smem = L.words || (width > 0 && width < 4) ? 0 : depth * L.threads * (size_t)(width ? width : 16);
                     }
                     if (kernel == KERNEL_BULK)
                         L.smem = (L.smem + 15) / 16 * 16 + (size_t)L.threads * 2 * (size_t)unit + (size_t)L.threads * 2 * 8;

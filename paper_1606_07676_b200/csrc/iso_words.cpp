@@ -367,7 +367,11 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     // of their own, which need no merging (and where everything is a multiple of 4 bytes, the few are
     // cheaper in smaller words: one-pass irregular 735 against 685); where they are many, they stay
     // with their neighbours (118-byte blocks, one merged word in eight: 88 against 134 microseconds).
-    const bool apart = merged * 12 < n_in_place, keep_partial = partial * 64 <= n_in_place;
+    // In one pass along three dimensions and more they stay with their neighbours further down: what is stored far from its
+    // sector-mates costs more in the L2 (120-byte blocks of 342 neighbours on 24x22x23 204 against 380, 232 bytes of 124 on 16x26x24
+    // 108 against 131, but 168 bytes of 8 along two dimensions on 525x492 147 against 127, irregular sizes on 64x64x32 705 against 679).
+    const size_t few = L.n_used < 3 ? 12 : (by8 ? 36 : 20);
+    const bool apart = merged * few < n_in_place, keep_partial = partial * 64 <= n_in_place;
     std::vector<uint32_t> plain, rest;  // of words16
     std::vector<Word> fine;
     std::vector<Run> fine_runs;

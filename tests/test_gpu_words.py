@@ -84,3 +84,33 @@ def test_many_rows_and_slabs(m):
 def test_coordinates_without_a_table(dims, offs, m):
     # launches whose table of coordinates does not fit beside the rings: every lane divides
     _compare(wl.Workload("w", "allgather", dims, offs, m, seed=m))
+
+
+@pytest.mark.parametrize("words", ["0", "1", None])
+@pytest.mark.parametrize("m", [1, 2, 8, 12, 24, 72, 100, 120, 504])
+def test_units_and_words(m, words, monkeypatch):
+    """The same calls in units, as words and as the library chooses: strides that are multiples of 16 bytes
+    (8 and 26 neighbours) and that are not (7 and 3), planes that divide into groups of rows and that do not."""
+    if words is not None:
+        monkeypatch.setenv("ISO_WORDS", words)
+    for call in ("alltoall", "allgather"):
+        for dims, offs in (((13, 11), wl.moore(2, 1)), ((12, 16), wl.positive_octant(2, 1)), ((5, 6, 7), wl.positive_octant(3, 1)),
+                           ((6, 5, 4), wl.moore(3, 1)), ((3, 4, 3, 5), wl.positive_octant(4, 1)), ((301,), wl.moore(1, 2))):
+            _compare(wl.Workload("w", call, dims, offs, m, seed=m), lead=(8, 8) if m % 8 == 0 and len(dims) == 2 else (0, 0))
+
+
+@pytest.mark.parametrize("words", ["0", "1", None])
+def test_units_and_words_mixed_sizes(words, monkeypatch):
+    # faces, edges and corners; sizes from 1 to 1024 bytes; launches long enough for the rules of the library
+    if words is not None:
+        monkeypatch.setenv("ISO_WORDS", words)
+    for r, side, dims in ((1, 9, (24, 35, 21)), (3, 7, (13, 11, 10)), (2, 12, (9, 10, 8))):
+        offs = wl.moore(3, r)
+        lens = np.asarray([side ** max(0, 3 - int(np.abs(v).sum())) for v in offs], np.int64)
+        _compare(wl.Workload("v", "alltoallv", dims, offs, 0, lens=lens, seed=r))
+    offs = wl.random_offsets(5, 3, 30, -3, 3)
+    _compare(wl.Workload("v", "alltoallv", (9, 8, 7), offs, 0, lens=wl.random_sizes(5, 30, choices=(1, 2, 4, 31, 256, 1024)), seed=3))
+    for call, dims, offs, m in (("alltoall", (120, 123), wl.positive_octant(2, 1), 120), ("allgather", (114, 102), wl.positive_octant(2, 3), 120),
+                                ("allgather", (258, 139), wl.moore(2, 1), 120), ("allgather", (35, 34, 33), wl.positive_octant(3, 3), 8),
+                                ("alltoall", (145571,), wl.moore(1, 1), 16), ("alltoall", (151916,), wl.moore(1, 1), 68), ("allgather", (89060,), wl.moore(1, 6), 24)):
+        _compare(wl.Workload("w", call, dims, offs, m, seed=m))
