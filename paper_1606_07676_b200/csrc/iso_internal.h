@@ -274,6 +274,7 @@ struct Request {
     unsigned long long wave_run = 0;  // starts since the counters were last zeroed
     int wave_counters = 0;      // counters allocated in d_counter
     bool lean_tables = false;   // word tables of one row each, where the room for tables is short
+    bool plain_units = false;   // no launches of words: every launch in units (Iso_neighbor_alltoall_static)
     bool hybrid = false;        // launches of mixed widths hand their long bodies to bulk warps (Iso_request_set_hybrid)
     int sender_side = 1;        // allgather phases in sender-side form: 0 never, 1 where measured faster, 2 wherever possible
     uint32_t wait_limit = 1u << 22;  // polls before a device-side wait on other CTAs gives up

@@ -1142,7 +1142,7 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                 const size_t side_smem = longs.empty() ? 0 : side_lanes * 2 * (size_t)side_chunk + side_lanes * 2 * 8;
                 // Launches that are not made of 16-byte units move as words (iso_gather_words) unless they are
                 // better off in units; those that are, move in units unless they are better off as words (below)
-                bool may_words = kernel == KERNEL_VEC && longs.empty() && r.knobs.words != 0;
+                bool may_words = kernel == KERNEL_VEC && longs.empty() && !r.plain_units && r.knobs.words != 0;
                 if (may_words && r.knobs.words != 1) {
                     LaunchShape s;
                     bool used[ISO_MAX_DIMS] = {false};

@@ -97,3 +97,21 @@ def test_static_entry_point_rejects_what_does_not_fit():
     assert "scratch" in iso.Iso_error_string(iso.ISO_ERR_TOO_LARGE)
     torch.cuda.synchronize()
     assert int(recv.min()) == 0x33 and int(recv.max()) == 0x33      # nothing was enqueued
+
+
+@pytest.mark.parametrize("m,s", [(8, 100001), (8, 65535), (1, 120001), (2, 65535), (1021, 1801)])
+def test_static_entry_point_takes_what_only_one_kind_of_table_fits(m, s):
+    """Unit tables need 64 bytes per unit; word tables need up to 128 bytes per short block, but less per
+    long one of an odd size: a problem is taken if either fits into the scratch area."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("needs a CUDA device")
+    torch.cuda.set_device(0)
+    P = 7  # one dimension: one hop per block and no intermediate storage, so that the tables alone have to fit
+    offs = (np.arange(s, dtype=np.int32) % P).reshape(s, 1)
+    send_h = wl.payload_np("uint8", s, 0, 0, P * s * m).reshape(P, s * m).copy()
+    send = torch.from_numpy(send_h).cuda()
+    got = torch.full((P, s * m), 0x5A, dtype=torch.uint8, device="cuda")
+    iso.Iso_neighbor_alltoall_static((P,), offs, send, got, m, iso.ISO_BYTE, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert np.array_equal(got.cpu().numpy(), oracle.alltoall((P,), offs, m, send_h))
