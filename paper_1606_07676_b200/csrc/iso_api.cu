@@ -905,6 +905,9 @@ void plan_slabs(const Request &r, std::vector<SlabPlan> &slabs, int want = 0)
     // slabs 216, in one 111; 3.8 MB in 32 slabs 426, in 3 210; 6.8 MB in 16 slabs 352, in 4 to 6 320).
     const int64_t bytes = c.P * std::max(r.send_stride, r.recv_stride);
     int n = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(p0, 32), bytes / kHostSlabBytes));
+    // Where Iso_Start runs slab by slab, at least as many: the intermediate buffer holds one slab of either, and
+    // larger slabs here would take back what the slabs there save.
+    n = std::max(n, (int)std::min<int64_t>(std::min(p0, 32), (int64_t)r.slab_plan.size()));
     if (want > 0) {
         n = std::min(p0, want);
     } else if (r.knobs.host_slabs >= 0) {

@@ -149,6 +149,78 @@ def test_random_cases(chunk):
         iso.Iso_comm_free(comm)
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("host_slabs", [2, 3, 5, 32])
+def test_random_cases_through_host_slabs(host_slabs, monkeypatch):
+    """The pipelined host-buffer path cuts small transfers into one slab, where the order of the uploads and the
+    windows of the slabs are trivial: here into several, with the device's slabs off, automatic and asked for."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("needs a CUDA device")
+    torch.cuda.set_device(0)
+    monkeypatch.setenv("ISO_HOST_SLABS", str(host_slabs))
+    piped = 0
+    for c in random_cases(100 + host_slabs, trials=60):
+        P, ss, rs = c["P"], c["ss"], c["rs"]
+        if not rs or not P * ss:
+            continue
+        send = torch.zeros((P, ss), dtype=torch.uint8, device="cuda")
+        recv = torch.full((P, rs), POISON, dtype=torch.uint8, device="cuda")
+        comm, req = make_request(c, send, recv)
+        want = expected(c)
+        hs = torch.from_numpy(c["send_h"]).pin_memory()
+        for (alg, fusion), (lay, _, bulk, slabs) in zip(c["choices"], c["options"]):
+            iso.Iso_request_set_layout(req, lay)
+            iso.Iso_request_set_slabs(req, slabs)
+            iso.Iso_request_set_bulk_threshold(req, bulk)
+            iso.Iso_request_set_algorithm(req, alg, fusion)
+            recv.fill_(POISON)
+            hr = torch.zeros((P, rs), dtype=torch.uint8).pin_memory()
+            torch.cuda.synchronize()
+            for _ in range(3):      # enqueued, captured, replayed
+                hr.zero_()
+                iso.Iso_Start_host(req, hs, hr)
+                iso.Iso_wait(req)
+                assert np.array_equal(hr.numpy(), want), dict(trial=c["trial"], dims=c["dims"], kind=c["kind"], alg=alg, fusion=fusion, slabs=slabs)
+            try:
+                used = iso.Iso_request_get_host_transfer_ms(req)["slabs"]
+            except iso.IsoError:    # not pipelined
+                continue
+            assert used == min(host_slabs, c["dims"][0])
+            piped += 1
+            assert iso.Iso_request_check_guards(req) == 0
+        iso.Iso_request_free(req)
+        iso.Iso_comm_free(comm)
+    assert piped >= 20
+
+
+@pytest.mark.gpu
+def test_device_slabs_keep_their_small_buffer():
+    """A request that asks for slabs has an intermediate buffer of one slab, also where the transfers of the host-buffer
+    path are small enough for one."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.fail("needs a CUDA device")
+    torch.cuda.set_device(0)
+    w = wl.Workload("w", "alltoall", (16, 4, 4, 4, 5), wl.moore(5, 1), 2, seed=5)     # 2.5 MB each way
+    send = wl.payload_torch("uint8", 5, 0, w.P * w.s * 2, "cuda").view(w.P, w.s * 2)
+    recv = torch.empty_like(send)
+    host_s = send.cpu().pin_memory()
+    host_r = torch.zeros_like(host_s).pin_memory()
+    comm = iso.Iso_neighborhood_create(w.dims, w.offsets)
+    req = iso.Iso_neighbor_alltoall_init(send, 2, 1, recv, 2, 1, comm)
+    iso.Iso_request_set_slabs(req, 8)
+    iso.Iso_Start_host(req, host_s, host_r)
+    iso.Iso_wait(req)
+    assert iso.Iso_request_get_execution(req)["slabs"] == 8
+    # one host slab would need room for the intermediate blocks of all processes, eight need what the device's need
+    assert iso.Iso_request_get_host_transfer_ms(req)["slabs"] == 8
+    assert iso.Iso_request_check_guards(req) == 0
+    assert np.array_equal(host_r.numpy(), oracle.alltoall(w.dims, w.offsets, 2, host_s.numpy()))
+    iso.Iso_request_free(req)
+    iso.Iso_comm_free(comm)
+
+
 @pytest.mark.parametrize("chunk", range(6))
 def test_random_cases_host_simulation(chunk):
     """The same random problems without a GPU: the exported parts are executed with numpy."""
