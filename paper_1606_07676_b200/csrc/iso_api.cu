@@ -52,7 +52,7 @@ void release_device(Request &r)
     if (r.d_err) cudaFree(r.d_err);
     for (void *st : r.host_streams) cudaStreamDestroy(static_cast<cudaStream_t>(st));
     r.host_streams.clear();
-    for (void *st : r.chain_streams) cudaStreamDestroy(static_cast<cudaStream_t>(st));
+    for (const Request::ChainStream &cs : r.chain_streams) cudaStreamDestroy(static_cast<cudaStream_t>(cs.stream));
     r.chain_streams.clear();
     for (void *e : r.chain_events) cudaEventDestroy(static_cast<cudaEvent_t>(e));
     r.chain_events.clear();
@@ -1838,12 +1838,22 @@ int Iso_Start(Iso_request request, void *cuda_stream)
         return ISO_SUCCESS;
     }
     if (r.slab_plan.size() > 1 && r.chains > 1) {
-        // two or more chains of slabs: the first on the caller's stream, the others beside it
+        // two or more chains of slabs: the first on the caller's stream, the others beside it on streams of the
+        // same priority
         std::vector<cudaStream_t> st(1, stream);
-        while (r.chain_streams.size() + 1 < (size_t)r.chains) {
-            cudaStream_t s;
-            ISO_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
-            r.chain_streams.push_back(s);
+        int priority = 0;
+        ISO_CUDA(cudaStreamGetPriority(stream, &priority));
+        for (int k = 1; k < r.chains; ++k) {
+            void *own = nullptr;
+            for (const Request::ChainStream &cs : r.chain_streams)
+                if (cs.chain == k && cs.priority == priority) own = cs.stream;
+            if (!own) {
+                cudaStream_t s;
+                ISO_CUDA(cudaStreamCreateWithPriority(&s, cudaStreamNonBlocking, priority));
+                own = s;
+                r.chain_streams.push_back(Request::ChainStream{k, priority, own});
+            }
+            st.push_back(static_cast<cudaStream_t>(own));
         }
         while (r.chain_events.size() < (size_t)r.chains) {
             cudaEvent_t e;
@@ -1852,10 +1862,7 @@ int Iso_Start(Iso_request request, void *cuda_stream)
         }
         auto event = [&](int k) { return static_cast<cudaEvent_t>(r.chain_events[k]); };
         ISO_CUDA(cudaEventRecord(event(0), stream));
-        for (int k = 1; k < r.chains; ++k) {
-            st.push_back(static_cast<cudaStream_t>(r.chain_streams[k - 1]));
-            ISO_CUDA(cudaStreamWaitEvent(st[k], event(0), 0));
-        }
+        for (int k = 1; k < r.chains; ++k) ISO_CUDA(cudaStreamWaitEvent(st[k], event(0), 0));
         int rc = enqueue_chains(r, st, use_pdl);
         // the caller's stream waits for the other chains whatever happened
         for (int k = 1; k < r.chains; ++k) {

@@ -261,7 +261,9 @@ struct Request {
     int chains_request = 0;     // slabs to run side by side, as asked for (0: the library chooses)
     bool graph_request = false; // graph replay, as asked for
     int chains = 1;             // slabs that run side by side (each on its share of the SMs)
-    std::vector<void *> chain_streams, chain_events;  // for chains outside a graph: all but the first, fork and joins
+    struct ChainStream { int chain, priority; void *stream; };
+    std::vector<ChainStream> chain_streams;  // for chains outside a graph: all but the first, by the priority of the caller's stream
+    std::vector<void *> chain_events;        // fork and joins
     bool use_graph = false;     // Iso_Start replays a captured graph of the launches
     void *graph_exec = nullptr; // cudaGraphExec_t, built at the first Iso_Start after a change
     // pipelined one-launch execution (items = slab x launch, per-item completion counters)
