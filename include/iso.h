@@ -273,9 +273,10 @@ int Iso_request_set_slabs(Iso_request request, int slabs);
  * the drain of one chain's short kernels are covered by the other chains.  The number of
  * slabs is rounded to a multiple of n; the launches are then replayed from a captured
  * graph (see Iso_request_set_graph).  1 turns it off; at most 8.  Until this is called the
- * library runs two chains (without a graph, on a second stream of its own beside the
- * caller's) where it chooses the slabs itself and there are four or more.  Ignored where
- * slab execution is (see there).  The result never depends on it.
+ * library runs two chains where it chooses the slabs itself and there are four or more: the
+ * first two starts launch by launch, on the caller's stream and a second one of the same
+ * priority, from the third on from a graph.  Ignored where slab execution is (see there).
+ * The result never depends on it.
  */
 int Iso_request_set_chains(Iso_request request, int chains);
 
@@ -286,7 +287,10 @@ int Iso_request_set_chains(Iso_request request, int chains);
  * submission per start instead of one per launch, which pays for schedules of many short
  * launches and costs a few microseconds on schedules of few long ones.  With `enable` == 0
  * (the default) the library replays from a graph only where a start has 128 launches or
- * more.  Ignored in single-launch mode.  The result never depends on it.
+ * more (such a start cannot be recorded into a graph of the caller's) or, from the third
+ * start on, where it runs two chains of its own choice (a start that is being recorded is
+ * then enqueued launch by launch).  Ignored in single-launch mode.  The result never
+ * depends on it.
  */
 int Iso_request_set_graph(Iso_request request, int enable);
 

@@ -272,6 +272,7 @@ int materialise(Request &r)
     // a captured graph holds the addresses of the tables and buffers that are replaced below
     if (r.graph_exec) cudaGraphExecDestroy(static_cast<cudaGraphExec_t>(r.graph_exec));
     r.graph_exec = nullptr;
+    r.plain_starts = 0;
     if (r.host_graph_exec) cudaGraphExecDestroy(static_cast<cudaGraphExec_t>(r.host_graph_exec));
     r.host_graph_exec = nullptr;
     r.host_last_hs = r.host_last_hr = nullptr;
@@ -1077,6 +1078,7 @@ void choose_slab_plan(Request &r)
     r.slab_plan.clear();
     r.inter_rows = c.P;
     r.chains = 1;
+    r.late_graph = false;
     r.use_graph = !r.persistent && r.graph_request;
     if (r.knobs.graph >= 0) r.use_graph = !r.persistent && r.knobs.graph != 0;
     if (r.wave_ok) {
@@ -1122,11 +1124,13 @@ void choose_slab_plan(Request &r)
     }
     // Left to the library, four slabs and more run as two chains of slabs half that size (as long as that
     // leaves 512 processes to a slab): the ramp and the drain of one chain's launches are covered by the
-    // other.  Measured in microseconds per start: 2 KB blocks on 256x256 1546 -> 1417, 512 bytes 374 ->
-    // 358, 48^3 with 26 blocks of 128 bytes 247 -> 228, Moore r=3 542 -> 530, 16^4 283 -> 280, irregular
-    // 64x64x32 1389 -> 1324 (from a graph another 2 % faster, but the first start then takes up to 6 ms
-    // longer); two slabs made four (8^5 torus) lost, 155 -> 162, as did two chains without halving the
-    // slabs (shells, one plane of dimension 0 each: 2.65 -> 2.75 ms).
+    // other.  Measured in turn in microseconds per start, one chain, two, two from a graph (and the host's time for a
+    // start): irregular 64x64x32 1411, 1328, 1327 (251, 494, 5); 2 KB blocks on 256x256 1578, 1414, 1463 (4.5 from its graph, 670,
+    // 5); 512 bytes 370, 351, 337 (82, 165, 4.5); 48^3 with 26 blocks of 128 bytes 235, 226, 221; Moore r=3 551, 532, 515; 16^4
+    // 282, 286, 277.  So from a graph, but as its capture takes the host a millisecond, only from the third start on.  Two slabs
+    // made four (8^5 torus) lost, 155 -> 162, as did two chains without halving the slabs (shells, one plane of
+    // dimension 0 each: 2.65 -> 2.75 ms) and slabs of 256 processes (2 KB blocks 1413 -> 1661; 4 KB blocks, the same within
+    // what runs differ by, 3.04 to 3.10 ms in 128 or 256 slabs, one or two chains).
     const bool two = r.chains_request == 0 && r.knobs.chains < 0 && r.slab_request == 0 && r.knobs.slabs < 0 && want >= 4 &&
                      want * 2 <= c.dims[0] && c.P / (want * 2) >= 512;
     if (two) want *= 2;
@@ -1146,6 +1150,7 @@ void choose_slab_plan(Request &r)
         // slabs side by side: every chain has its own one-slab part of the intermediate buffer
         r.chains = chains;
         if (!two) r.use_graph = true;
+        else r.late_graph = r.knobs.graph != 0;
         rows *= chains;
     }
     // a start of very many launches is replayed from a graph unless the environment says otherwise
@@ -1502,7 +1507,7 @@ int Iso_request_get_execution(Iso_request request, int *slabs, int *chains, int 
     const Request &r = *request;
     if (slabs) *slabs = r.dirty ? r.slab_request : (int)std::max<size_t>(1, r.slab_plan.size());
     if (chains) *chains = r.dirty ? std::max(1, r.chains_request) : r.chains;
-    if (graph) *graph = r.dirty ? (r.graph_request ? 1 : 0) : (r.use_graph ? 1 : 0);
+    if (graph) *graph = r.dirty ? (r.graph_request ? 1 : 0) : (r.use_graph || r.graph_exec ? 1 : 0);
     return ISO_SUCCESS;
 }
 
@@ -1826,7 +1831,15 @@ int Iso_Start(Iso_request request, void *cuda_stream)
         r.started = true;
         return ISO_SUCCESS;
     }
-    if (r.use_graph) {
+    bool replay = r.use_graph;
+    if (r.late_graph && r.plain_starts >= 2) {
+        // (a graph cannot be launched into a capture; the launches themselves can be recorded)
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        replay = cudaStreamIsCapturing(stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+        if (replay && !r.graph_exec && build_graph(r, use_pdl) != ISO_SUCCESS) replay = r.late_graph = false;
+        if (!replay) (void)cudaGetLastError();
+    }
+    if (replay) {
         // replay of the captured launches (chains of slabs side by side when asked for)
         if (!r.graph_exec) {
             int rc = build_graph(r, use_pdl);
@@ -1870,6 +1883,7 @@ int Iso_Start(Iso_request request, void *cuda_stream)
             ISO_CUDA(cudaStreamWaitEvent(stream, event(k), 0));
         }
         if (rc != ISO_SUCCESS) return rc;
+        if (r.plain_starts < 2) ++r.plain_starts;
         r.last_stream = cuda_stream;
         r.started = true;
         return ISO_SUCCESS;

@@ -265,6 +265,8 @@ struct Request {
     std::vector<ChainStream> chain_streams;  // for chains outside a graph: all but the first, by the priority of the caller's stream
     std::vector<void *> chain_events;        // fork and joins
     bool use_graph = false;     // Iso_Start replays a captured graph of the launches
+    bool late_graph = false;    // likewise, but only from the third start on
+    int plain_starts = 0;       // starts so far whose launches were enqueued one by one
     void *graph_exec = nullptr; // cudaGraphExec_t, built at the first Iso_Start after a change
     // pipelined one-launch execution (items = slab x launch, per-item completion counters)
     int wave_request = 0;       // 0: off, 1: one slab, n >= 2: n slabs of dimension 0

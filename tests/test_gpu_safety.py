@@ -131,6 +131,52 @@ def test_no_schedule_writes_outside_its_buffers(torch_cuda, name):
         iso.Iso_comm_free(comm)
 
 
+def test_chains_by_default(torch_cuda):
+    """A request whose slabs are left to the library and that has four or more runs them as two chains: the first
+    starts launch by launch on the caller's stream and one beside it, the later ones from a graph.  Starts follow one
+    another without a wait, on streams of either priority, each with its own contents; and a start can be recorded
+    into a caller's own graph, before and after the library has one."""
+    torch = torch_cuda
+    w = wl.Workload("w", "alltoall", (128, 64), wl.moore(2, 2), 1024, seed=31)
+    n = w.P * w.s * 1024
+    send_whole, send = _banded(torch, n, 0)
+    recv_whole, recv = _banded(torch, n, POISON)
+    contents = [wl.payload_torch("uint8", k, 0, n, "cuda") for k in range(2)]
+    want = [torch.from_numpy(oracle_result(w, c.cpu().numpy().reshape(w.P, -1)).reshape(-1)).cuda() for c in contents]
+    comm, req = make_request(w, send, recv)
+    try:
+        torch.cuda.synchronize()
+        for k, priority in enumerate((0, -1, 0, -1, -1, 0)):
+            stream = torch.cuda.Stream(priority=priority)
+            with torch.cuda.stream(stream):
+                results = []
+                for j in range(2):
+                    send.copy_(contents[(k + j) % 2])
+                    recv.fill_(POISON)
+                    iso.Iso_Start(req, stream)
+                    results.append(recv.clone())
+            stream.synchronize()
+            for j in range(2):
+                assert torch.equal(results[j], want[(k + j) % 2]), (k, j)
+            ex = iso.Iso_request_get_execution(req)
+            assert ex["slabs"] >= 8 and ex["chains"] == 2 and ex["graph"] == (0 if k == 0 else 1), ex
+            if k in (0, 2):
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph):
+                    iso.Iso_Start(req, torch.cuda.current_stream())
+                send.copy_(contents[1])
+                recv.fill_(POISON)
+                graph.replay()
+                torch.cuda.synchronize()
+                assert torch.equal(recv, want[1])
+                del graph
+            assert iso.Iso_request_check_guards(req) == 0
+            assert _bands_intact(send_whole, n) and _bands_intact(recv_whole, n)
+    finally:
+        iso.Iso_request_free(req)
+        iso.Iso_comm_free(comm)
+
+
 def test_plain_c_program_runs_a_collective_on_the_device(torch_cuda, tmp_path):
     """tests/c_abi_gpu.c: cudaMalloc'd buffers, Iso_Start and Iso_wait from C, compared with
     the hand-worked rows of the 4x4 example."""
