@@ -1631,35 +1631,39 @@ int Iso_request_tune(Iso_request request, void *cuda_stream, int flags)
         if (!any || rc != ISO_SUCCESS) continue;
     }
     std::vector<Choice> tried;
+    auto consider = [&](const Choice &c) {
+        if (r.started) rc = Iso_wait(request);
+        if (rc == ISO_SUCCESS) rc = apply(c);
+        if (rc == ISO_SUCCESS) rc = materialise(r);
+        if (rc != ISO_SUCCESS) return;
+        // what the schedule allowed may differ from what was asked for: skip repeats
+        const Choice got{(int)std::max<size_t>(1, r.slab_plan.size()), r.chains, r.use_graph ? 1 : 0, r.alg, r.fusion, hybrid, sched.order};
+        for (const Choice &t : tried)
+            if (t.slabs == got.slabs && t.chains == got.chains && t.graph == got.graph) return;
+        if (c.slabs > 0) tried.push_back(got);  // (a plan of the library's own may use other kernels)
+        float ms = 0.0f;
+        rc = measure(3, ms);  // a first look, then the real measurement scaled to it
+        if (rc != ISO_SUCCESS) return;
+        const int reps = (int)std::max(5.0f, std::min(200.0f, 2.0f / std::max(ms, 1e-3f)));
+        rc = measure(reps, ms);
+        if (rc != ISO_SUCCESS) return;
+        if (log)
+            std::fprintf(stderr, "iso tune: alg %d fusion %d order %d hybrid %d slabs %d chains %d graph %d: %.4f ms\n", got.alg, got.fusion,
+                         got.order, got.hybrid, got.slabs, got.chains, got.graph, ms);
+        // the plainer plans come first; a later one must win by 2 % to replace them
+        if (best_ms < 0.0f || ms < 0.98f * best_ms) {
+            best_ms = ms;
+            best = c;
+        }
+    };
+    // (the plan the library would choose for the schedule, as the request came with it unless it was told otherwise)
+    if (!hybrid) consider(Choice{0, 0, 0, sched.first, sched.second, 0, sched.order});
     for (int graph = 0; graph <= 1 && rc == ISO_SUCCESS; ++graph)
         for (int chains = 1; chains <= 4 && rc == ISO_SUCCESS; chains *= 2) {
-            if (chains > 1 && !graph) continue;  // chains only exist inside a graph
+            if (chains > 1 && !graph) continue;  // chains that are asked for run from a graph in any case
             for (int slabs = 1; slabs <= 64 && slabs <= std::max(1, p0) && rc == ISO_SUCCESS; slabs *= 2) {
                 if (chains > 1 && slabs < chains) continue;
-                if (r.started) rc = Iso_wait(request);
-                if (rc == ISO_SUCCESS) rc = apply(Choice{slabs, chains, graph, sched.first, sched.second, hybrid, sched.order});
-                if (rc == ISO_SUCCESS) rc = materialise(r);
-                if (rc != ISO_SUCCESS) break;
-                // what the schedule allowed may differ from what was asked for: skip repeats
-                const Choice got{(int)std::max<size_t>(1, r.slab_plan.size()), r.chains, r.use_graph ? 1 : 0, r.alg, r.fusion, hybrid, sched.order};
-                bool seen = false;
-                for (const Choice &c : tried) seen = seen || (c.slabs == got.slabs && c.chains == got.chains && c.graph == got.graph);
-                if (seen) continue;
-                tried.push_back(got);
-                float ms = 0.0f;
-                rc = measure(3, ms);  // a first look, then the real measurement scaled to it
-                if (rc != ISO_SUCCESS) break;
-                const int reps = (int)std::max(5.0f, std::min(200.0f, 2.0f / std::max(ms, 1e-3f)));
-                rc = measure(reps, ms);
-                if (rc != ISO_SUCCESS) break;
-                if (log)
-                    std::fprintf(stderr, "iso tune: alg %d fusion %d order %d hybrid %d slabs %d chains %d graph %d: %.4f ms\n", got.alg,
-                                 got.fusion, got.order, got.hybrid, got.slabs, got.chains, got.graph, ms);
-                // the plainer plans come first; a later one must win by 2 % to replace them
-                if (best_ms < 0.0f || ms < 0.98f * best_ms) {
-                    best_ms = ms;
-                    best = Choice{slabs, chains, graph, sched.first, sched.second, hybrid, sched.order};
-                }
+                consider(Choice{slabs, chains, graph, sched.first, sched.second, hybrid, sched.order});
             }
         }
     }
