@@ -359,7 +359,8 @@ class Bound:
             iso.Iso_request_set_bulk_threshold(self.req, Bound.bulk_threshold)
         ex = execution or {"slabs": Bound.slabs, "chains": Bound.chains, "graph": Bound.graph}
         iso.Iso_request_set_slabs(self.req, ex["slabs"] if ex["slabs"] is not None else 0)
-        iso.Iso_request_set_chains(self.req, ex["chains"] if ex["chains"] is not None else 1)
+        if ex["chains"] is not None:      # (else the library's choice, as for a caller that says nothing)
+            iso.Iso_request_set_chains(self.req, ex["chains"])
         iso.Iso_request_set_graph(self.req, bool(ex["graph"]))
         iso.Iso_request_set_pipeline(self.req, Bound.pipeline or 0)
         stream = self.torch.cuda.current_stream()
