@@ -511,6 +511,8 @@ LaunchDev make_launch_args(const Request &r, const LaunchPlan &L)
     // against 393 microseconds, shells in 32 slabs 2.63 against 2.84 ms, Moore r=3 in 16 slabs 540
     // against 547; with few slabs the kept lines crowd out the streamed ones: 8 slabs (16^4 torus)
     // 284 against 281, 2 slabs (8^5 torus) 158 against 155, no slabs (32^3 torus) 38.6 against 37.1.
+    // Counted over both chains where there are two: 16 slabs in two chains, 48^3 with 128-byte blocks 226 against 234,
+    // 18x20x20x20 with 32-byte blocks 223 against 235, 16^4 286 against 285.
     a.keep_inter = (r.knobs.l2_keep && r.slab_plan.size() >= 16) ? 1u : 0u;
     a.reverse = (uint32_t)(L.phase & 1);
     a.n_used = L.n_used;
@@ -712,8 +714,15 @@ cudaError_t launch_hybrid(Kernel kernel, const LaunchPlan &L, const LaunchDev &a
 template <int W, int NU, bool MESH, bool COMPACT>
 cudaError_t launch_rows_wide(bool tab, const LaunchPlan &L, const LaunchDev &a, cudaStream_t stream, bool dependent)
 {
-    if constexpr (W == 16 && !MESH && !COMPACT && NU >= 1 && NU <= 2) {
-        if (tab && a.keep_inter) return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, true, true>, L, a, stream, dependent, table_bytes(a));
+    // (the L2 policy in every shape of launch: 80 blocks of 256 bytes in two phases on 32x16x12x12, three dimensions
+    // shifted in the first, 830 microseconds without and 808 with it; 242 of 32 bytes on 20x8x8x8x8 423 and 398)
+    if constexpr (W == 16 && !MESH) {
+        if (a.keep_inter) {
+            if constexpr (COMPACT || NU <= 2) {
+                if (tab) return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, true, true>, L, a, stream, dependent, table_bytes(a));
+            }
+            return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, false, true>, L, a, stream, dependent, 0);
+        }
     }
     if constexpr (!MESH && (COMPACT || NU <= 2)) {
         if (tab) return launch_wide(iso_gather_rows_wide<W, kWideDepth, NU, MESH, COMPACT, true>, L, a, stream, dependent, table_bytes(a));

@@ -696,3 +696,19 @@ def test_host_buffers_pipelined_over_slabs(torch_cuda, name):
     finally:
         run.close()
 
+
+
+@pytest.mark.parametrize("table", ["1", "0"])
+def test_eviction_hint_in_every_shape_of_launch(torch_cuda, monkeypatch, table):
+    """With 16 slabs and more the stores into the intermediate buffer carry an L2 policy: launches that shift along
+    one to four dimensions, with and without a table of coordinates, with rows longer than a CTA."""
+    monkeypatch.setenv("ISO_COORD_TABLE", table)
+    for dims, offs, m in (((32, 3, 4, 3), wl.moore(4, 1), 256), ((16, 5, 4, 3, 3), wl.moore(5, 1), 80), ((32, 5, 6), wl.moore(3, 3), 64)):
+        run = Run(torch_cuda, wl.Workload("w", "alltoall", dims, offs, m, seed=m))
+        want = oracle_result(run.w, run.send_host)
+        iso.Iso_request_set_slabs(run.req, 16)
+        for fusion in range(1, len(dims)):
+            assert np.array_equal(run.result(iso.ISO_ALG_COMBINING, fusion), want), (dims, fusion)
+            assert iso.Iso_request_get_execution(run.req)["slabs"] == 16
+            assert iso.Iso_request_check_guards(run.req) == 0
+        run.close()
