@@ -1093,7 +1093,7 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
             L.uniform_units = uniform ? L.parts[0].units : 0;
             for (int j = 0; j < c.d; ++j)
                 if (used[j]) L.used_dim[L.n_used++] = j;
-            if (!uniform) {
+            if (!uniform && kernel == KERNEL_BULK) {  // (the vector kernels have a descriptor per unit or word)
                 int shift = 0;
                 while ((units >> shift) + 1 > 16384) ++shift;
                 L.lookup_shift = shift;

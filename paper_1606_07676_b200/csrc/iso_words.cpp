@@ -168,24 +168,31 @@ struct FineChunks {
         const uint32_t *place = places.data();
         for (uint32_t k = 0; k < n_words; ++k) {
             const Word &w = words[k];
-            FineDev f{};
-            TinyDev t{};
-            uint32_t mask[2] = {0, 0}, byte[4] = {0, 0, 0, 0};
-            for (uint32_t j = 0; j < w.n; ++j, ++place) {
-                const Run &q = runs[w.first + j];
-                for (int e = q.begin; e < q.begin + q.n && e < 4; ++e) {
-                    byte[e] = *place + (uint32_t)e;
-                    t.mask |= 1u << e;
-                    if (j < 2) mask[j] |= 1u << e;
+            const uint32_t off = (uint32_t)((w.at - words[0].at) >> 2);
+            if (tiny) {
+                TinyDev t{};
+                uint32_t byte[4] = {0, 0, 0, 0};
+                for (uint32_t j = 0; j < w.n; ++j, ++place) {
+                    const Run &q = runs[w.first + j];
+                    for (int e = q.begin; e < q.begin + q.n; ++e) {
+                        byte[e] = *place + (uint32_t)e;
+                        t.mask |= 1u << e;
+                    }
                 }
-                if (j < 2) f.a |= *place << (15 * j);
+                t.a = byte[0] | byte[1] << 15;
+                t.b = byte[2] | byte[3] << 15;
+                t.off = off;
+                T.tiny.push_back(t);
+            } else {
+                FineDev f{};
+                f.b = off;
+                for (uint32_t j = 0; j < w.n; ++j, ++place) {  // one or two blocks
+                    const Run &q = runs[w.first + j];
+                    f.a |= *place << (15 * j);
+                    f.b |= ((((1u << q.n) - 1u) << q.begin) & 15u) << (16 + 4 * j);
+                }
+                T.fine.push_back(f);
             }
-            t.a = byte[0] | byte[1] << 15;
-            t.b = byte[2] | byte[3] << 15;
-            t.off = (uint32_t)((w.at - words[0].at) / 4);
-            f.b = t.off | mask[0] << 16 | mask[1] << 20;
-            if (tiny) T.tiny.push_back(t);
-            else T.fine.push_back(f);
         }
         T.fine.resize((T.fine.size() + 31) / 32 * 32, FineDev{});
         T.tiny.resize((T.tiny.size() + 31) / 32 * 32, TinyDev{});
@@ -212,7 +219,9 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     for (int k = 0; k < L.n_used; ++k) used_index[L.used_dim[k]] = k;
 
     const std::vector<Block> blocks = merged_blocks(L, c.d);
-    auto at16 = [&](int buf) { return stride[buf] % 16 == 0 && addr[buf] == 0; };  // the same places inside a word for all rows
+    bool same_places[3];  // inside a word for all rows
+    for (int k = 0; k < 3; ++k) same_places[k] = stride[k] % 16 == 0 && addr[k] == 0;
+    auto at16 = [&](int buf) { return same_places[buf]; };
     bool fixed = true, dst_fixed = true;  // all buffers, all destinations are like that
     bool by4 = true, by8 = true;   // every address is a multiple of 4, of 8
     int64_t rows = 1, bytes = 0, words = 0, moving = 0, moving_bytes = 0;  // moving: blocks that are not, on either side
@@ -321,8 +330,9 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     // everything is a multiple of 8, of 8 bytes.
     std::vector<Run> runs;
     std::vector<Word> words16;
-    runs.reserve((size_t)(rows * words * 2));
-    words16.reserve((size_t)(rows * words * 2));
+    runs.reserve((size_t)(rows * (words + 2 * (int64_t)blocks.size())));
+    words16.reserve((size_t)(rows * words));
+    T.loads.reserve((size_t)(rows * words / 32 * 35 + 64));  // a few lanes of a chunk stay idle
     size_t n_in_place = 0, merged = 0, partial = 0;
     auto finish = [&]() {  // the last of words16 has all its runs
         if (words16.empty() || words16.back().n) return;
@@ -348,7 +358,7 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
             for (size_t k = lo; k < hi; ++k) {
                 const int64_t at = (int64_t)sub * stride[buf] + addr[buf] + blocks[k].dst_off, last = at + blocks[k].len;
                 for (int64_t p = at; p < last;) {
-                    const int64_t w = p / 16 * 16, end = std::min(w + 16, last);
+                    const int64_t w = p & ~(int64_t)15, end = std::min(w + 16, last);
                     if (words16.empty() || words16.back().buf != buf || words16.back().at != w) {
                         finish();
                         words16.push_back(Word{w, (uint32_t)runs.size(), 0, (uint8_t)buf, false, false});
@@ -390,7 +400,7 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
         for (uint32_t j = w.first; j < w.first + w.n; ++j) {
             const Run &q = runs[j];
             for (int at = q.begin; at < q.begin + q.n;) {
-                const int start = (int)(at / grain * grain), end = std::min(start + (int)grain, q.begin + q.n);
+                const int start = at & ~((int)grain - 1), end = std::min(start + (int)grain, q.begin + q.n);
                 if (fine.empty() || fine.back().buf != w.buf || fine.back().at != w.at + start)
                     fine.push_back(Word{w.at + start, (uint32_t)fine_runs.size(), 0, w.buf, false, false});
                 ++fine.back().n;
@@ -446,8 +456,8 @@ void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t
     for (size_t i = 0; i < blocks.size(); ++i) places[i] = placement(addr[blocks[i].src_buf] + blocks[i].src_off, stride[blocks[i].src_buf]);
     auto range = [&](const Run &q, int64_t &k0, int64_t &k1) -> int64_t {
         const Placement &pl = places[q.block];
-        k0 = (pl.lowest + q.x) / 16;
-        k1 = (pl.highest + q.x + q.n - 1) / 16;
+        k0 = (pl.lowest + q.x) >> 4;
+        k1 = (pl.highest + q.x + q.n - 1) >> 4;
         return at16(blocks[q.block].src_buf) ? pl.lowest : 0;  // (where it varies the kernel adds the row's own place)
     };
     auto load = [&](const Run &q, int64_t k) {
