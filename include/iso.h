@@ -17,7 +17,11 @@
  *     regular all-to-all : s * count * size            (s blocks back to back, Section II)
  *     allgather          : count * size   (send side), s * count * size (receive side)
  *     irregular          : max_i(displ_i + count_i * size), rounded up to a multiple of 16
- * `Iso_request_get_stats` reports the strides in use.
+ * `Iso_request_get_stats` reports the strides in use.  Buffers may start at any byte.  The
+ * kernels store exactly the bytes of the blocks; they may LOAD the whole aligned 16-byte
+ * word that holds a block's first or last byte, so up to 15 bytes in front of and behind a
+ * send or receive buffer are read (never leaving its page) and dropped - a memory checker
+ * may report that.
  *
  * Result (Section II).  With C^i the i-th relative coordinate vector and (-) the
  * component-wise subtraction modulo p_j, after `Iso_Start` + `Iso_wait`
@@ -260,8 +264,8 @@ int Iso_request_set_pipeline(Iso_request request, int slabs);
  * intermediate blocks are then read back while still in the L2 cache, and the intermediate
  * buffer only holds one slab and is reused, so its lines are overwritten in cache instead of
  * being written to device memory.  `slabs` = 0 (default) lets the library choose (vector
- * launches only, and only when a slab's launch still lasts about 12 microseconds), 1 turns
- * it off, n >= 2 asks for n slabs (at most the size of dimension 0; ignored when the
+ * launches only: the fewest slabs that bring the bytes a launch writes under 52 MB, as long
+ * as the grid keeps half a dozen rows for every one it holds at a time), 1 turns it off, n >= 2 asks for n slabs (at most the size of dimension 0; ignored when the
  * schedule does not allow it or in single-launch mode).  The result never depends on it.
  */
 int Iso_request_set_slabs(Iso_request request, int slabs);
@@ -297,7 +301,7 @@ int Iso_request_set_graph(Iso_request request, int enable);
 /*
  * Measures instead of guessing (no counterpart in the paper; in the spirit of its
  * persistent requests, which are set up once and started many times): runs the request
- * with 1, 2, 4, ... slabs, with 1, 2 and 4 chains, with and without graph replay (and, for
+ * with the plan the library would choose, with 1, 2, 4, ... slabs, with 1, 2 and 4 chains, with and without graph replay (and, for
  * ragged rows, with and without the bulk warps of Iso_request_set_hybrid), timing a
  * few starts of each on `cuda_stream` with events, and leaves the request on the fastest
  * combination (a less plain plan has to win by 2 %).  `flags` is a sum of ISO_TUNE_* values.

@@ -240,6 +240,16 @@ void plan_words(const Request &r, LaunchPlan &L, uintptr_t inter_addr)
     L.grid = std::max<long long>(1, (warps * 32 + L.threads - 1) / L.threads);
     L.grid = std::min<long long>(L.grid, (long long)r.sm_count * (kWordsThreads / L.threads));
     L.grid = std::max<long long>(L.grid, (entries * 32 + L.threads - 1) / L.threads);  // every entry has a warp
+    // Where the coordinate table does not fit, kernels for one to four dimensions: that for any number took 577 instead of 315
+    // microseconds for 342 stencil blocks in one pass on 43x44x41, 267 instead of 195 for an allgather of 96 bytes from 26
+    // neighbours on 71x61x66, 201 instead of 180 for 128 bytes of 7 on 128x128x32.  All-to-alls along three dimensions with longer
+    // rows that are copies nearly throughout (no chunk has more warps than another) keep it, for a reason that is not
+    // known: 60x60x36 with 30 irregular blocks 608 against 681, 64^3 with 26 blocks of 64 bytes 151 against 172, 12 of 160 bytes 187
+    // against 219, 26 of 128 bytes 312 against 330.
+    int64_t bytes = 0;
+    for (const LoweredPart &lp : L.parts) bytes += lp.p.len;
+    L.any_dims = L.tables.form == 0 && L.n_used == 3 && r.kind != ISO_KIND_ALLGATHER && bytes >= 1500 &&
+                 L.tables.entries.size() == L.tables.chunks.size();
     const int depth = L.tables.form == 0 ? kWordsDepth : kWordsDepthCoded;
     L.smem = kWordsPadFront + (size_t)depth * L.threads * 16 + kWordsPadBack;
 }
@@ -745,8 +755,9 @@ cudaError_t launch_words_nu(const LaunchPlan &L, LaunchDev &a, cudaStream_t stre
         a.tab_slots = (uint32_t)per_cta;
         return launch_wide(iso_gather_words<FORM, MESH, NU, true>, L, a, stream, dependent, table);
     }
-    // (NU as with the table: the kernel for any number of dimensions took 578 instead of 310 microseconds for 342 stencil
-    // blocks in one pass on 43x44x41, 254 instead of 185 for an allgather of 96 bytes from 26 neighbours on 71x61x66)
+    if constexpr (FORM == 0 && NU == 3) {
+        if (L.any_dims) return launch_wide(iso_gather_words<FORM, MESH, ISO_MAX_DIMS, false>, L, a, stream, dependent, 0);
+    }
     return launch_wide(iso_gather_words<FORM, MESH, NU, false>, L, a, stream, dependent, 0);
 }
 

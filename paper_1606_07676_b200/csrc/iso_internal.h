@@ -178,6 +178,7 @@ struct LaunchPlan {
                                    // run by one extra warp of the same CTAs
     bool words = false;           // vector launch whose blocks are not whole, equally placed 16-byte units
     WordTables tables;            // its tables (build_words)
+    bool any_dims = false;        // without a coordinate table: the kernel for any number of dimensions
     std::vector<FanParent> fans;  // KERNEL_FAN: the launch as parents and their destinations (parts: the same copies, one per destination)
     // byte offsets of this launch's tables inside the request's device blob
     size_t parts_off = 0, lookup_off = 0, units_off = 0, fine_off = 0, tiny_off = 0, entries_off = 0;

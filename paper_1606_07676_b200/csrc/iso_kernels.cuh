@@ -545,8 +545,8 @@ __global__ void __launch_bounds__(1024, 1) iso_fan_rows(const __grid_constant__ 
         unsigned char *const B2 = L.buf[db2] + dt2, *const B3 = L.buf[db3] + dt3;
         const long long s0 = L.buf_stride[db0], s1 = L.buf_stride[db1], s2 = L.buf_stride[db2], s3 = L.buf_stride[db3];
         // Every other phase goes through the rows backwards: it then begins with the parent blocks that the
-        // phase before it has just written, while they are still in the L2 (80 neighbours on 16^4: 96.8 ->
-        // 94.0 microseconds per start).
+        // phase before it has just written, while they are still in the L2 (80 neighbours on 16^4: 96.5 ->
+        // 92.6 microseconds per start).
         const bool reverse = L.reverse != 0;
         const long long mirror = L.row_lo + L.row_hi - 1;
         const long long src_step = (reverse ? -rstep : rstep) * stride_s;

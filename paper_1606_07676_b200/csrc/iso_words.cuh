@@ -4,7 +4,8 @@
 //
 // Such data used to move in units of the widest power of two that divides every offset: 4-byte
 // units for a block of 12 bytes, 1-byte units for one of 13, each a load and a store of its own,
-// which bounds the kernel by load/store instructions.  Here
+// which bounds the kernel by load/store instructions.  (Some still do, where that is the faster way:
+// better_in_units in iso_schedule.cpp.)  Here
 //   * a lane LOADS one aligned 16-byte word of a source row (cp.async into a ring of slots, as in
 //     the aligned kernel), whatever part of the word its block needs;
 //   * where every byte of a destination word has the same place in the words it comes from, a lane
@@ -25,7 +26,8 @@
 //   2  anything else, long blocks: a group of lanes per block, both alignments worked out per row;
 //      16-byte stores, only the first and the last word of a block in part.
 // An aligned word that holds one byte of a buffer never leaves the buffer's page, so words are
-// loaded whole at the ends of a buffer too; what is stored is exact to the byte.
+// loaded whole at the ends of a buffer too (iso.h says so: up to 15 bytes on either side are read and
+// dropped); what is stored is exact to the byte.
 #pragma once
 
 #include "iso_kernels.cuh"
@@ -108,8 +110,8 @@ __device__ __forceinline__ uint4 byte_masks(uint32_t m)
 // A warp works on two rows at a time: what it waits for, beside device memory, is its own chain of
 // shared-memory reads, shuffles and stores, and two rows are two such chains.  For the registers that
 // takes, a CTA has 24 warps instead of 32; the ring holds sixteen words per lane, so that the bytes in
-// flight per SM stay those of the aligned kernel (twelve: one-pass irregular 687 instead of 621
-// microseconds).
+// flight per SM stay those of the aligned kernel (with eight or twelve instead, one-pass irregular
+// sizes on 64x64x32 677 and 687 against 683 microseconds, 64^3 with 64-byte blocks 171 in all three).
 template <int FORM, bool MESH, int NU, bool TAB>
 __global__ void __launch_bounds__(kWordsThreads, 1) iso_gather_words(const __grid_constant__ LaunchDev L)
 {
