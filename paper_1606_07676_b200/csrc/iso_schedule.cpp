@@ -1239,8 +1239,10 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                         // So are launches in which a block moves along three dimensions and more, whose scattered
                         // loads gain from warps that run independently of one another: allgathers (64-byte
                         // blocks in one pass, 16^4 125 against 79 microseconds, 32^3 16.7 against 15.2; in three dimensions not
-                        // short blocks of 100000 processes and more: 96 bytes to 26 neighbours on 71x61x66 162 against 185, 32
-                        // bytes to 25 on 37x67x59 32 against 42, but 128 bytes to 26 on 71x57x41 123 against 114), and
+                        // short rows of short blocks of 100000 processes and more: 96 bytes to 26 neighbours on 71x61x66 162 against
+                        // 185, 32 bytes to 25 on 37x67x59 32 against 42, but 128 bytes to 26 on 71x57x41 123 against 114 and 48
+                        // bytes to 342 on 48^3 650 against 541; nor rows of 1400 units and more from 1 GB on: 1396 neighbours on 32^3
+                        // 599 against 712, 192 bytes to 124 on 40^3 330 against 358, but 256 bytes to 342 on 20^3 154 against 149), and
                         // all-to-alls from 96 MB of blocks of 64 bytes (64^3 184 against 150, 48^3 74.6 against
                         // 67.5; 32^3, 54 MB, 20.4 against 22.4; 32-byte blocks on 64^3 73.7 against 78.9) or in
                         // more dimensions (8^5 with 16-byte blocks 65 against 58), as long as a row fits a
@@ -1249,8 +1251,10 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
                         bool mesh_launch = false;
                         for (const LoweredPart &lp : L.parts) min_len = std::min(min_len, lp.p.len);
                         for (int k = 0; k < L.n_used; ++k) mesh_launch = mesh_launch || !c.periodic[L.used_dim[k]];
+                        const bool short_rows = c.P >= 100000 && min_len < 128 && units <= 256;
+                        const bool huge = units >= 1400 && (int64_t)c.P * (int64_t)units * 16 >= (int64_t)1 << 30;
                         const bool scattered = mesh_launch ||
-                                               (L.n_used >= 3 && ((r.kind == ISO_KIND_ALLGATHER && (L.n_used > 3 || c.P < 100000 || min_len >= 128)) ||
+                                               (L.n_used >= 3 && ((r.kind == ISO_KIND_ALLGATHER && (L.n_used > 3 || !(short_rows || huge))) ||
                                                                   (r.kind != ISO_KIND_ALLGATHER && (int64_t)c.P * (int64_t)units * 16 >= kWordsScattered && units <= 1024 &&
                                                                    (L.n_used > 3 || min_len >= 64))));
                         const bool small = may_words && width == 16 &&
