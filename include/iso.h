@@ -227,11 +227,19 @@ int Iso_request_set_layout(Iso_request request, int layout);
  * thread blocks go through the phases together and meet at a grid-wide barrier between
  * them (the ordering point the paper gets from completing a round's MPI_Sendrecv), which
  * saves the ramp-up and drain of one kernel per phase.  The barrier wait is bounded; if it
- * expires the kernel stops and Iso_wait returns ISO_ERR_TIMEOUT.  enable = 0 goes back to
- * one launch per phase, which is the default: with programmatic dependent launches between
+ * expires the kernel stops and Iso_wait returns ISO_ERR_TIMEOUT.  enable = 0 asks for
+ * one launch per phase: with programmatic dependent launches between
  * the phases the per-phase kernels are faster (36.1 against 44.9 microseconds on the 32^3
  * torus, 161 against 197 microseconds on the 8^5 torus with five phases).  Iso_request_get_stats
  * reports launches = 1 once the request has been started in this mode.
+ *
+ * Until this is called the library chooses: the phases of ISO_ALG_COMBINING with fusion level 1 or
+ * more, or one launch for all of them in which thread blocks act for tiles of processes and keep the
+ * intermediate blocks of those in shared memory (small blocks and small tori mostly; no waits on
+ * other thread blocks; Iso_request_get_stats reports launches = 1 after the first start).  Asking for anything
+ * else about the execution - slabs, chains, graph replay, the pipeline, hybrid or sender-side launches, a
+ * bulk threshold - asks for the launches per phase too.  Every hop of the schedule is made in either case;
+ * bytes_moved counts them wherever the block waits in between.
  */
 int Iso_request_set_single_launch(Iso_request request, int enable);
 

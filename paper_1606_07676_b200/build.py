@@ -9,8 +9,8 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libiso_b200.so")
-SOURCES = ["iso_api.cu", "iso_schedule.cpp", "iso_words.cpp"]
-HEADERS = ["iso_internal.h", "iso_kernels.cuh", "iso_words.cuh", os.path.join(ROOT, "include", "iso.h")]
+SOURCES = ["iso_api.cu", "iso_schedule.cpp", "iso_words.cpp", "iso_tiles.cpp"]
+HEADERS = ["iso_internal.h", "iso_kernels.cuh", "iso_words.cuh", "iso_tiles.cuh", os.path.join(ROOT, "include", "iso.h")]
 
 
 def _newest(paths) -> float:

@@ -13,6 +13,7 @@
 #include "iso.h"
 #include "iso_internal.h"
 #include "iso_kernels.cuh"
+#include "iso_tiles.cuh"
 #include "iso_words.cuh"
 
 using namespace iso;
@@ -157,6 +158,7 @@ constexpr size_t kGuardBytes = 4096;
 constexpr int kGuardPattern = 0xC3;
 
 LaunchDev make_launch_args(const Request &r, const LaunchPlan &L);
+void fill_tiles(Request &r);
 void choose_slab_plan(Request &r);
 int build_wave(Request &r, unsigned char *blob, size_t launches_off, size_t items_off, size_t slabs);
 
@@ -314,6 +316,7 @@ int materialise(Request &r)
         r.wave_ok = ok;
     }
     choose_slab_plan(r);
+    plan_tiles(r);
     const int64_t inter_bytes = r.inter_rows * r.inter_stride;
     if (inter_bytes != r.d_inter_bytes) {  // exactly sized, so that the trailing band sits right behind it
         if (r.d_inter_alloc) cudaFree(r.d_inter_alloc);
@@ -355,6 +358,10 @@ int materialise(Request &r)
         if (L.kernel == KERNEL_VEC) bytes += (size_t)L.units_per_proc * sizeof(UnitDev);
         if (L.kernel == KERNEL_FAN) bytes += (size_t)L.units_per_proc * sizeof(FanDev);
     }
+    bytes = (bytes + 15) / 16 * 16;
+    r.tiles.units_off = bytes;
+    r.tiles.shifts_off = bytes + r.tiles.units.size() * sizeof(TileUnit);
+    if (r.tiles.on) bytes = r.tiles.shifts_off + r.tiles.shifts.size() * sizeof(TileShift);
     // one-launch execution: every launch is a 16-byte vector launch on periodic dimensions
     bool single = r.persistent && !r.wave_ok && r.launches.size() >= 2;
     for (const LaunchPlan &L : r.launches) {
@@ -375,6 +382,10 @@ int materialise(Request &r)
     const size_t wave_items_off = bytes;
     bytes += wave_n * sizeof(WaveItem);
     std::vector<unsigned char> blob(bytes ? bytes : 16, 0);
+    if (r.tiles.on) {
+        std::memcpy(blob.data() + r.tiles.units_off, r.tiles.units.data(), r.tiles.units.size() * sizeof(TileUnit));
+        std::memcpy(blob.data() + r.tiles.shifts_off, r.tiles.shifts.data(), r.tiles.shifts.size() * sizeof(TileShift));
+    }
     for (const LaunchPlan *plan : plans) {
         const LaunchPlan &L = *plan;
         if (L.words) {
@@ -454,6 +465,7 @@ int materialise(Request &r)
         }
     }
     ISO_CUDA(cudaMemcpy(r.d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+    if (r.tiles.on) fill_tiles(r);
     // the error flag, only where a kernel may raise it: the vector kernels wait for nothing, and reading the
     // flag back would cost every Iso_wait a copy (8 microseconds)
     r.reports = single || wave_n > 0;
@@ -883,6 +895,115 @@ int launch_one(const Request &r, const LaunchPlan &L, cudaStream_t stream, bool 
 #undef ISO_ROWS_W
 #undef ISO_ROWS
     }
+    ISO_CUDA(e);
+    return ISO_SUCCESS;
+}
+
+// All phases of every tile in one launch.
+template <int W, bool MESH>
+cudaError_t launch_tiles_kernel(const TilesPlan &F, const TilesDev &a, cudaStream_t stream, bool dependent)
+{
+    static std::vector<int> opted_in;  // devices on which the kernel has the larger limits
+    static std::mutex guard;
+    auto *kernel = iso_gather_tiles<W, MESH>;
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    {
+        std::lock_guard<std::mutex> lock(guard);
+        if (std::find(opted_in.begin(), opted_in.end(), device) == opted_in.end()) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynamicSmem);
+            if (e != cudaSuccess) return e;
+            opted_in.push_back(device);
+        }
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)F.grid);
+    cfg.blockDim = dim3((unsigned)F.threads);
+    cfg.dynamicSmemBytes = F.smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+template <int W>
+cudaError_t launch_tiles_unit(const TilesPlan &F, const TilesDev &a, cudaStream_t stream, bool dependent)
+{
+    return F.mesh ? launch_tiles_kernel<W, true>(F, a, stream, dependent) : launch_tiles_kernel<W, false>(F, a, stream, dependent);
+}
+
+// The kernel's argument, the same for every start.
+void fill_tiles(Request &r)
+{
+    const Comm &c = *r.comm;
+    TilesPlan &F = r.tiles;
+    auto div = [](int64_t x) {
+        const FastDiv f = make_fastdiv((uint32_t)x);
+        return FastDivDev{f.m, f.s1, f.s2, f.div};
+    };
+    TilesDev a{};
+    a.units = reinterpret_cast<const TileUnit *>(static_cast<const unsigned char *>(r.d_blob) + F.units_off);
+    a.shifts = reinterpret_cast<const TileShift *>(static_cast<const unsigned char *>(r.d_blob) + F.shifts_off);
+    a.n_shifts = (uint32_t)F.shifts.size();
+    a.send = r.send;
+    a.recv = r.recv;
+    a.send_stride = (uint32_t)r.send_stride;
+    a.recv_stride = (uint32_t)r.recv_stride;
+    a.n_units = (uint32_t)F.units.size();
+    a.n_tiles = (uint32_t)(F.outer * F.intervals);
+    a.n_intervals = (uint32_t)F.intervals;
+    a.middle = (uint32_t)F.middle;
+    a.inner = (uint32_t)F.inner;
+    a.width = (uint32_t)F.width;
+    a.rows_per_tile = (uint32_t)F.rows_per_tile;
+    a.place_stride = (uint32_t)F.place_stride;
+    a.units_at = (uint32_t)F.units_at;
+    a.moved_at = (uint32_t)F.moved_at;
+    a.coords_at = (uint32_t)F.coords_at;
+    a.n_groups = (uint32_t)F.groups.size();
+    for (size_t k = 0; k < F.groups.size(); ++k) {
+        const TileGroup &g = F.groups[k];
+        TileGroupDev &d = a.group[k];
+        const uint32_t passes = (g.n + (uint32_t)F.threads - 1) / (uint32_t)F.threads;
+        d.kind = g.kind;
+        d.width = g.width;
+        d.first = g.first;
+        d.n = g.n;
+        d.owned = (g.n + passes - 1) / passes;
+        d.slots = (uint32_t)F.threads / d.owned;
+        d.div_owned = div(d.owned);
+        d.barrier = k + 1 < F.groups.size() && F.groups[k + 1].stage != g.stage;
+    }
+    a.div_intervals = div(F.intervals);
+    a.div_width = div(F.width);
+    a.div_last_width = div(F.inner - (F.intervals - 1) * F.width);
+    a.div_rows_per_tile = div(F.rows_per_tile);
+    a.n_coords = (uint32_t)F.coords.size();
+    for (size_t k = 0; k < F.coords.size(); ++k) {
+        const int j = F.coords[k];
+        a.size[k] = (uint32_t)c.dims[j];
+        a.div_size[k] = div(c.dims[j]);
+        a.div_stride[k] = div(c.rank_stride[j]);
+        a.stride[k] = (uint32_t)c.rank_stride[j];
+        a.row_stride[k] = (uint32_t)(c.rank_stride[j] / F.inner);
+    }
+    F.args.resize(sizeof(a));
+    std::memcpy(F.args.data(), &a, sizeof(a));
+}
+
+int launch_tiles(const Request &r, cudaStream_t stream, bool dependent)
+{
+    const TilesPlan &F = r.tiles;
+    TilesDev a;
+    std::memcpy(&a, F.args.data(), sizeof(a));
+    const cudaError_t e = F.unit == 16  ? launch_tiles_unit<16>(F, a, stream, dependent)
+                          : F.unit == 8 ? launch_tiles_unit<8>(F, a, stream, dependent)
+                          : F.unit == 4 ? launch_tiles_unit<4>(F, a, stream, dependent)
+                                        : launch_tiles_unit<0>(F, a, stream, dependent);
     ISO_CUDA(e);
     return ISO_SUCCESS;
 }
@@ -1459,6 +1580,7 @@ int Iso_request_set_single_launch(Iso_request request, int enable)
         if (rc != ISO_SUCCESS) return rc;
     }
     request->persistent = enable != 0;
+    request->per_phase = enable == 0;
     request->dirty = true;
     return ISO_SUCCESS;
     });
@@ -1855,6 +1977,13 @@ int Iso_Start(Iso_request request, void *cuda_stream)
         r.started = true;
         return ISO_SUCCESS;
     }
+    if (r.tiles.on) {
+        int rc = launch_tiles(r, stream, use_pdl);
+        if (rc != ISO_SUCCESS) return rc;
+        r.last_stream = cuda_stream;
+        r.started = true;
+        return ISO_SUCCESS;
+    }
     bool replay = r.use_graph;
     if (r.late_graph && r.plain_starts >= 2) {
         // (a graph cannot be launched into a capture; the launches themselves can be recorded)
@@ -2138,7 +2267,7 @@ int Iso_request_get_stats(Iso_request request, Iso_stats *out)
 {
     if (check_handle(request) || !out) return ISO_ERR_ARG;
     *out = request->stats;
-    if (!request->dirty && (request->multi_grid > 0 || request->wave_grid > 0)) out->launches = 1;
+    if (!request->dirty && (request->multi_grid > 0 || request->wave_grid > 0 || request->tiles.on)) out->launches = 1;
     else if (!request->dirty && request->slab_plan.size() > 1) out->launches *= (int)request->slab_plan.size();
     return ISO_SUCCESS;
 }

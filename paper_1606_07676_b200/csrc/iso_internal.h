@@ -184,6 +184,47 @@ struct LaunchPlan {
     size_t parts_off = 0, lookup_off = 0, units_off = 0, fine_off = 0, tiny_off = 0, entries_off = 0;
 };
 
+// ---- all phases of a tile of processes in one launch (iso_tiles.cuh) ----------------------------
+// One unit of a block's hop inside a process's payload.  A place is what a block with hops left (or a
+// trie node with children) occupies in shared memory, the same for every row of a tile.
+struct alignas(16) TileUnit {
+    uint32_t src_off;                 // in the source process's send buffer (stage 0) or places
+    int32_t place_dst, recv_dst;      // in the places, in the receive buffer (-1: not there)
+    uint32_t shift;                   // index of its shift
+};
+static_assert(sizeof(TileUnit) == 16, "unit descriptors are read as 16-byte words");
+// What is subtracted from a row's coordinates to find the process its bytes come from (or go to).  `c` along a periodic
+// dimension in [0, p); `check` as in Part, for the row itself.
+struct TileShift {
+    int32_t c[ISO_MAX_DIMS], check[ISO_MAX_DIMS];
+    uint8_t wraps[ISO_MAX_DIMS];      // the dimension is periodic
+    int32_t between;                  // the partner is a row of the tile
+};
+static_assert(sizeof(TileShift) == 9 * ISO_MAX_DIMS + 4, "compared byte by byte: no padding");
+// What a group of units does.  FETCH: a send buffer's bytes to places, asynchronously.  DELIVER: likewise to the receive buffer
+// (and places).  BETWEEN: from another row's places to the own ones (and the receive buffer).  FORWARD: from the own places to
+// the receive buffer of another process.
+enum : uint32_t { TILE_FETCH = 0, TILE_DELIVER = 1, TILE_BETWEEN = 2, TILE_FORWARD = 3 };
+struct TileGroup {
+    uint32_t kind = TILE_FETCH, width = 16, stage = 0, first = 0, n = 0;
+};
+constexpr int kTileGroups = 40;
+constexpr int kTileThreads = 512;  // of a CTA at most
+
+struct TilesPlan {
+    bool on = false;
+    int64_t outer = 1, middle = 1, inner = 1;  // processes in front of, along and behind the dimensions of the middle hops
+    int64_t width = 1, intervals = 1, rows_per_tile = 0, place_stride = 0, grid = 0;
+    int threads = 256, unit = 16;  // unit: bytes of every unit (0: several widths)
+    bool mesh = false;
+    size_t smem = 0, units_at = 0, moved_at = 0, coords_at = 0, units_off = 0, shifts_off = 0;
+    std::vector<int> coords;          // dimensions whose coordinates the units look at
+    std::vector<TileUnit> units;
+    std::vector<TileShift> shifts;    // the first: none
+    std::vector<TileGroup> groups;    // stage 0: whatever the send buffers provide, then the phases that read places
+    std::vector<unsigned char> args;  // the kernel's argument
+};
+
 // Experiment knobs, read from the environment ONCE, when a request is created, so that a
 // persistent request keeps one plan however the environment changes between its starts.
 // -1 (or 0 where stated) means "not set": the library's own choice applies.
@@ -208,6 +249,7 @@ struct Knobs {
     bool coord_table = true;  // ISO_COORD_TABLE=0: row coordinates by division in every thread
     bool l2_keep = true;      // ISO_L2_KEEP=0: no eviction-priority hint on stores into the intermediate buffer
     int ag_order = -1;        // ISO_AG_ORDER=0/1: allgather visits the dimensions first-to-last / last-to-first
+    int tiles = -1;           // ISO_TILES: 0 = never all phases of a tile in one launch, 1 = wherever possible
     int words = -1;           // ISO_WORDS: 0 = no launches of words, 1 = wherever they can be (-1: chosen by the library)
 };
 Knobs read_knobs();
@@ -278,6 +320,8 @@ struct Request {
     size_t wave_smem = 0, wave_launches_off = 0, wave_items_off = 0;
     unsigned long long wave_run = 0;  // starts since the counters were last zeroed
     int wave_counters = 0;      // counters allocated in d_counter
+    bool per_phase = false;     // one launch per phase was asked for (Iso_request_set_single_launch)
+    TilesPlan tiles;            // all phases of a tile in one launch
     bool lean_tables = false;   // word tables of one row each, where the room for tables is short
     bool plain_units = false;   // no launches of words: every launch in units (Iso_neighbor_alltoall_static)
     bool hybrid = false;        // launches of mixed widths hand their long bodies to bulk warps (Iso_request_set_hybrid)
@@ -298,6 +342,10 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
 
 // Fills L.tables for the lowered launch L (L.words).  The addresses are only used for their alignment.
 void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t recv_addr, uintptr_t inter_addr);
+
+// Whether Iso_Start runs all phases of a tile of processes in one launch, and how (fills r.tiles; the launches
+// stand beside it for the host-buffer path).
+void plan_tiles(Request &r);
 
 // Checks the executed parts for hazards: every range inside its buffer, no write to the send
 // buffer, and within a phase no written range overlapping another written or any read range.

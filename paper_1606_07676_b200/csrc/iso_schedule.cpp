@@ -67,6 +67,7 @@ Knobs read_knobs()
     k.ag_order = num("ISO_AG_ORDER", -1);
     k.l2_keep = num("ISO_L2_KEEP", 1) != 0;
     k.words = (int)num("ISO_WORDS", -1);
+    k.tiles = (int)num("ISO_TILES", -1);
     return k;
 }
 

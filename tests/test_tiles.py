@@ -1,0 +1,126 @@
+"""Schedules whose intermediate blocks fit in shared memory: all phases in one launch, tile by tile.  The plan is
+executed on the host against the schedule's parts; the kernel runs against the oracle."""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_1606_07676_b200 import binding as iso
+from paper_1606_07676_b200 import workloads as wl
+from schedule_sim import POISON
+from test_gpu_fuzz import expected, make_request, random_cases
+from test_gpu_words import _compare
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_1606_07676_b200", "csrc")
+
+
+def test_plans_on_the_host(tmp_path):
+    exe = str(tmp_path / "tiles_sim")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "include"), "-I", CSRC, os.path.join(ROOT, "tests", "tiles_sim.cpp")] +
+                          [os.path.join(CSRC, f) for f in ("iso_schedule.cpp", "iso_words.cpp", "iso_tiles.cpp")] + ["-o", exe])
+    for seed in ("1", "2", "3"):
+        out = subprocess.run([exe, seed], capture_output=True, text=True, timeout=300)
+        assert out.returncode == 0 and int(out.stdout) > 150, out.stdout + out.stderr
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("m", [1, 2, 3, 4, 7, 8, 12, 13, 16, 17, 24, 33, 48, 64, 100, 256, 481])
+@pytest.mark.parametrize("call", ["alltoall", "allgather"])
+def test_block_sizes(m, call, monkeypatch):
+    # tiles of one row and of many, a narrower last one, several tiles to a CTA (257x131), buffers that start anywhere, meshes
+    monkeypatch.setenv("ISO_TILES", "1")
+    for dims, offs in (((13, 11), wl.moore(2, 2)), ((6, 5, 7), wl.moore(3, 1)), ((4, 3, 3, 5), wl.positive_octant(4, 1)), ((257, 131), wl.moore(2, 1))):
+        _compare(wl.Workload("w", call, dims, offs, m, seed=m))
+    _compare(wl.Workload("w", call, (13, 11), wl.moore(2, 1), m, seed=m + 1), lead=(m % 16, (3 * m) % 16))
+    _compare(wl.Workload("w", call, (5, 9, 4), wl.moore(3, 1), m, seed=m + 2), periodic=[0, 1, 0])
+
+
+@pytest.mark.gpu
+def test_rows_of_several_kilobytes(monkeypatch):
+    # a table of units that stays where it is: longer than 1600 and more than two tiles to an SM
+    monkeypatch.setenv("ISO_TILES", "1")
+    _compare(wl.Workload("w", "alltoall", (33, 31), wl.moore(2, 3), 784, seed=1))
+    _compare(wl.Workload("w", "allgather", (33, 31), wl.moore(2, 3), 787, seed=2))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("chunk", range(8))
+def test_random_cases(chunk, monkeypatch):
+    import torch
+    monkeypatch.setenv("ISO_TILES", "1")
+    in_tiles = 0
+    for c in random_cases(300 + chunk):
+        P, ss, rs = c["P"], c["ss"], c["rs"]
+        if not rs or not P * ss:
+            continue
+        send = torch.from_numpy(c["send_h"]).cuda()
+        recv = torch.empty((P, rs), dtype=torch.uint8, device="cuda")
+        comm, req = make_request(c, send, recv)
+        want = expected(c)
+        for fusion in (1, 2, 3):
+            iso.Iso_request_set_algorithm(req, iso.ISO_ALG_COMBINING, fusion)
+            for _ in range(2):
+                recv.fill_(POISON)
+                iso.Iso_Start(req, torch.cuda.current_stream())
+            iso.Iso_wait(req)
+            assert np.array_equal(recv.cpu().numpy(), want), dict(chunk=chunk, trial=c["trial"], dims=c["dims"], kind=c["kind"], fusion=fusion,
+                                                                  periodic=c["periodic"], lens=c["lens"].tolist())
+            st = iso.Iso_request_get_stats(req)
+            in_tiles += st["phases"] > 1 and st["launches"] == 1
+        iso.Iso_request_free(req)
+        iso.Iso_comm_free(comm)
+    assert in_tiles >= 10
+
+
+@pytest.mark.gpu
+def test_left_to_the_library_and_asked_for():
+    """Small calls run in one launch unless something else is asked for; in a graph of the caller's and on another stream
+    as well."""
+    import torch
+    w = wl.Workload("w", "alltoall", (8, 6, 7), wl.moore(3, 1), 24, seed=3)
+    send = wl.payload_torch("uint8", 3, 0, w.P * w.s * 24, "cuda").view(w.P, w.s * 24)
+    recv = torch.empty_like(send)
+    import oracle
+    want = oracle.alltoall(w.dims, w.offsets, 24, send.cpu().numpy())
+    comm = iso.Iso_neighborhood_create(w.dims, w.offsets)
+    req = iso.Iso_neighbor_alltoall_init(send, 24, 1, recv, 24, 1, comm)
+
+    def start(stream=None):
+        recv.fill_(POISON)
+        torch.cuda.synchronize()
+        iso.Iso_Start(req, stream or torch.cuda.current_stream())
+        iso.Iso_wait(req)
+        assert np.array_equal(recv.cpu().numpy(), want)
+        return iso.Iso_request_get_stats(req)["launches"]
+
+    assert start() == 1
+    assert start(torch.cuda.Stream()) == 1
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        iso.Iso_Start(req, torch.cuda.current_stream())
+    recv.fill_(POISON)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(recv.cpu().numpy(), want)
+    iso.Iso_request_set_single_launch(req, False)
+    assert start() == 3
+    iso.Iso_request_free(req)
+    req = iso.Iso_neighbor_alltoall_init(send, 24, 1, recv, 24, 1, comm)
+    iso.Iso_request_set_graph(req, True)
+    assert start() == 3
+    iso.Iso_request_free(req)
+    iso.Iso_comm_free(comm)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("m", [1, 8, 13, 16, 40, 100, 497])
+def test_a_launch_per_phase_of_small_calls(m, monkeypatch):
+    # the kernels that small calls used to run
+    monkeypatch.setenv("ISO_TILES", "0")
+    for call in ("alltoall", "allgather"):
+        for dims, offs in (((13, 11), wl.moore(2, 2)), ((6, 5, 7), wl.moore(3, 1)), ((4, 3, 3, 5), wl.positive_octant(4, 1))):
+            _compare(wl.Workload("w", call, dims, offs, m, seed=m))
+        _compare(wl.Workload("w", call, (13, 11), wl.moore(2, 1), m, seed=m + 1), lead=(m % 16, (3 * m) % 16))
+        _compare(wl.Workload("w", call, (5, 9, 4), wl.moore(3, 1), m, seed=m + 2), periodic=[0, 1, 0])
