@@ -126,6 +126,12 @@ bool collect_hops(const Request &r, std::vector<Hop> &hops, std::list<Part> &own
     return true;
 }
 
+// Three rows and more to a thread: 32^3 with 26 64-byte blocks in CTAs of 256 threads 27, of 512 30, of 128 32 microseconds.
+int64_t tile_threads(int64_t unit_rows, int64_t resident)
+{
+    return std::min<int64_t>(resident == 1 ? kTileThreads : kTileThreads / 2, std::max<int64_t>(64, (unit_rows / 3 + 31) / 32 * 32));
+}
+
 }  // namespace
 
 void plan_tiles(Request &r)
@@ -179,6 +185,7 @@ void plan_tiles(Request &r)
     const int send_align = std::min(alignment16(r.send_stride), alignment16((int64_t)(uintptr_t)r.send));
     const int recv_align = std::min(alignment16(r.recv_stride), alignment16((int64_t)(uintptr_t)r.recv));
     std::vector<Piece> pieces;
+    int64_t apart = 0;  // units of a byte or two whose neighbours are wider: a sector of their own
     F.shifts.assign(1, TileShift{});
     auto before = [](const TileShift &x, const TileShift &y) { return std::memcmp(&x, &y, sizeof(x)) < 0; };  // (no padding)
     std::map<TileShift, uint32_t, decltype(before)> shift_index(before);
@@ -213,6 +220,7 @@ void plan_tiles(Request &r)
             // (asynchronous copies move at least 4 bytes)
             pieces.push_back(Piece{h.stage, h.kind == TILE_FETCH && w < 4 ? TILE_DELIVER : h.kind, (uint32_t)w, u});
             x += w;
+            apart += w < 4 && (a >= 4 || h.len < 4);
             if ((int64_t)pieces.size() > kTilePieces) return;
         }
     }
@@ -239,12 +247,18 @@ void plan_tiles(Request &r)
     const int64_t units = (int64_t)F.units.size(), shifts = (int64_t)F.shifts.size(), table = units * (int64_t)sizeof(TileUnit);
     const int64_t per_row = F.place_stride + 4 * shifts + 2 * (int64_t)F.coords.size();
     auto copied = [&](int64_t tiles) { return units <= 1600 || tiles <= 2 * r.sm_count; };
-    int64_t least = 0, most_tiles = 0;
+    int64_t longest = 1;
+    for (const TileGroup &g : F.groups) longest = std::max<int64_t>(longest, g.n);
+    double least = 0;
+    int64_t most_tiles = 0;
     for (int64_t w = 1; w <= F.inner; ++w) {
         const int64_t rows = F.middle * w, tiles = F.outer * ((F.inner + w - 1) / w);
-        if (rows * per_row + (copied(tiles) ? table : 0) + 128 > (w == 1 ? kTileSmem : kTileTarget)) break;
-        const int64_t per_sm = (tiles + r.sm_count - 1) / r.sm_count;
-        const int64_t cost = per_sm * (units * (rows + 1) + (F.mesh ? 6 : 2) * shifts * rows + 400);
+        const int64_t smem = rows * per_row + (copied(tiles) ? table : 0) + 128;
+        if (smem > (w == 1 ? kTileSmem : kTileTarget)) break;
+        const int64_t per_sm = (tiles + r.sm_count - 1) / r.sm_count, resident = std::max<int64_t>(1, 228 * 1024 / (smem + 1024));
+        const int64_t threads = tile_threads(longest * rows, resident);
+        const double warps = (double)(std::min({resident, 1024 / threads, per_sm}) * threads / 32);
+        const double cost = (double)per_sm * (double)(units * (rows + 1) + (F.mesh ? 6 : 2) * shifts * rows + 400) * (0.75 + 8.0 / warps);
         if (least != 0 && cost >= least) continue;
         least = cost;
         most_tiles = per_sm;
@@ -260,23 +274,26 @@ void plan_tiles(Request &r)
         F.units_at = (size_t)round16((int64_t)F.smem);
         F.smem = F.units_at + (size_t)table;
     }
-    // three rows and more to a thread: 32^3 with 26 64-byte blocks in CTAs of 256 threads 27, of 512 30, of 128 32 microseconds
-    int64_t longest = 1;
-    for (const TileGroup &g : F.groups) longest = std::max<int64_t>(longest, g.n);
     const int64_t resident = std::max<int64_t>(1, 228 * 1024 / ((int64_t)F.smem + 1024));
-    F.threads = (int)std::min<int64_t>(resident == 1 ? kTileThreads : kTileThreads / 2,
-                                       std::max<int64_t>(64, (longest * F.rows_per_tile / 3 + 31) / 32 * 32));
+    F.threads = (int)tile_threads(longest * F.rows_per_tile, resident);
     F.grid = std::min<int64_t>(F.outer * F.intervals, std::min<int64_t>(resident, 1024 / F.threads) * r.sm_count);
 
-    // Which is faster?  Both sides fitted to 210 calls of all sorts (2 to 5 phases, 3 to 630 microseconds; the times of either side
-    // within some 30 % of these), in microseconds.  A launch per phase costs 2.6 each and what is moved at nearly the rate of a copy,
-    // less of it where blocks are not made of 16-byte units; a tile costs what its rows' units do.  The line lies where next to
-    // none of those calls lost: used for 140 of them, in 0.69 of the time (a third took less than half).
-    const double moved = (double)r.stats.bytes_moved / 6.537e6;
-    const double per_phase = 2.6 * r.stats.phases + (r.kind == ISO_KIND_ALLGATHER ? 0.88 : 0.80) * moved +
-                             (F.unit == 16 ? 0.0 : (F.unit == 0 ? 0.39 : 0.82)) * moved;
-    const double in_tiles = 1.6 + 0.23 * (double)F.groups.size() + 0.0003 * (double)least + 0.7 * (double)most_tiles;
-    F.on = r.knobs.tiles >= 1 || in_tiles < 0.8 * per_phase;
+    // Which is faster?  Both sides fitted to 402 calls of all sorts (2 to 5 phases, 3 to 600 microseconds; the times of either side
+    // within some 30 % of these), in microseconds.  A launch costs 2.5, and what is moved nearly the rate of a copy, less of it
+    // where blocks are not made of 16-byte units; where some go to the bulk kernel, which wants long launches, more.  A tile costs
+    // what its rows' units do, and at least what the receive buffers take at 3.6 or 3.3 TB/s (31x22x22 with 342 neighbours, allgather of
+    // 48 bytes, 71 against 60 in phases; 11x11x15x13 with 80, 152 bytes, 142 against 116).  The line lies where next to none of those calls lost: used for 260 of them, in 0.64 of
+    // the time (a quarter took less than half).
+    bool bulk = false;
+    for (const LaunchPlan &L : r.launches) bulk = bulk || L.kernel == KERNEL_BULK;
+    const double moved = (double)r.stats.bytes_moved / 6.537e6, received = (double)r.stats.bytes_min / 2.0 / (F.unit == 16 ? 3.6e6 : 3.3e6);
+    const double per_phase = 2.5 * r.stats.phases + 2.2 * (double)(r.launches.size() - r.stats.phases) + (bulk ? 4.0 - 0.6 * r.stats.phases : 0.0) +
+                             ((r.kind == ISO_KIND_ALLGATHER ? 0.84 : 0.76) + (F.unit == 16 ? 0.0 : (F.unit == 0 ? 0.4 : 0.82))) * moved;
+    // (a byte or two between wider units is a sector of its own on either side: stencil blocks of 324, 18 and 1 bytes on 43x44x39 228
+    // against 167)
+    const double work = least * (1.0 + 4.0 * (double)apart / (double)units);
+    const double in_tiles = std::max(1.3 + 0.23 * (double)F.groups.size() + 0.000215 * work + 0.3 * (double)most_tiles, received);
+    F.on = r.knobs.tiles >= 1 || in_tiles < (F.unit == 0 ? 0.75 : 0.8) * per_phase;
 }
 
 }  // namespace iso
