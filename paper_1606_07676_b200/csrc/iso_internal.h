@@ -195,12 +195,15 @@ struct alignas(16) TileUnit {
 static_assert(sizeof(TileUnit) == 16, "unit descriptors are read as 16-byte words");
 // What is subtracted from a row's coordinates to find the process its bytes come from (or go to).  `c` along a periodic
 // dimension in [0, p); `check` as in Part, for the row itself.
-struct TileShift {
+struct alignas(16) TileShift {
+    uint32_t first_two;               // how many dimensions it moves along (8 bits), `between` (8), the first two of them (8 each)
+    int32_t c_first, c_second;        // and the shifts along those
+    int32_t between;                  // the partner is a row of the tile
     int32_t c[ISO_MAX_DIMS], check[ISO_MAX_DIMS];
     uint8_t wraps[ISO_MAX_DIMS];      // the dimension is periodic
-    int32_t between;                  // the partner is a row of the tile
+    int32_t pad[2];
 };
-static_assert(sizeof(TileShift) == 9 * ISO_MAX_DIMS + 4, "compared byte by byte: no padding");
+static_assert(sizeof(TileShift) == 16 + 9 * ISO_MAX_DIMS + 8, "compared byte by byte: no padding");
 // What a group of units does.  FETCH: a send buffer's bytes to places, asynchronously.  DELIVER: likewise to the receive buffer
 // (and places).  BETWEEN: from another row's places to the own ones (and the receive buffer).  FORWARD: from the own places to
 // the receive buffer of another process.

@@ -126,10 +126,13 @@ bool collect_hops(const Request &r, std::vector<Hop> &hops, std::list<Part> &own
     return true;
 }
 
-// Three rows and more to a thread: 32^3 with 26 64-byte blocks in CTAs of 256 threads 27, of 512 30, of 128 32 microseconds.
+// Threads of a CTA, by how many an SM holds for their shared memory (64 registers each: 1024 threads to an SM), three rows and
+// more to a thread: 32^3 with 26 64-byte blocks, three CTAs, of 320 threads 26.5 microseconds, of 256 27.8, of 512 (two
+// CTAs) 30, of 128 32; irregular sizes on 26x31x22, two of 512 177, of 256 201.
 int64_t tile_threads(int64_t unit_rows, int64_t resident)
 {
-    return std::min<int64_t>(resident == 1 ? kTileThreads : kTileThreads / 2, std::max<int64_t>(64, (unit_rows / 3 + 31) / 32 * 32));
+    const int64_t most = resident <= 2 ? kTileThreads : (resident == 3 ? 320 : kTileThreads / 2);
+    return std::min<int64_t>(most, std::max<int64_t>(64, (unit_rows / 3 + 31) / 32 * 32));
 }
 
 }  // namespace
@@ -175,7 +178,7 @@ void plan_tiles(Request &r)
         bool used = false;
         for (const Part &p : r.parts) used = used || p.shift[j] != 0 || p.check[j] != 0;
         if (!used) continue;
-        if (c.dims[j] > 65535) return;  // (coordinates are kept in 16 bits)
+        if (c.dims[j] > 65535) return;  // (on a mesh coordinates are kept in 16 bits)
         F.mesh = F.mesh || !c.periodic[j];
         coord_of[j] = (int)F.coords.size();
         F.coords.push_back(j);
@@ -207,6 +210,16 @@ void plan_tiles(Request &r)
                 sh.check[e] = c.periodic[j] ? 0 : h.p->check[j] - v;
             }
         }
+        int n = 0;
+        for (int e = 0; e < (int)F.coords.size(); ++e) {
+            if (!sh.c[e]) continue;
+            if (n < 2) {
+                sh.first_two |= (uint32_t)e << (16 + 8 * n);
+                (n == 0 ? sh.c_first : sh.c_second) = sh.c[e];
+            }
+            ++n;
+        }
+        sh.first_two |= (uint32_t)n | (sh.between ? 1u << 8 : 0u);
         const uint32_t index = shift_index.emplace(sh, (uint32_t)F.shifts.size()).first->second;
         if (index == F.shifts.size()) F.shifts.push_back(sh);
         for (int64_t x = 0; x < h.len;) {
@@ -245,7 +258,7 @@ void plan_tiles(Request &r)
     // bytes, two dimensions per phase, 2640 units 373 -> 234 microseconds without; 110x59 with 359 bytes, 752 units, 10.1 with and
     // 13.7 without).
     const int64_t units = (int64_t)F.units.size(), shifts = (int64_t)F.shifts.size(), table = units * (int64_t)sizeof(TileUnit);
-    const int64_t per_row = F.place_stride + 4 * shifts + 2 * (int64_t)F.coords.size();
+    const int64_t per_row = F.place_stride + 4 * shifts + (F.mesh ? 2 * (int64_t)F.coords.size() : 0);
     auto copied = [&](int64_t tiles) { return units <= 1600 || tiles <= 2 * r.sm_count; };
     int64_t longest = 1;
     for (const TileGroup &g : F.groups) longest = std::max<int64_t>(longest, g.n);
@@ -269,7 +282,7 @@ void plan_tiles(Request &r)
     F.rows_per_tile = F.middle * F.width;
     F.moved_at = (size_t)(F.rows_per_tile * F.place_stride);
     F.coords_at = F.moved_at + (size_t)(F.rows_per_tile * shifts) * 4;
-    F.smem = F.coords_at + (size_t)(F.rows_per_tile * 2) * F.coords.size();
+    F.smem = F.coords_at + (F.mesh ? (size_t)(F.rows_per_tile * 2) * F.coords.size() : 0);
     if (copied(F.outer * F.intervals)) {
         F.units_at = (size_t)round16((int64_t)F.smem);
         F.smem = F.units_at + (size_t)table;

@@ -227,45 +227,75 @@ __global__ void __launch_bounds__(kTileThreads, 2) iso_gather_tiles(const __grid
         const uint32_t width = last ? L.inner - interval * L.width : L.width;
         const uint32_t n_rows = L.middle * width;
         const uint32_t rank0 = outer * (L.middle * L.inner) + interval * L.width;
-        for (uint32_t j = threadIdx.x; j < n_rows; j += nthr) {
+        auto rank_of = [&](uint32_t j) -> uint32_t {
             const uint32_t m = last ? fastdiv(L.div_last_width, j) : fastdiv(L.div_width, j);
-            const uint32_t r = rank0 + m * L.inner + (j - m * width);
-            moved[j] = r;
-            for (uint32_t k = 0; k < L.n_coords; ++k) {
-                const uint32_t t = fastdiv(L.div_stride[k], r);
-                coords[j * L.n_coords + k] = (uint16_t)(t - fastdiv(L.div_size[k], t) * L.size[k]);
-            }
-        }
-        __syncthreads();
-        for (uint32_t e = threadIdx.x; e < (L.n_shifts - 1) * L.rows_per_tile; e += nthr) {
-            const uint32_t s = fastdiv(L.div_rows_per_tile, e) + 1, j = e - (s - 1) * L.rows_per_tile;
-            if (j >= n_rows) continue;
-            const TileShift *const sh = L.shifts + s;
-            const bool between = __ldg(&sh->between) != 0;
-            uint32_t r = between ? j : moved[j];
-            for (uint32_t k = 0; k < L.n_coords; ++k) {
-                const int c = __ldg(&sh->c[k]);
-                if (!MESH && c == 0) continue;
-                const int x = coords[j * L.n_coords + k];
-                if (c) {
+            return rank0 + m * L.inner + (j - m * width);
+        };
+        auto coordinate = [&](uint32_t k, uint32_t r) -> uint32_t {
+            const uint32_t t = fastdiv(L.div_stride[k], r);
+            return t - fastdiv(L.div_size[k], t) * L.size[k];
+        };
+        if (!MESH) {
+            // (a row's coordinates are worked out where a shift asks for them: one or two of them mostly, and nothing waits for a
+            // table of them)
+            for (uint32_t e = threadIdx.x; e < L.n_shifts * L.rows_per_tile; e += nthr) {
+                const uint32_t s = fastdiv(L.div_rows_per_tile, e), j = e - s * L.rows_per_tile;
+                if (j >= n_rows) continue;
+                const uint32_t own = rank_of(j);
+                const uint4 h = __ldg(reinterpret_cast<const uint4 *>(L.shifts + s));
+                const uint32_t n = h.x & 0xffu;
+                const bool between = (h.x & 0x100u) != 0;
+                uint32_t r = between ? j : own;
+                auto move = [&](uint32_t k, uint32_t c) {
                     const uint32_t step = between ? L.row_stride[k] * width : L.stride[k];
-                    r -= (uint32_t)c * step;
-                    if (!MESH || __ldg(&sh->wraps[k])) {
-                        if (x < c) r += L.size[k] * step;
-                    } else if (x - c < 0 || x - c >= (int)L.size[k]) {
-                        r = kNobody;
-                        break;
+                    r -= c * step;
+                    if (coordinate(k, own) < c) r += L.size[k] * step;
+                };
+                if (n > 2) {
+                    for (uint32_t k = 0; k < L.n_coords; ++k) {
+                        const uint32_t c = (uint32_t)__ldg(&L.shifts[s].c[k]);
+                        if (c) move(k, c);
                     }
+                } else {
+                    if (n > 0) move((h.x >> 16) & 0xffu, h.y);
+                    if (n > 1) move(h.x >> 24, h.z);
                 }
-                if (MESH) {
-                    const int y = x - __ldg(&sh->check[k]);
-                    if (y < 0 || y >= (int)L.size[k]) {
-                        r = kNobody;
-                        break;
-                    }
-                }
+                moved[e] = r;
             }
-            moved[s * L.rows_per_tile + j] = r;
+        } else {
+            for (uint32_t j = threadIdx.x; j < n_rows; j += nthr) {
+                const uint32_t r = rank_of(j);
+                moved[j] = r;
+                for (uint32_t k = 0; k < L.n_coords; ++k) coords[j * L.n_coords + k] = (uint16_t)coordinate(k, r);
+            }
+            __syncthreads();
+            for (uint32_t e = threadIdx.x; e < (L.n_shifts - 1) * L.rows_per_tile; e += nthr) {
+                const uint32_t s = fastdiv(L.div_rows_per_tile, e) + 1, j = e - (s - 1) * L.rows_per_tile;
+                if (j >= n_rows) continue;
+                const TileShift *const sh = L.shifts + s;
+                const bool between = __ldg(&sh->between) != 0;
+                uint32_t r = between ? j : moved[j];
+                for (uint32_t k = 0; k < L.n_coords; ++k) {
+                    const int c = __ldg(&sh->c[k]);
+                    const int x = coords[j * L.n_coords + k];
+                    bool there = true;
+                    if (c) {
+                        const uint32_t step = between ? L.row_stride[k] * width : L.stride[k];
+                        r -= (uint32_t)c * step;
+                        if (__ldg(&sh->wraps[k])) {
+                            if (x < c) r += L.size[k] * step;
+                        } else {
+                            there = x - c >= 0 && x - c < (int)L.size[k];
+                        }
+                    }
+                    const int y = x - __ldg(&sh->check[k]);
+                    if (!there || y < 0 || y >= (int)L.size[k]) {
+                        r = kNobody;
+                        break;
+                    }
+                }
+                moved[s * L.rows_per_tile + j] = r;
+            }
         }
         __syncthreads();
         if (!ordered) {
