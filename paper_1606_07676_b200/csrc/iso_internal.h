@@ -190,7 +190,7 @@ struct LaunchPlan {
 struct alignas(16) TileUnit {
     uint32_t src_off;                 // in the source process's send buffer (stage 0) or places
     int32_t place_dst, recv_dst;      // in the places, in the receive buffer (-1: not there)
-    uint32_t shift;                   // index of its shift
+    uint32_t shift : 24, width : 8;   // index of its shift, its bytes
 };
 static_assert(sizeof(TileUnit) == 16, "unit descriptors are read as 16-byte words");
 // What is subtracted from a row's coordinates to find the process its bytes come from (or go to).  `c` along a periodic
@@ -209,7 +209,7 @@ static_assert(sizeof(TileShift) == 16 + 9 * ISO_MAX_DIMS + 8, "compared byte by 
 // the receive buffer of another process.
 enum : uint32_t { TILE_FETCH = 0, TILE_DELIVER = 1, TILE_BETWEEN = 2, TILE_FORWARD = 3 };
 struct TileGroup {
-    uint32_t kind = TILE_FETCH, width = 16, stage = 0, first = 0, n = 0;
+    uint32_t kind = TILE_FETCH, width = 16, stage = 0, first = 0, n = 0;  // width 0: units of 8, 4, 2 and 1 bytes, the wider ones first
 };
 constexpr int kTileGroups = 40;
 constexpr int kTileThreads = 512;  // of a CTA at most

@@ -25,7 +25,7 @@
 namespace iso {
 
 struct TileGroupDev {
-    uint32_t kind, width;  // TILE_FETCH ..., bytes of its units
+    uint32_t kind, width;  // TILE_FETCH ..., bytes of its units (0: narrow ones)
     uint32_t first, n;     // units
     uint32_t owned, slots; // unit positions that threads own at a time, rows worked on at a time
     FastDivDev div_owned;
@@ -105,12 +105,66 @@ template <int W> __device__ __forceinline__ void copy_async_at(uint32_t place, c
     else asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(place), "l"(src), "n"(W) : "memory");
 }
 
+// The same for units of W bytes, or (W is kNarrow) of `width`: 8, 4, 2 or 1.
+constexpr int kNarrow = 0;
+template <int W> struct TileVec { using type = typename VecOf<W>::type; };
+template <> struct TileVec<kNarrow> { using type = uint2; };
+template <int W> __device__ __forceinline__ typename TileVec<W>::type unit_from_place(uint32_t a, uint32_t width)
+{
+    if constexpr (W != kNarrow) {
+        return load_shared<W>(a);
+    } else {
+        uint2 v = make_uint2(0, 0);
+        if (width == 8) v = load_shared<8>(a);
+        else if (width == 4) v.x = load_shared<4>(a);
+        else if (width == 2) v.x = load_shared<2>(a);
+        else v.x = load_shared<1>(a);
+        return v;
+    }
+}
+template <int W> __device__ __forceinline__ void unit_to_place(uint32_t a, const typename TileVec<W>::type &v, uint32_t width)
+{
+    if constexpr (W != kNarrow) {
+        store_shared(a, v);
+    } else {
+        if (width == 8) store_shared(a, v);
+        else if (width == 4) store_shared(a, v.x);
+        else if (width == 2) store_shared(a, (uint16_t)v.x);
+        else store_shared(a, (uint8_t)v.x);
+    }
+}
+template <int W> __device__ __forceinline__ typename TileVec<W>::type unit_from_device(const unsigned char *p, uint32_t width)
+{
+    if constexpr (W != kNarrow) {
+        return *reinterpret_cast<const typename TileVec<W>::type *>(p);
+    } else {
+        uint2 v = make_uint2(0, 0);
+        if (width == 8) v = *reinterpret_cast<const uint2 *>(p);
+        else if (width == 4) v.x = *reinterpret_cast<const uint32_t *>(p);
+        else if (width == 2) v.x = *reinterpret_cast<const uint16_t *>(p);
+        else v.x = *p;
+        return v;
+    }
+}
+template <int W> __device__ __forceinline__ void unit_to_device(unsigned char *p, const typename TileVec<W>::type &v, uint32_t width)
+{
+    if constexpr (W != kNarrow) {
+        *reinterpret_cast<typename TileVec<W>::type *>(p) = v;
+    } else {
+        if (width == 8) *reinterpret_cast<uint2 *>(p) = v;
+        else if (width == 4) *reinterpret_cast<uint32_t *>(p) = v.x;
+        else if (width == 2) *reinterpret_cast<uint16_t *>(p) = (uint16_t)v.x;
+        else *p = (unsigned char)v.x;
+    }
+}
+
 constexpr uint32_t kNobody = 0xffffffffu;  // no partner: outside a mesh
 
-// What a thread needs to know about the unit it moves, beside the group's kind and width.
+// What a thread needs to know about the unit it moves, beside the group's kind.
 struct TileWalk {
     uint32_t src_off;
     int place_dst, recv_dst;
+    uint32_t width;
     uint32_t partner;  // shared-memory address of the partner of the thread's first row
     uint32_t own;      // of that row's rank
     uint32_t row;      // that row
@@ -128,18 +182,23 @@ __device__ __forceinline__ void fetch_tile(const TilesDev &L, uint32_t places_at
 #pragma unroll 4
     for (int left = t.left; left > 0; left -= (int)t.step) {
         const uint32_t r = load_shared<4>(partner);
-        if (!MESH || r != kNobody) copy_async_at<W>(to, src + (unsigned long long)r * L.send_stride);
+        if (!MESH || r != kNobody) {
+            const unsigned char *const from = src + (unsigned long long)r * L.send_stride;
+            if constexpr (W != kNarrow) copy_async_at<W>(to, from);
+            else if (t.width == 8) copy_async_at<8>(to, from);
+            else copy_async_at<4>(to, from);  // (asynchronous copies move at least 4 bytes; narrower units are delivered)
+        }
         partner += 4 * t.step;
         to += place_step;
     }
 }
 
-// The other kinds of a group's units of W bytes, as one thread moves them.  What a row costs here is what the kernel costs: a
+// The other kinds of a group's units, as one thread moves them.  What a row costs here is what the kernel costs: a
 // table entry, an address, a load and a store.
 template <int W, int R, uint32_t KIND, bool MESH>
 __device__ __forceinline__ void walk_tile(const TilesDev &L, uint32_t places_at, const TileWalk &t)
 {
-    using V = typename VecOf<W>::type;
+    using V = typename TileVec<W>::type;
     const uint32_t place_step = t.step * L.place_stride;
     const unsigned char *const src = L.send + t.src_off;
     unsigned char *const dst = L.recv + t.recv_dst;
@@ -160,11 +219,11 @@ __device__ __forceinline__ void walk_tile(const TilesDev &L, uint32_t places_at,
             const bool there = MESH ? r[i] != kNobody : left > i * (int)t.step;
             if (there) {
                 if (KIND == TILE_DELIVER) {
-                    v[i] = *reinterpret_cast<const V *>(src + (unsigned long long)r[i] * L.send_stride);
+                    v[i] = unit_from_device<W>(src + (unsigned long long)r[i] * L.send_stride, t.width);
                 } else if (KIND == TILE_FORWARD) {
-                    v[i] = load_shared<W>(from + i * place_step);
+                    v[i] = unit_from_place<W>(from + i * place_step, t.width);
                 } else {
-                    v[i] = load_shared<W>(from0 + r[i] * L.place_stride);
+                    v[i] = unit_from_place<W>(from0 + r[i] * L.place_stride, t.width);
                 }
             }
         }
@@ -173,11 +232,11 @@ __device__ __forceinline__ void walk_tile(const TilesDev &L, uint32_t places_at,
             const bool there = MESH ? r[i] != kNobody : left > i * (int)t.step;
             if (there) {
                 if (KIND == TILE_FORWARD) {
-                    *reinterpret_cast<V *>(dst + (unsigned long long)r[i] * L.recv_stride) = v[i];
+                    unit_to_device<W>(dst + (unsigned long long)r[i] * L.recv_stride, v[i], t.width);
                 } else {
-                    if (t.place_dst >= 0) store_shared(to + i * place_step, v[i]);
+                    if (t.place_dst >= 0) unit_to_place<W>(to + i * place_step, v[i], t.width);
                     if (t.recv_dst >= 0)
-                        *reinterpret_cast<V *>(dst + (unsigned long long)load_shared<4>(own + 4 * i * t.step) * L.recv_stride) = v[i];
+                        unit_to_device<W>(dst + (unsigned long long)load_shared<4>(own + 4 * i * t.step) * L.recv_stride, v[i], t.width);
                 }
             }
         }
@@ -192,7 +251,7 @@ template <int W, int R, bool MESH>
 __device__ __forceinline__ void walk_group(const TilesDev &L, uint32_t kind, uint32_t places_at, const TileWalk &t)
 {
     if (kind == TILE_FETCH) {
-        if constexpr (W >= 4) fetch_tile<W, MESH>(L, places_at, t);  // (asynchronous copies move at least 4 bytes)
+        fetch_tile<W, MESH>(L, places_at, t);
     } else if (kind == TILE_DELIVER) {
         walk_tile<W, R, TILE_DELIVER, MESH>(L, places_at, t);
     } else if (kind == TILE_BETWEEN) {
@@ -202,9 +261,9 @@ __device__ __forceinline__ void walk_group(const TilesDev &L, uint32_t kind, uin
     }
 }
 
-// W: bytes of every unit, 0: those of its group.  MESH: some dimensions are not periodic, and a row may
+// W: bytes of every unit, 0: 16, or fewer in some groups.  MESH: some dimensions are not periodic, and a row may
 // have no partner for a shift.
-// A thread owns a unit position of a group (a kind of move, a width) and walks down the rows (processes) of
+// A thread owns a unit position of a group (a kind of move, 16 bytes or fewer) and walks down the rows (processes) of
 // its CTA.  Which process a row's bytes come from or go to depends on the shift and the row alone: the CTA
 // tabulates it for every tile.
 template <int W, bool MESH>
@@ -314,16 +373,15 @@ __global__ void __launch_bounds__(kTileThreads, 2) iso_gather_tiles(const __grid
                     t.place_dst = (int)a.y;
                     t.recv_dst = (int)a.z;
                     t.own = places_at + L.moved_at + 4 * g;
-                    t.partner = t.own + 4 * (a.w * L.rows_per_tile);
+                    t.partner = t.own + 4 * ((a.w & 0xffffffu) * L.rows_per_tile);
                     t.row = g;
                     t.left = (int)(n_rows - g);
                     t.step = T.slots;
+                    t.width = a.w >> 24;
                     if (W != 0) walk_group<(W != 0 ? W : 16), 4, MESH>(L, T.kind, places_at, t);
                     else if (T.width == 16) walk_group<16, 2, MESH>(L, T.kind, places_at, t);
-                    else if (T.width == 8) walk_group<8, 2, MESH>(L, T.kind, places_at, t);
-                    else if (T.width == 4) walk_group<4, 2, MESH>(L, T.kind, places_at, t);
-                    else if (T.width == 2) walk_group<2, 2, MESH>(L, T.kind, places_at, t);
-                    else walk_group<1, 2, MESH>(L, T.kind, places_at, t);
+                    else if (!MESH && T.width == 8) walk_group<8, 2, MESH>(L, T.kind, places_at, t);  // (with it the mesh kernel spills: 126 -> 147)
+                    else walk_group<kNarrow, 2, MESH>(L, T.kind, places_at, t);
                 }
             if (T.barrier) {
                 cp_async_commit();

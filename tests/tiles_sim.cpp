@@ -92,23 +92,25 @@ Bytes by_tiles(const Request &r, const Bytes &send)
             stage = g.stage;
             for (uint32_t u = g.first; u < g.first + g.n; ++u) {
                 const TileUnit &t = F.units[u];
+                require(g.width == 0 ? t.width < 16 : t.width == g.width, "width");
+                require(g.kind != TILE_FETCH || t.width >= 4, "asynchronous copies");
                 for (int64_t j = 0; j < rows; ++j) {
                     const int64_t p = partner(F.shifts[t.shift], j);
                     if (p < 0) continue;
                     const bool global = g.kind == TILE_FETCH || g.kind == TILE_DELIVER;
                     const int64_t row = g.kind == TILE_FORWARD ? j : p;
-                    require(global ? p < c.P && t.src_off + g.width <= r.send_stride : row < rows && t.src_off + g.width <= F.place_stride, "source");
+                    require(global ? p < c.P && t.src_off + t.width <= r.send_stride : row < rows && t.src_off + t.width <= F.place_stride, "source");
                     const unsigned char *from = global ? &send[p * r.send_stride + t.src_off] : &before[row * F.place_stride + t.src_off];
                     const uintptr_t src_at = global ? (uintptr_t)r.send + p * r.send_stride + t.src_off : t.src_off;
-                    require(src_at % g.width == 0, "alignment of a source");
+                    require(src_at % t.width == 0, "alignment of a source");
                     if (g.kind != TILE_FORWARD && t.place_dst >= 0) {
-                        require(t.place_dst + g.width <= F.place_stride && t.place_dst % g.width == 0, "place");
-                        std::memcpy(&places[j * F.place_stride + t.place_dst], from, g.width);
+                        require(t.place_dst + t.width <= F.place_stride && t.place_dst % t.width == 0, "place");
+                        std::memcpy(&places[j * F.place_stride + t.place_dst], from, t.width);
                     }
                     if (t.recv_dst >= 0) {
                         const int64_t to = (g.kind == TILE_FORWARD ? p : rank[j]) * r.recv_stride + t.recv_dst;
-                        require(t.recv_dst + g.width <= r.recv_stride && ((uintptr_t)r.recv + to) % g.width == 0, "receive buffer");
-                        std::memcpy(&recv[to], from, g.width);
+                        require(t.recv_dst + t.width <= r.recv_stride && ((uintptr_t)r.recv + to) % t.width == 0, "receive buffer");
+                        std::memcpy(&recv[to], from, t.width);
                     }
                 }
             }
