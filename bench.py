@@ -342,7 +342,7 @@ class Bound:
             self.req = iso.Iso_neighbor_alltoallv_init(self.send, self.lens, self.sd, 1, self.recv, self.lens, self.rd, 1, self.comm)
 
     bulk_threshold = None
-    single_launch = False
+    single_launch = None  # None: the library's choice
     slabs = None      # None: the library's choice
     chains = None
     graph = None
@@ -600,7 +600,7 @@ def run_ours(args):
 
     peak, peak_kind = measured_peak()
     Bound.bulk_threshold = args.bulk_threshold
-    Bound.single_launch = args.single_launch
+    Bound.single_launch = args.single_launch or None
     Bound.slabs, Bound.chains, Bound.graph, Bound.tune = args.slabs, args.chains, args.graph, args.tune
     Bound.pipeline = args.pipeline
     reps = Replicas(torch, iso, wl, args.workload)
@@ -852,7 +852,7 @@ def main():
                     help="one K-step run of the headline schedule and nothing else (short runs under a profiler)")
     ap.add_argument("--no-detail", action="store_true", help="skip the table of configurations")
     ap.add_argument("--single-launch", action="store_true",
-                    help="run all phases in one cooperative launch instead of one launch per phase")
+                    help="run all phases in one cooperative launch (default: the library's choice)")
     ap.add_argument("--bulk-threshold", type=int, default=None,
                     help="override the size from which parts go to the bulk-copy kernel (0: never)")
     ap.add_argument("--slabs", type=int, default=None, help="slabs of dimension 0 (default: the library's choice)")

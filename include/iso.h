@@ -233,7 +233,8 @@ int Iso_request_set_layout(Iso_request request, int layout);
  * torus, 161 against 197 microseconds on the 8^5 torus with five phases).  Iso_request_get_stats
  * reports launches = 1 once the request has been started in this mode.
  *
- * Until this is called the library chooses: the phases of ISO_ALG_COMBINING with fusion level 1 or
+ * Until this is called, and again after a call with ISO_LAUNCH_AUTO, the library chooses: the phases
+ * of ISO_ALG_COMBINING with fusion level 1 or
  * more, or one launch for all of them in which thread blocks act for tiles of processes and keep the
  * intermediate blocks of those in shared memory (small blocks and small tori mostly; no waits on
  * other thread blocks; Iso_request_get_stats reports launches = 1 after the first start).  Asking for anything
@@ -241,6 +242,7 @@ int Iso_request_set_layout(Iso_request request, int layout);
  * bulk threshold - asks for the launches per phase too.  Every hop of the schedule is made in either case;
  * bytes_moved counts them wherever the block waits in between.
  */
+enum { ISO_LAUNCH_AUTO = -1 };
 int Iso_request_set_single_launch(Iso_request request, int enable);
 
 /*

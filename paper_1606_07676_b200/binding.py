@@ -251,8 +251,13 @@ def Iso_request_set_layout(request: int, layout: int) -> None:
     _check(load_library().Iso_request_set_layout(request, layout), "Iso_request_set_layout")
 
 
-def Iso_request_set_single_launch(request: int, enable: bool) -> None:
-    _check(load_library().Iso_request_set_single_launch(request, 1 if enable else 0), "Iso_request_set_single_launch")
+ISO_LAUNCH_AUTO = -1
+
+
+def Iso_request_set_single_launch(request: int, enable: bool | None) -> None:
+    """True: one cooperative launch, False: one launch per phase, None: the library chooses (the default)."""
+    value = ISO_LAUNCH_AUTO if enable is None else (1 if enable else 0)
+    _check(load_library().Iso_request_set_single_launch(request, value), "Iso_request_set_single_launch")
 
 
 def Iso_request_set_pipeline(request: int, slabs: int) -> None:

@@ -1579,7 +1579,7 @@ int Iso_request_set_single_launch(Iso_request request, int enable)
         int rc = Iso_wait(request);
         if (rc != ISO_SUCCESS) return rc;
     }
-    request->persistent = enable != 0;
+    request->persistent = enable != 0 && enable != ISO_LAUNCH_AUTO;
     request->per_phase = enable == 0;
     request->dirty = true;
     return ISO_SUCCESS;

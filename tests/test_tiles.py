@@ -106,12 +106,29 @@ def test_left_to_the_library_and_asked_for():
     assert np.array_equal(recv.cpu().numpy(), want)
     iso.Iso_request_set_single_launch(req, False)
     assert start() == 3
+    iso.Iso_request_set_single_launch(req, None)
+    assert start() == 1
+    iso.Iso_request_set_single_launch(req, True)    # (24-byte blocks do not run in a cooperative launch)
+    assert start() == 3
+    iso.Iso_request_set_single_launch(req, None)
+    assert start() == 1
     iso.Iso_request_free(req)
     req = iso.Iso_neighbor_alltoall_init(send, 24, 1, recv, 24, 1, comm)
     iso.Iso_request_set_graph(req, True)
     assert start() == 3
     iso.Iso_request_free(req)
     iso.Iso_comm_free(comm)
+
+
+@pytest.mark.gpu
+def test_the_benchmark_measures_the_default():
+    import sys
+    import torch
+    sys.path.insert(0, ROOT)
+    import bench
+    b = bench.Bound(torch, iso, wl, "cfg2_alltoall")
+    assert b.set(iso.ISO_ALG_COMBINING, 1)["launches"] == 1
+    b.close()
 
 
 @pytest.mark.gpu
