@@ -237,9 +237,11 @@ int Iso_request_set_layout(Iso_request request, int layout);
  * of ISO_ALG_COMBINING with fusion level 1 or
  * more, or one launch for all of them in which thread blocks act for tiles of processes and keep the
  * intermediate blocks of those in shared memory (small blocks and small tori mostly; no waits on
- * other thread blocks; Iso_request_get_stats reports launches = 1 after the first start).  Asking for anything
- * else about the execution - slabs, chains, graph replay, the pipeline, hybrid or sender-side launches, a
- * bulk threshold - asks for the launches per phase too.  Every hop of the schedule is made in either case;
+ * other thread blocks; Iso_request_get_stats reports launches = 1 after the first start, and
+ * Iso_request_get_execution one slab, one chain and no graph).  Asking for anything
+ * else about the execution - two slabs or chains and more, graph replay, the pipeline, hybrid or sender-side
+ * launches, a bulk threshold - asks for the launches per phase too; so does Iso_request_tune where it measured
+ * those to be faster.  Every hop of the schedule is made in either case;
  * bytes_moved counts them wherever the block waits in between.
  */
 enum { ISO_LAUNCH_AUTO = -1 };

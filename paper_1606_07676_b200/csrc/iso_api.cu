@@ -1647,9 +1647,10 @@ int Iso_request_get_execution(Iso_request request, int *slabs, int *chains, int 
 {
     if (check_handle(request)) return ISO_ERR_ARG;
     const Request &r = *request;
-    if (slabs) *slabs = r.dirty ? r.slab_request : (int)std::max<size_t>(1, r.slab_plan.size());
-    if (chains) *chains = r.dirty ? std::max(1, r.chains_request) : r.chains;
-    if (graph) *graph = r.dirty ? (r.graph_request ? 1 : 0) : (r.use_graph || r.graph_exec ? 1 : 0);
+    const bool tiles = !r.dirty && r.tiles.on;  // (one launch: the plan of the launches stands aside)
+    if (slabs) *slabs = r.dirty ? r.slab_request : (tiles ? 1 : (int)std::max<size_t>(1, r.slab_plan.size()));
+    if (chains) *chains = r.dirty ? std::max(1, r.chains_request) : (tiles ? 1 : r.chains);
+    if (graph) *graph = r.dirty ? (r.graph_request ? 1 : 0) : (!tiles && (r.use_graph || r.graph_exec) ? 1 : 0);
     return ISO_SUCCESS;
 }
 
@@ -1685,8 +1686,9 @@ int Iso_request_tune(Iso_request request, void *cuda_stream, int flags)
     }
     const bool log = r.knobs.tune_log;
     // order: visiting order of the allgather's trie (-1: as it was, 0: first dimension first, 1: last first)
-    struct Choice { int slabs, chains, graph, alg, fusion, hybrid, order; };
-    const Choice before{r.slab_request, r.chains_request, r.graph_request ? 1 : 0, r.alg, r.fusion, r.hybrid ? 1 : 0, -1};
+    // per_phase: no tiles (they are what the library chooses where it chooses them, and have neither slabs nor chains)
+    struct Choice { int slabs, chains, graph, alg, fusion, hybrid, order; bool per_phase; };
+    const Choice before{r.slab_request, r.chains_request, r.graph_request ? 1 : 0, r.alg, r.fusion, r.hybrid ? 1 : 0, -1, r.per_phase};
     int order_before[ISO_MAX_DIMS];
     std::copy(r.dim_order, r.dim_order + ISO_MAX_DIMS, order_before);
     int order_now = -1;
@@ -1699,6 +1701,7 @@ int Iso_request_tune(Iso_request request, void *cuda_stream, int flags)
         r.chains_request = c.chains;
         r.graph_request = c.graph != 0;
         r.hybrid = c.hybrid != 0;
+        r.per_phase = c.per_phase;
         r.dirty = true;
         if (c.order != order_now) {
             int order[ISO_MAX_DIMS];
@@ -1766,7 +1769,7 @@ int Iso_request_tune(Iso_request request, void *cuda_stream, int flags)
         // ragged rows only: does the lowering hand anything to bulk warps?
         r.hybrid = true;
         if (r.started) rc = Iso_wait(request);
-        if (rc == ISO_SUCCESS) rc = apply(Choice{1, 1, 0, sched.first, sched.second, 1, sched.order});
+        if (rc == ISO_SUCCESS) rc = apply(Choice{1, 1, 0, sched.first, sched.second, 1, sched.order, true});
         if (rc == ISO_SUCCESS) rc = lower_schedule(r, (uintptr_t)r.send, (uintptr_t)r.recv, (uintptr_t)r.d_inter);
         bool any = false;
         for (const LaunchPlan &L : r.launches) any = any || !L.side.empty();
@@ -1779,7 +1782,7 @@ int Iso_request_tune(Iso_request request, void *cuda_stream, int flags)
         if (rc == ISO_SUCCESS) rc = materialise(r);
         if (rc != ISO_SUCCESS) return;
         // what the schedule allowed may differ from what was asked for: skip repeats
-        const Choice got{(int)std::max<size_t>(1, r.slab_plan.size()), r.chains, r.use_graph ? 1 : 0, r.alg, r.fusion, hybrid, sched.order};
+        const Choice got{(int)std::max<size_t>(1, r.slab_plan.size()), r.chains, r.use_graph ? 1 : 0, r.alg, r.fusion, hybrid, sched.order, c.per_phase};
         for (const Choice &t : tried)
             if (t.slabs == got.slabs && t.chains == got.chains && t.graph == got.graph) return;
         if (c.slabs > 0) tried.push_back(got);  // (a plan of the library's own may use other kernels)
@@ -1799,13 +1802,13 @@ int Iso_request_tune(Iso_request request, void *cuda_stream, int flags)
         }
     };
     // (the plan the library would choose for the schedule, as the request came with it unless it was told otherwise)
-    if (!hybrid) consider(Choice{0, 0, 0, sched.first, sched.second, 0, sched.order});
+    if (!hybrid) consider(Choice{0, 0, 0, sched.first, sched.second, 0, sched.order, false});
     for (int graph = 0; graph <= 1 && rc == ISO_SUCCESS; ++graph)
         for (int chains = 1; chains <= 4 && rc == ISO_SUCCESS; chains *= 2) {
             if (chains > 1 && !graph) continue;  // chains that are asked for run from a graph in any case
             for (int slabs = 1; slabs <= 64 && slabs <= std::max(1, p0) && rc == ISO_SUCCESS; slabs *= 2) {
                 if (chains > 1 && slabs < chains) continue;
-                consider(Choice{slabs, chains, graph, sched.first, sched.second, hybrid, sched.order});
+                consider(Choice{slabs, chains, graph, sched.first, sched.second, hybrid, sched.order, true});
             }
         }
     }

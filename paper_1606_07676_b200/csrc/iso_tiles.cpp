@@ -37,11 +37,12 @@ struct Piece {
     TileUnit u;
 };
 
-// Whether anything but the schedule was asked for: how it is cut into launches, or by which kernels it runs.
+// Whether anything but the schedule was asked for: how it is cut into launches, or by which kernels it runs.  (One slab and
+// one chain are what a single launch has: a plan read back from one request and asked for on another stays what it was.)
 bool execution_asked_for(const Request &r)
 {
     const Knobs &k = r.knobs;
-    return r.per_phase || r.persistent || r.wave_request || r.slab_request || r.chains_request || r.graph_request || r.hybrid ||
+    return r.per_phase || r.persistent || r.wave_request || r.slab_request > 1 || r.chains_request > 1 || r.graph_request || r.hybrid ||
            r.bulk_threshold_asked >= 0 || r.sender_side != 1 || k.slabs >= 0 || k.chains >= 0 || k.graph >= 0 || k.vec_threads ||
            k.vec_ctas_per_sm || k.words >= 0 || k.sender_side >= 0 || k.hybrid >= 0 || k.mixed >= 0 || k.bulk_chunk || k.bulk_tile;
 }

@@ -121,6 +121,47 @@ def test_left_to_the_library_and_asked_for():
 
 
 @pytest.mark.gpu
+def test_execution_read_back_and_tuned(monkeypatch):
+    """What is reported is what runs, and asked for on another request it runs there too; the tuner knows this route
+    whatever the request was told before."""
+    import torch
+
+    def bound(w):
+        send = wl.payload_torch("uint8", 3, 0, w.P * w.s * w.block_bytes, "cuda")
+        recv = torch.empty_like(send)
+        comm = iso.Iso_neighborhood_create(w.dims, w.offsets)
+        req = iso.Iso_neighbor_alltoall_init(send, w.block_bytes, 1, recv, w.block_bytes, 1, comm)
+        iso.Iso_comm_free(comm)
+        return send, recv, req
+
+    def launches(req):
+        iso.Iso_Start(req, torch.cuda.current_stream())
+        iso.Iso_wait(req)
+        return iso.Iso_request_get_stats(req)["launches"]
+
+    small = wl.Workload("w", "alltoall", (8, 6, 7), wl.moore(3, 1), 24, seed=3)
+    one, two = bound(small), bound(small)
+    assert launches(one[2]) == 1
+    ex = iso.Iso_request_get_execution(one[2])
+    assert ex == {"slabs": 1, "chains": 1, "graph": 0}
+    iso.Iso_request_set_slabs(two[2], ex["slabs"])
+    iso.Iso_request_set_chains(two[2], ex["chains"])
+    iso.Iso_request_set_graph(two[2], bool(ex["graph"]))
+    assert launches(two[2]) == 1
+    iso.Iso_request_set_single_launch(one[2], False)
+    assert launches(one[2]) == 3
+    iso.Iso_request_tune(one[2], torch.cuda.current_stream())   # 3.1 microseconds against 7
+    assert launches(one[2]) == 1
+    iso.Iso_request_set_slabs(two[2], 2)
+    assert launches(two[2]) == 6
+    monkeypatch.setenv("ISO_TILES", "1")
+    many = bound(wl.Workload("w", "alltoall", (256, 256), wl.moore(2, 2), 64, seed=4))  # (two slabs, were it run in phases)
+    assert launches(many[2]) == 1 and iso.Iso_request_get_execution(many[2]) == ex
+    for b in (one, two, many):
+        iso.Iso_request_free(b[2])
+
+
+@pytest.mark.gpu
 def test_the_benchmark_measures_the_default():
     import sys
     import torch
