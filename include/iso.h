@@ -406,8 +406,8 @@ int Iso_comm_set_periodic(Iso_comm isocomm, const int periodic[]);
  * Runs the collective: enqueues the schedule's kernels on `cuda_stream` (a cudaStream_t
  * cast to void*, NULL = the default stream) and returns without waiting (the non-blocking
  * start proposed in Section VII).  The first start after an init or a set_* call also
- * allocates the intermediate buffer and uploads the index tables (cudaMalloc and a blocking
- * copy), so it must not happen inside a stream capture.  Starts of one request are ordered
+ * uploads the index tables and, unless all phases run in tiles, allocates the intermediate
+ * buffer (cudaMalloc and a blocking copy), so it must not happen inside a stream capture.  Starts of one request are ordered
  * by the stream they are enqueued on: a request owns one intermediate buffer, so two starts
  * of the same request on different streams must not overlap.
  * Errors: ISO_ERR_STATE (request has no buffers), ISO_ERR_NOMEM, ISO_ERR_CUDA.
@@ -423,7 +423,8 @@ int Iso_Start(Iso_request request, void *cuda_stream);
  * its receive buffers travel back while later slabs are still being uploaded (uploads and
  * downloads on two internal streams created by the first such call, kernels on
  * `cuda_stream`, which is made to wait for the downloads).  Otherwise: one upload, the
- * schedule, one download, all on `cuda_stream`.  The copies are asynchronous when the host
+ * schedule, one download, all on `cuda_stream`.  The slabs run one launch per phase: for a request whose starts
+ * run in tiles the first such call sets those up (tables and intermediate buffer).  The copies are asynchronous when the host
  * memory is page-locked.  Complete after Iso_wait or a synchronisation of `cuda_stream`. */
 int Iso_Start_host(Iso_request request, const void *host_sendbuf, void *host_recvbuf,
                    void *cuda_stream);

@@ -48,6 +48,8 @@ void release_device(Request &r)
     if (r.host_main_stream) cudaStreamDestroy(static_cast<cudaStream_t>(r.host_main_stream));
     r.host_main_stream = nullptr;
     if (r.d_blob) cudaFree(r.d_blob);
+    if (r.d_tiles) cudaFree(r.d_tiles);
+    r.d_tiles = nullptr;
     if (r.d_inter_alloc) cudaFree(r.d_inter_alloc);
     r.d_inter_alloc = nullptr;
     if (r.d_err) cudaFree(r.d_err);
@@ -158,7 +160,8 @@ constexpr size_t kGuardBytes = 4096;
 constexpr int kGuardPattern = 0xC3;
 
 LaunchDev make_launch_args(const Request &r, const LaunchPlan &L);
-void fill_tiles(Request &r);
+int upload_tiles(Request &r);
+int materialise_launches(Request &r, cudaStream_t up);
 void choose_slab_plan(Request &r);
 int build_wave(Request &r, unsigned char *blob, size_t launches_off, size_t items_off, size_t slabs);
 
@@ -277,7 +280,8 @@ void fill_words(const LaunchPlan &L, unsigned char *blob)
     put(L.fine_off, L.tables.fine);
 }
 
-// Uploads the lowered schedule and allocates the intermediate buffer.
+// Decides how the request runs and uploads what Iso_Start needs for that: the tables of the tiles, or those of the launches
+// beside their intermediate buffer.
 int materialise(Request &r)
 {
     const Comm &c = *r.comm;
@@ -317,6 +321,23 @@ int materialise(Request &r)
     }
     choose_slab_plan(r);
     plan_tiles(r);
+    if (r.d_tiles) cudaFree(r.d_tiles);
+    r.d_tiles = nullptr;
+    r.launches_ready = false;
+    r.multi_grid = 0;
+    r.reports = false;
+    const int rc = r.tiles.on ? upload_tiles(r) : materialise_launches(r, nullptr);
+    if (rc != ISO_SUCCESS) return rc;
+    r.dirty = false;
+    return ISO_SUCCESS;
+}
+
+// Uploads the tables of the launches and allocates the intermediate buffer, on the default stream or, as a whole, on the stream `up`.
+int materialise_launches(Request &r, cudaStream_t up)
+{
+    const Comm &c = *r.comm;
+    int device = 0;
+    ISO_CUDA(cudaGetDevice(&device));
     const int64_t inter_bytes = r.inter_rows * r.inter_stride;
     if (inter_bytes != r.d_inter_bytes) {  // exactly sized, so that the trailing band sits right behind it
         if (r.d_inter_alloc) cudaFree(r.d_inter_alloc);
@@ -328,8 +349,8 @@ int materialise(Request &r)
         ISO_CUDA(cudaMalloc((void **)&r.d_inter_alloc, (size_t)inter_bytes + 2 * kGuardBytes));
         r.d_inter = r.d_inter_alloc + kGuardBytes;
         r.d_inter_bytes = inter_bytes;
-        ISO_CUDA(cudaMemset(r.d_inter_alloc, kGuardPattern, kGuardBytes));
-        ISO_CUDA(cudaMemset(r.d_inter + inter_bytes, kGuardPattern, kGuardBytes));
+        ISO_CUDA(cudaMemsetAsync(r.d_inter_alloc, kGuardPattern, kGuardBytes, up));
+        ISO_CUDA(cudaMemsetAsync(r.d_inter + inter_bytes, kGuardPattern, kGuardBytes, up));
         }
     }
     // (the launches stand: the lowering only looks at the buffer's alignment, and every intermediate
@@ -358,10 +379,6 @@ int materialise(Request &r)
         if (L.kernel == KERNEL_VEC) bytes += (size_t)L.units_per_proc * sizeof(UnitDev);
         if (L.kernel == KERNEL_FAN) bytes += (size_t)L.units_per_proc * sizeof(FanDev);
     }
-    bytes = (bytes + 15) / 16 * 16;
-    r.tiles.units_off = bytes;
-    r.tiles.shifts_off = bytes + r.tiles.units.size() * sizeof(TileUnit);
-    if (r.tiles.on) bytes = r.tiles.shifts_off + r.tiles.shifts.size() * sizeof(TileShift);
     // one-launch execution: every launch is a 16-byte vector launch on periodic dimensions
     bool single = r.persistent && !r.wave_ok && r.launches.size() >= 2;
     for (const LaunchPlan &L : r.launches) {
@@ -382,10 +399,6 @@ int materialise(Request &r)
     const size_t wave_items_off = bytes;
     bytes += wave_n * sizeof(WaveItem);
     std::vector<unsigned char> blob(bytes ? bytes : 16, 0);
-    if (r.tiles.on) {
-        std::memcpy(blob.data() + r.tiles.units_off, r.tiles.units.data(), r.tiles.units.size() * sizeof(TileUnit));
-        std::memcpy(blob.data() + r.tiles.shifts_off, r.tiles.shifts.data(), r.tiles.shifts.size() * sizeof(TileShift));
-    }
     for (const LaunchPlan *plan : plans) {
         const LaunchPlan &L = *plan;
         if (L.words) {
@@ -439,7 +452,7 @@ int materialise(Request &r)
             r.wave_counters = need;
         }
         // a changed plan counts afresh
-        ISO_CUDA(cudaMemset(r.d_counter, 0, (size_t)r.wave_counters * sizeof(unsigned long long)));
+        ISO_CUDA(cudaMemsetAsync(r.d_counter, 0, (size_t)r.wave_counters * sizeof(unsigned long long), up));
         r.epoch = 0;
         r.wave_run = 0;
     }
@@ -464,15 +477,15 @@ int materialise(Request &r)
             for (size_t k = 0; k < r.launches.size(); ++k) ld[k] = make_launch_args(r, r.launches[k]);
         }
     }
-    ISO_CUDA(cudaMemcpy(r.d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice));
-    if (r.tiles.on) fill_tiles(r);
+    if (!up) ISO_CUDA(cudaMemcpy(r.d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+    else ISO_CUDA(cudaMemcpyAsync(r.d_blob, blob.data(), blob.size(), cudaMemcpyHostToDevice, up));
     // the error flag, only where a kernel may raise it: the vector kernels wait for nothing, and reading the
     // flag back would cost every Iso_wait a copy (8 microseconds)
     r.reports = single || wave_n > 0;
     for (const LaunchPlan *plan : plans) r.reports = r.reports || plan->kernel == KERNEL_BULK;
     if (r.reports && !r.d_err) {
         ISO_CUDA(cudaMalloc((void **)&r.d_err, sizeof(int)));
-        ISO_CUDA(cudaMemset(r.d_err, 0, sizeof(int)));
+        ISO_CUDA(cudaMemsetAsync(r.d_err, 0, sizeof(int), up));
     }
     if (r.reports && !r.h_err) {
         ISO_CUDA(cudaMallocHost((void **)&r.h_err, sizeof(int)));
@@ -488,8 +501,28 @@ int materialise(Request &r)
             devices_set.push_back(device);
         }
     }
-    r.dirty = false;
+    if (up) ISO_CUDA(cudaStreamSynchronize(up));
+    r.launches_ready = true;
     return ISO_SUCCESS;
+}
+
+// The launches of a request whose starts run in tiles: Iso_Start_host runs them slab by slab.  Its first call may be recorded into
+// a graph of the caller's, where allocating is allowed in the relaxed mode and only streams that do not take part can be waited for.
+int ensure_launches(Request &r)
+{
+    if (r.launches_ready) return ISO_SUCCESS;
+    struct Relaxed {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaStream_t own = nullptr;
+        Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+        ~Relaxed()
+        {
+            if (own) cudaStreamDestroy(own);
+            cudaThreadExchangeStreamCaptureMode(&mode);
+        }
+    } relaxed;
+    ISO_CUDA(cudaStreamCreateWithFlags(&relaxed.own, cudaStreamNonBlocking));
+    return materialise_launches(r, relaxed.own);
 }
 
 LaunchDev make_launch_args(const Request &r, const LaunchPlan &L)
@@ -936,18 +969,24 @@ cudaError_t launch_tiles_unit(const TilesPlan &F, const TilesDev &a, cudaStream_
     return F.mesh ? launch_tiles_kernel<W, true>(F, a, stream, dependent) : launch_tiles_kernel<W, false>(F, a, stream, dependent);
 }
 
-// The kernel's argument, the same for every start.
-void fill_tiles(Request &r)
+// The tables, and the kernel's argument, which is the same for every start.
+int upload_tiles(Request &r)
 {
     const Comm &c = *r.comm;
     TilesPlan &F = r.tiles;
+    const size_t units_bytes = F.units.size() * sizeof(TileUnit), shifts_bytes = F.shifts.size() * sizeof(TileShift);
+    std::vector<unsigned char> blob(units_bytes + shifts_bytes);
+    std::memcpy(blob.data(), F.units.data(), units_bytes);
+    std::memcpy(blob.data() + units_bytes, F.shifts.data(), shifts_bytes);
+    ISO_CUDA(cudaMalloc(&r.d_tiles, blob.size()));
+    ISO_CUDA(cudaMemcpy(r.d_tiles, blob.data(), blob.size(), cudaMemcpyHostToDevice));
     auto div = [](int64_t x) {
         const FastDiv f = make_fastdiv((uint32_t)x);
         return FastDivDev{f.m, f.s1, f.s2, f.div};
     };
     TilesDev a{};
-    a.units = reinterpret_cast<const TileUnit *>(static_cast<const unsigned char *>(r.d_blob) + F.units_off);
-    a.shifts = reinterpret_cast<const TileShift *>(static_cast<const unsigned char *>(r.d_blob) + F.shifts_off);
+    a.units = static_cast<const TileUnit *>(r.d_tiles);
+    a.shifts = reinterpret_cast<const TileShift *>(static_cast<const unsigned char *>(r.d_tiles) + units_bytes);
     a.n_shifts = (uint32_t)F.shifts.size();
     a.send = r.send;
     a.recv = r.recv;
@@ -993,6 +1032,7 @@ void fill_tiles(Request &r)
     }
     F.args.resize(sizeof(a));
     std::memcpy(F.args.data(), &a, sizeof(a));
+    return ISO_SUCCESS;
 }
 
 int launch_tiles(const Request &r, cudaStream_t stream, bool dependent)
@@ -2103,6 +2143,10 @@ int Iso_Start_host(Iso_request request, const void *host_sendbuf, void *host_rec
         return ISO_SUCCESS;
     }
 
+    {
+        int rc = ensure_launches(r);
+        if (rc != ISO_SUCCESS) return rc;
+    }
     // Pipelined over slabs of the leading dimension (enqueue_host_pipeline).  The same call
     // with the same host buffers is a fixed sequence of a few hundred copies, launches and
     // event operations: the first such call enqueues them one by one, the second captures

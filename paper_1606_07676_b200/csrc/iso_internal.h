@@ -220,7 +220,7 @@ struct TilesPlan {
     int64_t width = 1, intervals = 1, rows_per_tile = 0, place_stride = 0, grid = 0;
     int threads = 256, unit = 16;  // unit: bytes of every unit (0: several widths)
     bool mesh = false;
-    size_t smem = 0, units_at = 0, moved_at = 0, coords_at = 0, units_off = 0, shifts_off = 0;
+    size_t smem = 0, units_at = 0, moved_at = 0, coords_at = 0;
     std::vector<int> coords;          // dimensions whose coordinates the units look at
     std::vector<TileUnit> units;
     std::vector<TileShift> shifts;    // the first: none
@@ -279,7 +279,9 @@ struct Request {
     Iso_stats stats{};
     // device side (owned by iso_api.cu)
     bool dirty = true;
-    void *d_blob = nullptr;
+    void *d_blob = nullptr;                  // tables of the launches
+    void *d_tiles = nullptr;                 // tables of the tiles
+    bool launches_ready = false;             // the former and the intermediate buffer stand (not while nothing but starts in tiles ran)
     unsigned char *d_inter = nullptr;        // first usable byte (behind the leading guard band)
     unsigned char *d_inter_alloc = nullptr;  // the allocation: guard band, buffer, guard band
     int64_t d_inter_bytes = 0;
@@ -347,7 +349,7 @@ int lower_schedule(Request &r, uintptr_t send_addr, uintptr_t recv_addr, uintptr
 void build_words(const Request &r, LaunchPlan &L, uintptr_t send_addr, uintptr_t recv_addr, uintptr_t inter_addr);
 
 // Whether Iso_Start runs all phases of a tile of processes in one launch, and how (fills r.tiles; the launches
-// stand beside it for the host-buffer path).
+// are lowered beside it, and set up when the host-buffer path asks for them).
 void plan_tiles(Request &r);
 
 // Checks the executed parts for hazards: every range inside its buffer, no write to the send

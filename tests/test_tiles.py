@@ -162,6 +162,55 @@ def test_execution_read_back_and_tuned(monkeypatch):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("recorded", [False, True])
+def test_launches_are_set_up_when_host_buffers_need_them(recorded):
+    """A request whose starts run in tiles allocates no intermediate buffer; the host-buffer path, which runs the launches slab by
+    slab, makes up for it, in between starts and inside a graph of the caller's too."""
+    import torch
+    import oracle
+    w = wl.Workload("w", "alltoall", (32, 32, 32), wl.moore(3, 1), 64, seed=3)
+    n = w.P * w.s * 64
+    host_s = wl.payload_torch("uint8", 4, 0, n, "cuda").cpu().pin_memory()
+    host_r = torch.zeros(n, dtype=torch.uint8).pin_memory()
+    send, recv = wl.payload_torch("uint8", 3, 0, n, "cuda"), torch.empty(n, dtype=torch.uint8, device="cuda")
+    comm = iso.Iso_neighborhood_create(w.dims, w.offsets)
+    req = iso.Iso_neighbor_alltoall_init(send, 64, 1, recv, 64, 1, comm)
+    want = [oracle.alltoall(w.dims, w.offsets, 64, x.cpu().numpy().reshape(w.P, -1)).reshape(-1) for x in (send, host_s)]
+
+    def start(expect):
+        recv.fill_(POISON)
+        iso.Iso_Start(req, torch.cuda.current_stream())
+        iso.Iso_wait(req)
+        assert np.array_equal(recv.cpu().numpy(), expect) and iso.Iso_request_get_stats(req)["launches"] == 1
+
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    start(want[0])
+    assert free - torch.cuda.mem_get_info()[0] < (16 << 20)     # (the intermediate buffer has 58 MB)
+    if recorded:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            iso.Iso_Start_host(req, host_s, host_r, torch.cuda.current_stream())
+        graph.replay()
+        torch.cuda.synchronize()
+    else:
+        iso.Iso_Start_host(req, host_s, host_r, torch.cuda.current_stream())
+        iso.Iso_wait(req)
+        assert iso.Iso_request_get_host_transfer_ms(req)["slabs"] > 1
+    assert np.array_equal(host_r.numpy(), want[1])
+    start(want[1])      # (the send buffer holds what came from the host)
+    assert iso.Iso_request_check_guards(req) == 0
+    if not recorded:
+        for _ in range(3):
+            host_r.zero_()
+            iso.Iso_Start_host(req, host_s, host_r, torch.cuda.current_stream())
+            iso.Iso_wait(req)
+            assert np.array_equal(host_r.numpy(), want[1])
+    iso.Iso_request_free(req)
+    iso.Iso_comm_free(comm)
+
+
+@pytest.mark.gpu
 def test_the_benchmark_measures_the_default():
     import sys
     import torch
