@@ -25,6 +25,19 @@ def test_plans_on_the_host(tmp_path):
         assert out.returncode == 0 and int(out.stdout) > 150, out.stdout + out.stderr
 
 
+def test_no_kernel_spills(tmp_path):
+    src = tmp_path / "kernels.cu"
+    kernels = ["iso_gather_tiles<%d, %s>" % (w, mesh) for w in (0, 4, 8, 16) for mesh in ("false", "true")]
+    src.write_text('#include "iso_tiles.cuh"\nnamespace iso {\n' +
+                   "".join("template __global__ void %s(const __grid_constant__ TilesDev);\n" % k for k in kernels) + "}\n")
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    out = subprocess.run([nvcc, "-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-Xptxas", "-v", "-I", os.path.join(ROOT, "include"),
+                          "-I", CSRC, "-c", str(src), "-o", str(tmp_path / "kernels.o")], capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr
+    spills = [ln for ln in out.stderr.splitlines() if "spill stores" in ln]
+    assert len(spills) >= len(kernels) and all("0 bytes spill stores" in ln for ln in spills), out.stderr
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("m", [1, 2, 3, 4, 7, 8, 12, 13, 16, 17, 24, 33, 48, 64, 100, 256, 481])
 @pytest.mark.parametrize("call", ["alltoall", "allgather"])
