@@ -179,11 +179,12 @@ void plan_tiles(Request &r)
         bool used = false;
         for (const Part &p : r.parts) used = used || p.shift[j] != 0 || p.check[j] != 0;
         if (!used) continue;
-        if (c.dims[j] > 65535) return;  // (on a mesh coordinates are kept in 16 bits)
         F.mesh = F.mesh || !c.periodic[j];
         coord_of[j] = (int)F.coords.size();
         F.coords.push_back(j);
     }
+    for (int j : F.coords)
+        if (F.mesh && c.dims[j] > 65535) return;  // (on a mesh coordinates are kept in 16 bits)
 
     // units, in groups of one stage and one kind, of 16 bytes or of fewer
     const int send_align = std::min(alignment16(r.send_stride), alignment16((int64_t)(uintptr_t)r.send));

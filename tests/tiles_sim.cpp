@@ -120,10 +120,40 @@ Bytes by_tiles(const Request &r, const Bytes &send)
     return recv;
 }
 
+// Sides above 65 535: on a mesh, where coordinates are kept in 16 bits, they stay out of tiles.
+void long_sides()
+{
+    for (int mesh = 0; mesh < 2; ++mesh) {
+        Comm c;
+        c.d = 2;
+        c.dims[0] = 70001, c.dims[1] = 3;
+        c.P = 3 * 70001;
+        c.rank_stride[0] = 3, c.rank_stride[1] = 1;
+        c.periodic[0] = !mesh, c.periodic[1] = 1;
+        c.coords = {-1, 1, 2, 0, 1, -1};
+        Request r;
+        r.comm = &c;
+        r.s = c.s = 3;
+        r.len = {16, 16, 16};
+        r.sdispl = r.rdispl = {0, 16, 32};
+        r.send_stride = r.recv_stride = 48;
+        r.send = reinterpret_cast<const unsigned char *>((uintptr_t)4096);
+        r.recv = reinterpret_cast<unsigned char *>((uintptr_t)1 << 40);
+        r.knobs.tiles = 1;
+        require(build_schedule(r) == ISO_SUCCESS && lower_schedule(r, (uintptr_t)r.send, (uintptr_t)r.recv, 0) == ISO_SUCCESS, "schedule");
+        plan_tiles(r);
+        require(r.tiles.on == !mesh, "long sides");
+        Bytes send(c.P * r.send_stride);
+        for (size_t k = 0; k < send.size(); ++k) send[k] = (unsigned char)(k * 2654435761u >> 13);
+        if (r.tiles.on) require(by_tiles(r, send) == by_phases(r, send), "long sides, result");
+    }
+}
+
 }  // namespace
 
 int main(int argc, char **argv)
 {
+    long_sides();
     std::mt19937 rng(argc > 1 ? std::atoi(argv[1]) : 1);
     auto pick = [&](int lo, int hi) { return (int)(rng() % (unsigned)(hi - lo + 1)) + lo; };
     int compared = 0;
