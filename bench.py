@@ -42,7 +42,8 @@ HEADLINE = "cfg3_m4096"
 # the kernel sources it was taken on; an entry whose stamp is not the present sources' is
 # ignored (traffic: null)
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic.txt")
-KERNEL_SOURCES = ("iso_kernels.cuh", "iso_words.cuh", "iso_api.cu", "iso_schedule.cpp", "iso_words.cpp", "iso_internal.h")
+KERNEL_SOURCES = ("iso_kernels.cuh", "iso_words.cuh", "iso_tiles.cuh", "iso_api.cu", "iso_schedule.cpp", "iso_words.cpp", "iso_tiles.cpp",
+                  "iso_internal.h")
 
 
 def sources_hash() -> str:
@@ -649,6 +650,8 @@ def run_ours(args):
 
     # ---- roofline of the dominant kernel ----------------------------------------------
     kernel = "iso_gather_bulk" if st["bulk_bytes"] * 2 > moved else "iso_gather_rows_wide"
+    if launches == 1 and st["phases"] > 1 and not args.single_launch and not args.pipeline:
+        kernel = "iso_gather_tiles"
     rec = recorded_traffic(args.workload, args.alg) if (
         args.fusion == 1 and not args.single_launch and args.bulk_threshold is None and not args.tune
         and args.slabs is None and args.pipeline is None) else None

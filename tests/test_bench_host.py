@@ -78,3 +78,8 @@ def test_traffic_entries_are_ignored_once_the_kernels_change(tmp_path, monkeypat
     rows = [ln.split() for ln in open(bench.TRAFFIC_FILE) if ln.strip() and not ln.startswith("#")]
     assert rows and all(len(f) == 8 and int(f[2]) > 0 and float(f[3]) > 0 and len(f[6]) == 16 for f in rows)
     assert any(f[0] == bench.HEADLINE and f[1] == "combining" for f in rows)
+
+
+def test_recorded_traffic_expires_with_any_source():
+    csrc = os.path.join(ROOT, "paper_1606_07676_b200", "csrc")
+    assert sorted(bench.KERNEL_SOURCES) == sorted(os.listdir(csrc))
