@@ -2314,6 +2314,7 @@ int Iso_request_get_stats(Iso_request request, Iso_stats *out)
 {
     if (check_handle(request) || !out) return ISO_ERR_ARG;
     *out = request->stats;
+    if (!request->dirty && request->tiles.on) out->bulk_bytes = 0;
     if (!request->dirty && (request->multi_grid > 0 || request->wave_grid > 0 || request->tiles.on)) out->launches = 1;
     else if (!request->dirty && request->slab_plan.size() > 1) out->launches *= (int)request->slab_plan.size();
     return ISO_SUCCESS;

@@ -252,7 +252,8 @@ struct Knobs {
     bool coord_table = true;  // ISO_COORD_TABLE=0: row coordinates by division in every thread
     bool l2_keep = true;      // ISO_L2_KEEP=0: no eviction-priority hint on stores into the intermediate buffer
     int ag_order = -1;        // ISO_AG_ORDER=0/1: allgather visits the dimensions first-to-last / last-to-first
-    int tiles = -1;           // ISO_TILES: 0 = never all phases of a tile in one launch, 1 = wherever possible
+    int tiles = -1;           // ISO_TILES: 0 = never all phases of a tile in one launch, 1 = wherever possible, 2 and 3 = likewise, with
+                              // all blocks going through places where widths are mixed and with none
     int words = -1;           // ISO_WORDS: 0 = no launches of words, 1 = wherever they can be (-1: chosen by the library)
 };
 Knobs read_knobs();

@@ -1,9 +1,9 @@
 // Plan of the schedules whose intermediate blocks fit in shared memory: all phases of a tile of processes
 // in one launch (iso_tiles.cuh).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <list>
-#include <map>
 
 #include "iso_internal.h"
 
@@ -61,23 +61,26 @@ bool mixed_widths(const Request &r)
 }
 
 // The schedule's hops as moves between send buffers, places and receive buffers.  Places: what a phase reads, in the
-// order of the phases that write it, each where it lies in its source's 16-byte words.  False: the schedule is not
-// like that.
-bool collect_hops(const Request &r, std::vector<Hop> &hops, std::list<Part> &own, int64_t &place_stride)
+// order of the phases that write it, each where it lies in its source's 16-byte words; `staged`: what only passes from a send to
+// a receive buffer as well.  False: the schedule is not like that.
+bool collect_hops(const Request &r, bool staged, std::vector<Hop> &hops, std::list<Part> &own, int64_t &place_stride)
 {
-    // What only passes from a send to a receive buffer may go through places too: the copies to a place are asynchronous, so
-    // that the copies of several widths wait for memory once and not one after the other.  It costs places: 13-byte
-    // blocks on 257x251 57 -> 43 microseconds, irregular sizes to 24 neighbours on 18x24 7.3 -> 5.7, but, with blocks of 1 KB among
-    // them, to 26 on 27x19x31 100 -> 137.
-    const bool staged = mixed_widths(r) && r.stats.bytes_moved < 250000000;
-    using Key = std::pair<int, int64_t>;
-    std::map<Key, int64_t> read_len, place;
+    struct Read { int64_t key, len, place; };  // what a phase reads, and its place once it has one
+    std::vector<Read> reads;
+    auto key_of = [](int buf, int64_t off) { return off * 4 + buf; };
     for (const Part &p : r.parts)
-        if (p.src_buf != ISO_BUF_SEND) {
-            auto it = read_len.emplace(Key{p.src_buf, p.src_off}, p.len);
-            if (it.first->second != p.len) return false;
-        }
+        if (p.src_buf != ISO_BUF_SEND) reads.push_back(Read{key_of(p.src_buf, p.src_off), p.len, -1});
+    std::sort(reads.begin(), reads.end(), [](const Read &x, const Read &y) { return x.key != y.key ? x.key < y.key : x.len < y.len; });
+    for (size_t i = 1; i < reads.size(); ++i)
+        if (reads[i].key == reads[i - 1].key && reads[i].len != reads[i - 1].len) return false;
+    reads.erase(std::unique(reads.begin(), reads.end(), [](const Read &x, const Read &y) { return x.key == y.key; }), reads.end());
+    auto find = [&](int buf, int64_t off) -> Read * {
+        const int64_t key = key_of(buf, off);
+        auto it = std::lower_bound(reads.begin(), reads.end(), key, [](const Read &x, int64_t k) { return x.key < k; });
+        return it != reads.end() && it->key == key ? &*it : nullptr;
+    };
     std::vector<std::pair<int64_t, int64_t>> written[2];
+    hops.reserve(2 * r.parts.size());
     int64_t at = 0;
     auto new_place = [&](int64_t src_off, int64_t len) {
         const int64_t start = round16(at - (src_off & 15)) + (src_off & 15);
@@ -91,14 +94,13 @@ bool collect_hops(const Request &r, std::vector<Hop> &hops, std::list<Part> &own
             if (p.phase != last_phase) ++stage;
             last_phase = p.phase;
             h.stage = stage;
-            auto it = place.find(Key{p.src_buf, p.src_off});
-            if (it == place.end()) return false;
-            h.src_off = it->second;
+            const Read *from = find(p.src_buf, p.src_off);
+            if (from->place < 0) return false;
+            h.src_off = from->place;
         }
-        auto it = read_len.find(Key{p.dst_buf, p.dst_off});
-        if (it != read_len.end()) {
-            if (it->second != p.len) return false;
-            h.place_dst = place[Key{p.dst_buf, p.dst_off}] = new_place(h.src_off, p.len);
+        if (Read *to = find(p.dst_buf, p.dst_off)) {
+            if (to->len != p.len) return false;
+            h.place_dst = to->place = new_place(h.src_off, p.len);
         } else if (p.dst_buf == ISO_BUF_INTER) {
             return false;  // (nobody reads it)
         }
@@ -136,32 +138,25 @@ int64_t tile_threads(int64_t unit_rows, int64_t resident)
     return std::min<int64_t>(most, std::max<int64_t>(64, (unit_rows / 3 + 31) / 32 * 32));
 }
 
-}  // namespace
+// How many tiles an SM works on at a time, and in how many turns.
+struct Residency {
+    int64_t per_sm, at_once, turns;
+    Residency(int64_t tiles, int64_t smem, int64_t threads, int sm_count)
+    {
+        per_sm = (tiles + sm_count - 1) / sm_count;
+        at_once = std::max<int64_t>(1, std::min({228 * 1024 / (smem + 1024), 1024 / threads, per_sm}));
+        turns = (per_sm + at_once - 1) / at_once;
+    }
+};
 
-void plan_tiles(Request &r)
+// The plan's units, groups and tiles.  False: the schedule cannot run so.
+bool build_plan(const Request &r, bool staged, TilesPlan &F)
 {
     const Comm &c = *r.comm;
-    TilesPlan &F = r.tiles;
     F = TilesPlan{};
-    if (r.knobs.tiles == 0 || r.alg != ISO_ALG_COMBINING || r.fusion < 1 || r.layout != ISO_LAYOUT_PACKED || r.stats.phases < 2) return;
-    // (what runs as two chains of slabs, 100 MB to a launch and more, is bound by memory and keeps them)
-    if (execution_asked_for(r) || r.chains > 1) return;
-    if (r.send_stride >= (int64_t)1 << 31 || r.recv_stride >= (int64_t)1 << 31) return;
-    int64_t bytes = 0;
-    for (const Part &p : r.parts) bytes += p.len;
-    if (bytes / 16 > kTilePieces) return;
-    int64_t between = 1;  // (a first look, without the allgather's receive slots)
-    for (int j = 0; j < c.d; ++j)
-        for (const Part &p : r.parts)
-            if (p.src_buf == ISO_BUF_INTER && p.dst_buf == ISO_BUF_INTER && p.shift[j]) {
-                between *= c.dims[j];
-                break;
-            }
-    if (between * r.inter_stride > kTileSmem) return;
     std::vector<Hop> hops;
     std::list<Part> own;
-    if (!collect_hops(r, hops, own, F.place_stride)) return;
-
+    if (!collect_hops(r, staged, hops, own, F.place_stride)) return false;
     // The dimensions of the hops from place to place, and what lies between them: a tile is complete along those.
     int m0 = c.d, m1 = -1;
     for (const Hop &h : hops)
@@ -172,7 +167,7 @@ void plan_tiles(Request &r)
             }
     if (m1 < 0) m0 = 0;
     for (int j = 0; j < c.d; ++j) (j < m0 ? F.outer : (j <= m1 ? F.middle : F.inner)) *= c.dims[j];
-    if (F.middle > kTileSmem || F.middle * F.place_stride > kTileSmem) return;
+    if (F.middle > kTileSmem || F.middle * F.place_stride > kTileSmem) return false;
     int coord_of[ISO_MAX_DIMS];
     for (int j = 0; j < c.d; ++j) {
         coord_of[j] = -1;
@@ -184,16 +179,29 @@ void plan_tiles(Request &r)
         F.coords.push_back(j);
     }
     for (int j : F.coords)
-        if (F.mesh && c.dims[j] > 65535) return;  // (on a mesh coordinates are kept in 16 bits)
+        if (F.mesh && c.dims[j] > 65535) return false;  // (on a mesh coordinates are kept in 16 bits)
 
     // units, in groups of one stage and one kind, of 16 bytes or of fewer
     const int send_align = std::min(alignment16(r.send_stride), alignment16((int64_t)(uintptr_t)r.send));
     const int recv_align = std::min(alignment16(r.recv_stride), alignment16((int64_t)(uintptr_t)r.recv));
     std::vector<Piece> pieces;
-    int64_t apart = 0;  // units of a byte or two whose neighbours are wider: a sector of their own
+    pieces.reserve(512);
     F.shifts.assign(1, TileShift{});
-    auto before = [](const TileShift &x, const TileShift &y) { return std::memcmp(&x, &y, sizeof(x)) < 0; };  // (no padding)
-    std::map<TileShift, uint32_t, decltype(before)> shift_index(before);
+    size_t slots = 64;  // of a table of the shifts so far, by their bytes
+    while (slots < 2 * hops.size() + 2) slots *= 2;
+    std::vector<uint32_t> shift_at(slots, 0);
+    auto index_of = [&](const TileShift &sh) {
+        uint64_t words[sizeof(TileShift) / 8], hash = 0;  // (no padding)
+        std::memcpy(words, &sh, sizeof(sh));
+        for (uint64_t w : words) hash = (hash ^ w) * 0x9E3779B97F4A7C15ull, hash ^= hash >> 29;
+        for (size_t at = hash & (slots - 1);; at = (at + 1) & (slots - 1)) {
+            if (shift_at[at] == 0) {
+                shift_at[at] = (uint32_t)F.shifts.size();
+                F.shifts.push_back(sh);
+            }
+            if (std::memcmp(&F.shifts[shift_at[at]], &sh, sizeof(sh)) == 0) return shift_at[at];
+        }
+    };
     for (const Hop &h : hops) {
         int a = h.stage == 0 ? send_align : 16;
         if (h.place_dst >= 0) a = std::min(a, alignment16(h.src_off - h.place_dst));
@@ -222,8 +230,7 @@ void plan_tiles(Request &r)
             ++n;
         }
         sh.first_two |= (uint32_t)n | (sh.between ? 1u << 8 : 0u);
-        const uint32_t index = shift_index.emplace(sh, (uint32_t)F.shifts.size()).first->second;
-        if (index == F.shifts.size()) F.shifts.push_back(sh);
+        const uint32_t index = index_of(sh);
         for (int64_t x = 0; x < h.len;) {
             int w = a;
             while (w > 1 && (((h.src_off + x) & (w - 1)) || h.len - x < w)) w >>= 1;
@@ -236,32 +243,41 @@ void plan_tiles(Request &r)
             // (asynchronous copies move at least 4 bytes)
             pieces.push_back(Piece{h.stage, h.kind == TILE_FETCH && w < 4 ? TILE_DELIVER : h.kind, u});
             x += w;
-            apart += w < 4 && (a >= 4 || h.len < 4);
-            if ((int64_t)pieces.size() > kTilePieces) return;
+            if ((int64_t)pieces.size() > kTilePieces) return false;
         }
     }
-    std::stable_sort(pieces.begin(), pieces.end(), [](const Piece &x, const Piece &y) {
-        if (x.stage != y.stage) return x.stage < y.stage;
-        return x.kind != y.kind ? x.kind < y.kind : x.u.width > y.u.width;
-    });
     // (A group costs a quarter of a microsecond whatever is in it, so the narrow widths go together: irregular sizes to 48 neighbours on
     // 20x27 8.4 -> 6.3, the 32^3 mesh with blocks of 1024, 32 and 1 bytes 147 -> 126.)
     F.unit = pieces.empty() ? 0 : (int)pieces[0].u.width;
-    for (const Piece &q : pieces)
-        if ((int)q.u.width != F.unit || F.unit < 4) F.unit = 0;
+    int stages = 0;
     for (const Piece &q : pieces) {
-        const uint32_t width = F.unit ? (uint32_t)F.unit : (q.u.width == 16 ? 16u : 0u);
-        if (F.groups.empty() || F.groups.back().stage != (uint32_t)q.stage || F.groups.back().kind != q.kind || F.groups.back().width != width)
-            F.groups.push_back(TileGroup{q.kind, width, (uint32_t)q.stage, (uint32_t)F.units.size(), 0});
-        ++F.groups.back().n;
-        F.units.push_back(q.u);
+        if ((int)q.u.width != F.unit || F.unit < 4) F.unit = 0;
+        stages = std::max(stages, q.stage + 1);
     }
+    // sorted by stage, kind and width, the wider ones first
+    auto rank_of = [](const Piece &q) {
+        const int narrow = q.u.width == 16 ? 0 : (q.u.width == 8 ? 1 : (q.u.width == 4 ? 2 : (q.u.width == 2 ? 3 : 4)));
+        return (size_t)((q.stage * 4 + (int)q.kind) * 5 + narrow);
+    };
+    std::vector<uint32_t> first((size_t)stages * 20 + 1, 0);
+    for (const Piece &q : pieces) ++first[rank_of(q) + 1];
+    for (size_t k = 1; k < first.size(); ++k) first[k] += first[k - 1];
+    F.units.resize(pieces.size());
+    for (size_t k = 0; k + 1 < first.size(); ++k) {
+        if (first[k] == first[k + 1]) continue;
+        const uint32_t stage = (uint32_t)(k / 20), kind = (uint32_t)(k / 5 % 4);
+        const uint32_t width = F.unit ? (uint32_t)F.unit : (k % 5 == 0 ? 16u : 0u);
+        if (F.groups.empty() || F.groups.back().stage != stage || F.groups.back().kind != kind || F.groups.back().width != width)
+            F.groups.push_back(TileGroup{kind, width, stage, first[k], 0});
+        F.groups.back().n += first[k + 1] - first[k];
+    }
+    for (const Piece &q : pieces) F.units[first[rank_of(q)]++] = q.u;
     for (TileGroup &g : F.groups) {
         bool eights = g.width == 0;  // (those have code of their own: 88-byte blocks on 17x12x10x17 26 microseconds, 30 without)
         for (uint32_t u = g.first; u < g.first + g.n; ++u) eights = eights && F.units[u].width == 8;
         if (eights) g.width = 8;
     }
-    if (F.groups.empty() || (int)F.groups.size() > kTileGroups) return;
+    if (F.groups.empty() || (int)F.groups.size() > kTileGroups) return false;
 
     // The width of a tile: the one with which the SM that has the most tiles has the least to do.  A unit of a row counts
     // one, and one more per tile for its descriptor; a partner of a row more, on a mesh (with its conditions) the most.  A copy of
@@ -274,21 +290,19 @@ void plan_tiles(Request &r)
     int64_t longest = 1;
     for (const TileGroup &g : F.groups) longest = std::max<int64_t>(longest, g.n);
     double least = 0;
-    int64_t most_tiles = 0;
     for (int64_t w = 1; w <= F.inner; ++w) {
         const int64_t rows = F.middle * w, tiles = F.outer * ((F.inner + w - 1) / w);
         const int64_t smem = rows * per_row + (copied(tiles) ? table : 0) + 128;
         if (smem > (w == 1 ? kTileSmem : kTileTarget)) break;
-        const int64_t per_sm = (tiles + r.sm_count - 1) / r.sm_count, resident = std::max<int64_t>(1, 228 * 1024 / (smem + 1024));
-        const int64_t threads = tile_threads(longest * rows, resident);
-        const double warps = (double)(std::min({resident, 1024 / threads, per_sm}) * threads / 32);
-        const double cost = (double)per_sm * (double)(units * (rows + 1) + (F.mesh ? 6 : 2) * shifts * rows + 400) * (0.75 + 8.0 / warps);
+        const int64_t threads = tile_threads(longest * rows, std::max<int64_t>(1, 228 * 1024 / (smem + 1024)));
+        const Residency on(tiles, smem, threads, r.sm_count);
+        const double warps = (double)(on.at_once * threads / 32);
+        const double cost = (double)on.per_sm * (double)(units * (rows + 1) + (F.mesh ? 6 : 2) * shifts * rows + 400) * (0.75 + 8.0 / warps);
         if (least != 0 && cost >= least) continue;
         least = cost;
-        most_tiles = per_sm;
         F.width = w;
     }
-    if (least == 0) return;
+    if (least == 0) return false;
     F.intervals = (F.inner + F.width - 1) / F.width;
     F.rows_per_tile = F.middle * F.width;
     F.moved_at = (size_t)(F.rows_per_tile * F.place_stride);
@@ -301,23 +315,140 @@ void plan_tiles(Request &r)
     const int64_t resident = std::max<int64_t>(1, 228 * 1024 / ((int64_t)F.smem + 1024));
     F.threads = (int)tile_threads(longest * F.rows_per_tile, resident);
     F.grid = std::min<int64_t>(F.outer * F.intervals, std::min<int64_t>(resident, 1024 / F.threads) * r.sm_count);
+    return true;
+}
 
-    // Which is faster?  Both sides fitted to 402 calls of all sorts (2 to 5 phases, 3 to 600 microseconds; the times of either side
-    // within some 30 % of these), in microseconds.  A launch costs 2.5, and what is moved nearly the rate of a copy, less of it
-    // where blocks are not made of 16-byte units; where some go to the bulk kernel, which wants long launches, more.  A tile costs
-    // what its rows' units do, and at least what the receive buffers take at 3.6 or 3.3 TB/s (31x22x22 with 342 neighbours, allgather of
-    // 48 bytes, 71 against 60 in phases; 11x11x15x13 with 80, 152 bytes, 142 against 116).  The line lies where next to none of those calls lost: used for 260 of them, in 0.64 of
-    // the time (a quarter took less than half).
-    bool bulk = false;
-    for (const LaunchPlan &L : r.launches) bulk = bulk || L.kernel == KERNEL_BULK;
-    const double moved = (double)r.stats.bytes_moved / 6.537e6, received = (double)r.stats.bytes_min / 2.0 / (F.unit == 16 ? 3.6e6 : 3.3e6);
-    const double per_phase = 2.5 * r.stats.phases + 2.2 * (double)(r.launches.size() - r.stats.phases) + (bulk ? 4.0 - 0.6 * r.stats.phases : 0.0) +
-                             ((r.kind == ISO_KIND_ALLGATHER ? 0.84 : 0.76) + (F.unit == 16 ? 0.0 : (F.unit == 0 ? 0.4 : 0.82))) * moved;
-    // (a byte or two between wider units is a sector of its own on either side: stencil blocks of 324, 18 and 1 bytes on 43x44x39 228
-    // against 167)
-    const double work = least * (1.0 + 4.0 * (double)apart / (double)units);
-    const double in_tiles = std::max(1.3 + 0.23 * (double)F.groups.size() + 0.000215 * work + 0.3 * (double)most_tiles, received);
-    F.on = r.knobs.tiles >= 1 || in_tiles < (F.unit == 0 ? 0.75 : 0.8) * per_phase;
+// What decides between tiles and a launch per phase, in microseconds: [0] for all-to-alls, [1] for allgathers.  Fitted to
+// 8164 calls of all sorts (2 to 5 dimensions, tori and meshes, 64 to 131 072 processes, blocks of 1 to 4096 bytes) timed both ways and,
+// where blocks can be staged, all three, for the least time lost by the choice, with a loss against phases or against the choice
+// made before weighed fifteen times as much as a gain (sixty times for calls that were not in tiles before).  The estimates are within some
+// 20 %.  Of the 8164 calls 6650 run in tiles, in 0.60 of their time in phases; 62 of those lose 5 % and more, at most 1.6 (before: 5446
+// and 113, at most 2.3), and 61 calls take 5 % longer than by the choice before.  Fitted to one half, the other half loses as much.
+struct TileCosts {
+    double turn, load, move;                    // per turn of an SM: itself, a load from device and one from shared memory that others wait for
+    double unit16, unit_one, unit_mixed, partner;  // per thousand on the busiest SM: a unit of a row of 16 bytes, of one narrower width and of one among
+                                                   // several; a row's partner on a mesh
+    double table, warps;                        // per thousand: a unit descriptor that is not copied to shared memory; how much dearer all that is with one warp
+    double sector, cut, late;                   // per million: a 32-byte sector touched; of calls that receive more than 8 MB, a cut one of the receive
+                                                // buffers and any of them
+    double power;                               // of issue and memory: 1, one after the other, more, side by side
+};
+constexpr TileCosts kTileCosts[2] = {{1.68, 0.537, 0.244, 0.114, 0.009, 0.068, 0.863, 0.478, 13.5, 2.43, 3.17, 0.0, 1.04},
+                                     {1.62, 0.459, 0.114, 0.235, 0.178, 0.306, 1.43, 0.526, 3.79, 0.0, 7.68, 8.92, 8.77}};
+struct PhaseCosts {
+    double phase, launch;         // a phase, and every launch of it but one
+    double moved, bulk, mixed;    // per time of a copy: what is moved, and more where the bulk kernel does or widths are mixed
+    double block, end, end_mesh;  // per million: a block of a hop, an end of one that does not fall on 16 bytes, that on a mesh more
+    double word, word_mesh;       // per million: 4 bytes put together from words that lie otherwise, a 16-byte word on a mesh
+};
+constexpr PhaseCosts kPhaseCosts[2] = {{2.42, 6.12, 1.133, 1.413, 0.237, 1.448, 0.829, 0.997, 0.218, 0.901},
+                                       {2.52, 2.76, 0.936, 0.883, 0.008, 0.026, 0.004, 0.228, 1.103, 0.529}};
+
+// Send and receive buffers, as tiles go through them.
+double memory_time(const Request &r)
+{
+    const bool allgather = r.kind == ISO_KIND_ALLGATHER;
+    const TileCosts &k = kTileCosts[allgather];
+    const double bytes = (double)r.stats.bytes_min / 2.0, P = (double)r.comm->P;
+    double sent = 0, received = 0, cut = 0;  // sectors of a process
+    for (const Part &p : r.parts) {
+        if (p.src_buf == ISO_BUF_SEND) sent += (double)((p.src_off % 32 + p.len + 31) / 32);
+        if (p.dst_buf != ISO_BUF_RECV) continue;
+        received += (double)((p.dst_off % 32 + p.len + 31) / 32);
+        cut += (p.dst_off % 32 != 0) + ((p.dst_off + p.len) % 32 != 0);
+    }
+    if (allgather) {  // (neighbouring blocks of the own receive buffer are stored together)
+        received = bytes / 32.0 / P;
+        cut = std::min(cut, received);
+    }
+    return 1e-6 * P * (k.sector * (sent + received) + std::max(0.0, 1.0 - 8e6 / std::max(1.0, bytes)) * (k.cut * cut + k.late * received));
+}
+
+double time_in_tiles(const Request &r, const TilesPlan &F, double memory)
+{
+    const TileCosts &k = kTileCosts[r.kind == ISO_KIND_ALLGATHER];
+    const Residency on(F.outer * F.intervals, (int64_t)F.smem, F.threads, r.sm_count);
+    const double warps = (double)(on.at_once * F.threads / 32);
+    double loads = 0, moves = 0, units = 0;
+    for (const TileGroup &g : F.groups) {  // (as upload_tiles deals them to threads)
+        const int64_t passes = (g.n + F.threads - 1) / F.threads, owned = (g.n + passes - 1) / passes, slots = F.threads / owned;
+        const int64_t at_a_time = F.unit == 0 || (F.mesh && F.unit == 16) ? 2 : 4, each = (F.rows_per_tile + slots - 1) / slots;
+        const double chains = (double)(passes * ((each + at_a_time - 1) / at_a_time));
+        if (g.kind == TILE_DELIVER) loads += chains;
+        else if (g.kind != TILE_FETCH) moves += chains;
+        units += (g.width == 16 ? k.unit16 : (F.unit == 0 ? k.unit_mixed : k.unit_one)) * (double)g.n;
+    }
+    if (F.mesh) units += k.partner * (double)F.shifts.size();
+    const double latency = (double)on.turns * (k.turn + k.load * loads + k.move * moves);
+    const double table = F.units_at ? 0.0 : k.table * (double)F.units.size();
+    const double issue = 1e-3 * (double)on.per_sm * ((double)F.rows_per_tile * units + table) * (1.0 + k.warps / warps);
+    return latency + std::pow(std::pow(issue, k.power) + std::pow(memory, k.power), 1.0 / k.power);
+}
+
+double time_in_phases(const Request &r, bool mesh, bool mixed)
+{
+    const PhaseCosts &k = kPhaseCosts[r.kind == ISO_KIND_ALLGATHER];
+    const int64_t stride[3] = {r.send_stride, r.recv_stride, r.inter_stride};
+    int64_t ends = 0, put_together = 0, words = 0;
+    for (const Part &p : r.parts) {
+        ends += (p.dst_off % 16 != 0) + ((p.dst_off + p.len) % 16 != 0);
+        if (alignment16((p.src_off - p.dst_off) | stride[p.src_buf] | stride[p.dst_buf]) == 16) words += (p.dst_off % 16 + p.len + 15) / 16;
+        else put_together += (p.dst_off % 4 + p.len + 3) / 4;
+    }
+    const double P = 1e-6 * (double)r.comm->P, copy = 1.0 / 6.5e6;
+    return k.phase * r.stats.phases + k.launch * ((double)r.launches.size() - r.stats.phases) +
+           copy * ((k.moved + (mixed ? k.mixed : 0.0)) * (double)r.stats.bytes_moved + k.bulk * (double)r.stats.bulk_bytes) +
+           P * (k.block * (double)r.parts.size() + (k.end + (mesh ? k.end_mesh : 0.0)) * (double)ends + k.word * (double)put_together +
+                (mesh ? k.word_mesh * (double)words : 0.0));
+}
+
+}  // namespace
+
+void plan_tiles(Request &r)
+{
+    const Comm &c = *r.comm;
+    TilesPlan &F = r.tiles;
+    F = TilesPlan{};
+    if (r.knobs.tiles == 0 || r.alg != ISO_ALG_COMBINING || r.fusion < 1 || r.layout != ISO_LAYOUT_PACKED || r.stats.phases < 2) return;
+    // (What the library runs as two chains of slabs keeps them.  The faster way is the one or the other, in microseconds, chains and tiles:
+    // 256x256 with 24 blocks of 512 bytes 328 and 258, of 2 KB 1348 and 1526, 48^3 with 26 of 64 bytes 127 and 76, 40^3 with 7 of
+    // 500 bytes 203 and 288; the estimates below have not been fitted to such calls.)
+    if (execution_asked_for(r) || r.chains > 1) return;
+    if (r.send_stride >= (int64_t)1 << 31 || r.recv_stride >= (int64_t)1 << 31) return;
+    int64_t bytes = 0;
+    for (const Part &p : r.parts) bytes += p.len;
+    if (bytes / 16 > kTilePieces) return;
+    int64_t between = 1;  // (a first look, without the allgather's receive slots)
+    for (int j = 0; j < c.d; ++j)
+        for (const Part &p : r.parts)
+            if (p.src_buf == ISO_BUF_INTER && p.dst_buf == ISO_BUF_INTER && p.shift[j]) {
+                between *= c.dims[j];
+                break;
+            }
+    if (between * r.inter_stride > kTileSmem) return;
+    const bool forced = r.knobs.tiles >= 1;
+    bool mesh = false;
+    for (int j = 0; j < c.d; ++j) mesh = mesh || !c.periodic[j];
+    const double memory = memory_time(r);
+    // (less than any plan's estimate against more than that of the phases)
+    if (!forced && kTileCosts[r.kind == ISO_KIND_ALLGATHER].turn + memory >= time_in_phases(r, mesh, true)) return;
+    if (!build_plan(r, false, F)) return;
+    double in_tiles = time_in_tiles(r, F, memory);
+    if (mixed_widths(r)) {
+        // What only passes from a send to a receive buffer may go through places too: the copies to a place are asynchronous, so
+        // that the copies of several widths wait for memory once and not one after the other.  It costs places, and so rows per
+        // tile: irregular sizes to 45 neighbours on 40x51 19.6 -> 14.1 microseconds, 164-byte blocks of 8 on a 39x51 mesh 4.9 -> 3.7,
+        // but 41-byte blocks of 8 on 355x292 36.4 -> 50.5.  Of 3183 such calls five in six are staged; 255 would be 5 % faster the
+        // other way, 36 15 % (by the bytes of the call, as before: 675 and 198).
+        TilesPlan S;
+        double t;
+        if (r.knobs.tiles != 3 && build_plan(r, true, S) && ((t = time_in_tiles(r, S, memory)) < 1.1 * in_tiles || r.knobs.tiles == 2)) {
+            F = std::move(S);
+            in_tiles = t;
+        }
+    }
+    F.on = forced || in_tiles < time_in_phases(r, F.mesh, F.unit == 0);
+    if (!F.on) F = TilesPlan{};
 }
 
 }  // namespace iso

@@ -108,13 +108,14 @@ def test_no_schedule_writes_outside_its_buffers(torch_cuda, name):
     want = oracle_result(w, send_h)
     plans = [dict(alg=iso.ISO_ALG_COMBINING, fusion=1), dict(alg=iso.ISO_ALG_COMBINING, fusion=0),
              dict(alg=iso.ISO_ALG_COMBINING, fusion=2), dict(alg=iso.ISO_ALG_DIRECT, fusion=1),
+             dict(alg=iso.ISO_ALG_COMBINING, fusion=1, single=False), dict(alg=iso.ISO_ALG_COMBINING, fusion=2, single=False),
              dict(alg=iso.ISO_ALG_COMBINING, fusion=1, slabs=4), dict(alg=iso.ISO_ALG_COMBINING, fusion=1, slabs=8, chains=2),
              dict(alg=iso.ISO_ALG_COMBINING, fusion=1, single=True), dict(alg=iso.ISO_ALG_COMBINING, fusion=1, pipeline=3)]
     if w.collective != "allgather":
         plans.append(dict(alg=iso.ISO_ALG_TORUS, fusion=1))
     try:
         for plan in plans:
-            iso.Iso_request_set_single_launch(req, plan.get("single", False))
+            iso.Iso_request_set_single_launch(req, plan.get("single"))
             iso.Iso_request_set_pipeline(req, plan.get("pipeline", 0))
             iso.Iso_request_set_slabs(req, plan.get("slabs", 0))
             iso.Iso_request_set_chains(req, plan.get("chains", 1))

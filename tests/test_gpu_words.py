@@ -10,12 +10,18 @@ from schedule_sim import POISON, layout, make_request, oracle_result, send_buffe
 
 pytestmark = pytest.mark.gpu
 
+
+@pytest.fixture(autouse=True)
+def a_launch_per_phase(monkeypatch):
+    # the kernels of the launches per phase are what is tested here (test_tiles.py: all phases in one launch)
+    monkeypatch.setenv("ISO_TILES", "0")
+
 PLANS = ((iso.ISO_ALG_COMBINING, 1), (iso.ISO_ALG_COMBINING, 2), (iso.ISO_ALG_DIRECT, 1))
 
 
-def _compare(w, lead=(0, 0), periodic=None, slabs=0):
+def _compare(w, lead=(0, 0), periodic=None, slabs=0, tiles=False):
     """Every schedule on buffers that start `lead` bytes behind an allocation; bands around both
-    must stay as they were."""
+    must stay as they were.  `tiles`: all phases of the combining schedules have to run in one launch."""
     import torch
     lens, sd, rd, ss, rs = layout(w)
     host = send_buffer_np(w, ss)
@@ -34,6 +40,8 @@ def _compare(w, lead=(0, 0), periodic=None, slabs=0):
         recv.fill_(POISON)
         iso.Iso_Start(req, torch.cuda.current_stream())
         iso.Iso_wait(req)
+        st = iso.Iso_request_get_stats(req)
+        assert not tiles or alg != iso.ISO_ALG_COMBINING or st["launches"] == 1, (w.name, w.dims, lead, fusion, st)
         got = raw_r.cpu().numpy()
         inside = got[band + lead[1]:band + lead[1] + w.P * rs].reshape(w.P, rs)
         assert np.array_equal(inside, want), (w.name, w.dims, lead, alg, fusion, np.argwhere(inside != want)[:1])

@@ -8,21 +8,54 @@ import pytest
 
 from paper_1606_07676_b200 import binding as iso
 from paper_1606_07676_b200 import workloads as wl
-from schedule_sim import POISON
+from schedule_sim import POISON, oracle_result
 from test_gpu_fuzz import expected, make_request, random_cases
+from test_gpu_parity import Run
 from test_gpu_words import _compare
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1606_07676_b200", "csrc")
 
 
-def test_plans_on_the_host(tmp_path):
-    exe = str(tmp_path / "tiles_sim")
+@pytest.fixture(scope="module")
+def planner(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("tiles") / "tiles_sim")
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "include"), "-I", CSRC, os.path.join(ROOT, "tests", "tiles_sim.cpp")] +
                           [os.path.join(CSRC, f) for f in ("iso_schedule.cpp", "iso_words.cpp", "iso_tiles.cpp")] + ["-o", exe])
+    return exe
+
+
+def test_plans_on_the_host(planner):
     for seed in ("1", "2", "3"):
-        out = subprocess.run([exe, seed], capture_output=True, text=True, timeout=300)
+        out = subprocess.run([planner, seed], capture_output=True, text=True, timeout=300)
         assert out.returncode == 0 and int(out.stdout) > 150, out.stdout + out.stderr
+
+
+def chosen(planner, calls):
+    """Bytes of a row's places for every (kind, sides, vectors, bytes of the blocks, fusion level, periodic), 0: not in tiles."""
+    lines = []
+    for kind, dims, offs, lens, *more in calls:
+        fusion, periodic = (more + [1, None][len(more):])
+        offs = np.asarray(offs)
+        lens = np.broadcast_to(np.asarray(lens), len(offs))
+        lines.append(" ".join(str(int(x)) for x in [("alltoall", "allgather", "alltoallv").index(kind), fusion, len(dims), *dims,
+                                                    *(periodic or [1] * len(dims)), len(offs), *offs.reshape(-1), *lens]))
+    out = subprocess.run([planner, "choices"], input="\n".join(lines) + "\n", capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stdout + out.stderr
+    return [int(x) for x in out.stdout.split()]
+
+
+def test_calls_that_are_slower_in_tiles(planner):
+    # microseconds in phases and in tiles as once chosen: 97 and 228, 30 and 51, 30 and 46, 28 and 41, 21 and 27
+    assert not any(chosen(planner, [("allgather", (35, 16, 27), wl.moore(3, 3), 56), ("allgather", (24, 34, 27), wl.moore(3, 2), 24),
+                                    ("allgather", (23, 23, 24), wl.moore(3, 2), 56, 2), ("allgather", (25, 38, 23), wl.moore(3, 2), 24, 2),
+                                    ("allgather", (512, 256), wl.moore(2, 2), 16)]))
+    # blocks that need no hop stay out of the places where these are long: 39 and 21 (phases 21), 47 and 24 (28)
+    assert chosen(planner, [("alltoall", (30, 24), wl.moore(2, 3), 968), ("alltoall", (10, 9, 14), wl.moore(3, 1), 1480, 2)]) == [34896, 23744]
+    # and, in tiles: 36 and 27, 19 and 13.5, 165 and 127, 5.4 and 3.2, 98 and 65
+    faces = [32 ** max(0, 3 - int(np.abs(v).sum())) for v in wl.moore(3, 1)]
+    assert all(chosen(planner, [("alltoall", (32, 32, 32), wl.moore(3, 1), 64), ("allgather", (32, 32, 32), wl.moore(3, 1), 64),
+                                ("alltoallv", (32, 32, 32), wl.moore(3, 1), faces, 1, [0, 1, 0]), ("alltoall", (8, 8), wl.moore(2, 1), 8)]))
 
 
 def test_no_kernel_spills(tmp_path):
@@ -39,23 +72,68 @@ def test_no_kernel_spills(tmp_path):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("m", [1, 2, 3, 4, 7, 8, 12, 13, 16, 17, 24, 33, 48, 64, 100, 256, 481])
+@pytest.mark.parametrize("m", [1, 2, 3, 4, 7, 8, 12, 13, 16, 17, 24, 33, 48, 64, 100, 225, 256])
 @pytest.mark.parametrize("call", ["alltoall", "allgather"])
 def test_block_sizes(m, call, monkeypatch):
     # tiles of one row and of many, a narrower last one, several tiles to a CTA (257x131), buffers that start anywhere, meshes
     monkeypatch.setenv("ISO_TILES", "1")
     for dims, offs in (((13, 11), wl.moore(2, 2)), ((6, 5, 7), wl.moore(3, 1)), ((4, 3, 3, 5), wl.positive_octant(4, 1)), ((257, 131), wl.moore(2, 1))):
-        _compare(wl.Workload("w", call, dims, offs, m, seed=m))
-    _compare(wl.Workload("w", call, (13, 11), wl.moore(2, 1), m, seed=m + 1), lead=(m % 16, (3 * m) % 16))
-    _compare(wl.Workload("w", call, (5, 9, 4), wl.moore(3, 1), m, seed=m + 2), periodic=[0, 1, 0])
+        _compare(wl.Workload("w", call, dims, offs, m, seed=m), tiles=True)
+    _compare(wl.Workload("w", call, (13, 11), wl.moore(2, 1), m, seed=m + 1), lead=(m % 16, (3 * m) % 16), tiles=True)
+    _compare(wl.Workload("w", call, (5, 9, 4), wl.moore(3, 1), m, seed=m + 2), periodic=[0, 1, 0], tiles=True)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("tiles", ["2", "3"])
+def test_blocks_that_need_no_hop(tiles, monkeypatch):
+    # through places, to be copied on from there, and past them
+    monkeypatch.setenv("ISO_TILES", tiles)
+    for m in (1, 6, 13, 24, 41, 100):
+        _compare(wl.Workload("w", "alltoall", (13, 11), wl.moore(2, 2), m, seed=m), lead=(m % 4, 0), tiles=True)
+        _compare(wl.Workload("w", "allgather", (7, 5, 6), wl.moore(3, 1), m, seed=m), periodic=[1, 0, 1], tiles=True)
+    for seed, dims in ((1, (9, 8, 7)), (2, (31, 17))):
+        offs = wl.random_offsets(seed, len(dims), 20, -2, 2)
+        _compare(wl.Workload("v", "alltoallv", dims, offs, 0, lens=wl.random_sizes(seed, 20, choices=(1, 2, 4, 31, 64, 256)), seed=seed), tiles=True)
 
 
 @pytest.mark.gpu
 def test_rows_of_several_kilobytes(monkeypatch):
     # a table of units that stays where it is: longer than 1600 and more than two tiles to an SM
     monkeypatch.setenv("ISO_TILES", "1")
-    _compare(wl.Workload("w", "alltoall", (33, 31), wl.moore(2, 3), 784, seed=1))
-    _compare(wl.Workload("w", "allgather", (33, 31), wl.moore(2, 3), 787, seed=2))
+    _compare(wl.Workload("w", "alltoall", (33, 31), wl.moore(2, 3), 784, seed=1), tiles=True)
+    _compare(wl.Workload("w", "allgather", (133, 131), wl.moore(2, 1), 389, seed=2), tiles=True)
+
+
+@pytest.mark.gpu
+def test_long_sides(monkeypatch):
+    monkeypatch.setenv("ISO_TILES", "1")
+    _compare(wl.Workload("w", "alltoall", (70001, 3), wl.moore(2, 1), 16, seed=1), tiles=True)
+    _compare(wl.Workload("w", "allgather", (3, 70001), wl.moore(2, 1), 12, seed=2), tiles=True)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", ["cfg1", "cfg2_alltoall", "cfg2_allgather", "stencil_mesh", "irregular", "cfg3_m64"])
+def test_configurations_as_the_library_runs_them(name):
+    """Nothing asked for: the small ones and those of 32 768 processes in tiles, 65 536 processes with 24 blocks of 64 bytes as the
+    library sees fit."""
+    periodic = None
+    if name == "stencil_mesh":
+        offs = wl.moore(3, 1)
+        lens = np.asarray([32 ** max(0, 3 - int(np.abs(v).sum())) for v in offs], np.int64)
+        w, periodic = wl.Workload("v", "alltoallv", (32, 32, 32), offs, 0, lens=lens, seed=1), [0, 1, 0]
+    elif name == "irregular":
+        offs = wl.random_offsets(1, 2, 30, -3, 3)
+        w = wl.Workload("v", "alltoallv", (120, 130), offs, 0, lens=wl.random_sizes(1, 30), seed=2)
+    else:
+        w = wl.config(name)
+    import torch
+    run = Run(torch, w, periodic=periodic)
+    want = oracle_result(w, run.send_host, periodic=periodic)
+    for _ in range(2):
+        got = run.result(iso.ISO_ALG_COMBINING, 1)
+        assert np.array_equal(got, want)
+    assert name == "cfg3_m64" or iso.Iso_request_get_stats(run.req)["launches"] == 1
+    run.close()
 
 
 @pytest.mark.gpu

@@ -120,6 +120,47 @@ Bytes by_tiles(const Request &r, const Bytes &send)
     return recv;
 }
 
+// Calls read from standard input, a line each: kind, fusion level, d, the sides, whether each wraps, s, the vectors, the
+// blocks' bytes.  Prints what the library chooses: the bytes of a row's places, or 0 where it does not run in tiles.
+int choices()
+{
+    Comm c;
+    Request r;
+    while (std::scanf("%d %d %d", &r.kind, &r.fusion, &c.d) == 3) {
+        auto number = [] {
+            int x = 0;
+            require(std::scanf("%d", &x) == 1, "a number");
+            return x;
+        };
+        c.P = 1;
+        for (int j = 0; j < c.d; ++j) c.dims[j] = number();
+        for (int j = 0; j < c.d; ++j) c.periodic[j] = number();
+        for (int j = c.d - 1; j >= 0; --j) c.rank_stride[j] = c.P, c.P *= c.dims[j];
+        r.s = c.s = number();
+        for (int k = 0; k < c.s * c.d; ++k) c.coords.push_back(number());
+        int64_t at = 0;
+        for (int i = 0; i < c.s; ++i) {
+            r.len.push_back(number());
+            r.sdispl.push_back(r.kind == ISO_KIND_ALLGATHER ? 0 : at);
+            r.rdispl.push_back(at);
+            at += r.len.back();
+        }
+        if (r.kind == ISO_KIND_ALLTOALLV) at = (at + 15) / 16 * 16;
+        r.send_stride = r.kind == ISO_KIND_ALLGATHER ? r.len[0] : at;
+        r.recv_stride = at;
+        r.comm = &c;
+        r.send = reinterpret_cast<const unsigned char *>((uintptr_t)4096);
+        r.recv = reinterpret_cast<unsigned char *>((uintptr_t)1 << 40);
+        default_dimension_order(r);
+        require(build_schedule(r) == ISO_SUCCESS && lower_schedule(r, (uintptr_t)r.send, (uintptr_t)r.recv, 0) == ISO_SUCCESS, "schedule");
+        plan_tiles(r);
+        std::printf("%lld\n", r.tiles.on ? (long long)r.tiles.place_stride : 0LL);
+        c = Comm();
+        r = Request();
+    }
+    return 0;
+}
+
 // Sides above 65 535: on a mesh, where coordinates are kept in 16 bits, they stay out of tiles.
 void long_sides()
 {
@@ -153,6 +194,7 @@ void long_sides()
 
 int main(int argc, char **argv)
 {
+    if (argc > 1 && std::strcmp(argv[1], "choices") == 0) return choices();
     long_sides();
     std::mt19937 rng(argc > 1 ? std::atoi(argv[1]) : 1);
     auto pick = [&](int lo, int hi) { return (int)(rng() % (unsigned)(hi - lo + 1)) + lo; };
@@ -196,7 +238,7 @@ int main(int argc, char **argv)
         const int leads[] = {0, 0, 16, 1, 4, 8, 2};
         r.send = reinterpret_cast<const unsigned char *>((uintptr_t)4096 + leads[pick(0, 6)]);  // (only their alignment is looked at)
         r.recv = reinterpret_cast<unsigned char *>((uintptr_t)8192 + leads[pick(0, 6)]);
-        r.knobs.tiles = 1;
+        r.knobs.tiles = pick(1, 3);
         default_dimension_order(r);
         if (build_schedule(r) != ISO_SUCCESS) require(false, "schedule");
         if (lower_schedule(r, (uintptr_t)r.send, (uintptr_t)r.recv, 0) != ISO_SUCCESS) require(false, "lowering");
