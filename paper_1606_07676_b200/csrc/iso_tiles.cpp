@@ -414,6 +414,8 @@ void plan_tiles(Request &r)
     // 256x256 with 24 blocks of 512 bytes 328 and 258, of 2 KB 1348 and 1526, 48^3 with 26 of 64 bytes 127 and 76, 40^3 with 7 of
     // 500 bytes 203 and 288; the estimates below have not been fitted to such calls.)
     if (execution_asked_for(r) || r.chains > 1) return;
+    const bool long_launches = (double)r.stats.bytes_moved / 2.0 > 2.0 * kSlabLaunchBytes * (double)r.launches.size();
+    if ((r.slab_request == 1 || r.chains_request == 1) && r.kind != ISO_KIND_ALLGATHER && long_launches) return;  // (would be such a call)
     if (r.send_stride >= (int64_t)1 << 31 || r.recv_stride >= (int64_t)1 << 31) return;
     int64_t bytes = 0;
     for (const Part &p : r.parts) bytes += p.len;

@@ -11,10 +11,10 @@
 //
 // What bounds it.  Small calls: the latency of one chain of a global load, a shared-memory hop per phase and a
 // global store, about a microsecond beside the launch, where a launch per phase costs 2.6 microseconds each
-// (8^2 with 8-byte blocks 5.3 -> 3.1, 11x9x8 with 30 4-byte blocks 6.9 -> 3.4, 16x20x18 allgather of 44 bytes 9.3 ->
-// 3.5).  Large ones: the instructions per unit and row, a third of the issue slots, with half of the warps waiting for
-// memory or a barrier (32^3 with 26 64-byte blocks 35 -> 27, DRAM traffic 174 -> 65 MB during the kernel; allgather there
-// 16.5 -> 12.6; 67x57x65 with 24 8-byte blocks 113 -> 50).  Why a thread owns a unit position and the partners of the
+// (8^2 with 8-byte blocks 5.2 -> 3.1, 11x9x8 with 30 4-byte blocks 7.1 -> 3.1, 20x27 with 48 irregular ones 8.3 ->
+// 6.8).  Large ones: the instructions per unit and row, 1.5 of four a cycle, with 0.42 of the warps there and most of them waiting for
+// memory, shared memory or a barrier (32^3 with 26 64-byte blocks 35.8 -> 27.1, DRAM traffic 174 -> 65 MB during the kernel; allgather there
+// 19.0 -> 13.5; 17x12x10x17 with 15 88-byte blocks 82 -> 34).  Why a thread owns a unit position and the partners of the
 // rows are tabulated: with a division per row and dimension and a wrap test per unit and row the
 // same 32^3 took 73, with coordinates in a table 30.  Clusters that share a tile (distributed shared memory) were
 // slower than a launch per phase: 64x64x32 with 30 irregular blocks 2750 against 1300.

@@ -105,6 +105,27 @@ def test_rows_of_several_kilobytes(monkeypatch):
 
 
 @pytest.mark.gpu
+def test_buffers_of_more_than_four_gigabytes(monkeypatch):
+    import oracle
+    import torch
+    monkeypatch.setenv("ISO_TILES", "1")
+    dims, offs, m = (512, 257), wl.moore(2, 1), 4160       # 4.4 GB received
+    P, s = 512 * 257, len(offs)
+    send = wl.payload_torch("uint8", 9, 0, P * m, "cuda")
+    recv = torch.full((P, s * m), POISON, dtype=torch.uint8, device="cuda")
+    comm = iso.Iso_neighborhood_create(dims, offs)
+    req = iso.Iso_neighbor_allgather_init(send, m, 1, recv, m, 1, comm)
+    iso.Iso_Start(req, torch.cuda.current_stream())
+    iso.Iso_wait(req)
+    assert iso.Iso_request_get_stats(req)["launches"] == 1 and recv.numel() > 1 << 32
+    host = send.cpu().numpy()
+    for r0 in (0, P // 3, int((1 << 31) // (s * m)) - 5, int((1 << 32) // (s * m)) - 5, P - 300):
+        assert np.array_equal(recv[r0:r0 + 300].cpu().numpy(), oracle.allgather(dims, offs, m, host, r0, r0 + 300)), r0
+    iso.Iso_request_free(req)
+    iso.Iso_comm_free(comm)
+
+
+@pytest.mark.gpu
 def test_long_sides(monkeypatch):
     monkeypatch.setenv("ISO_TILES", "1")
     _compare(wl.Workload("w", "alltoall", (70001, 3), wl.moore(2, 1), 16, seed=1), tiles=True)
@@ -245,10 +266,13 @@ def test_execution_read_back_and_tuned(monkeypatch):
     assert launches(one[2]) == 1
     iso.Iso_request_set_slabs(two[2], 2)
     assert launches(two[2]) == 6
+    large = bound(wl.Workload("w", "alltoall", (128, 128), wl.moore(2, 2), 1024, seed=4))
+    iso.Iso_request_set_slabs(large[2], 1)      # (in two chains of slabs otherwise)
+    assert launches(large[2]) == 2
     monkeypatch.setenv("ISO_TILES", "1")
     many = bound(wl.Workload("w", "alltoall", (256, 256), wl.moore(2, 2), 64, seed=4))  # (two slabs, were it run in phases)
     assert launches(many[2]) == 1 and iso.Iso_request_get_execution(many[2]) == ex
-    for b in (one, two, many):
+    for b in (one, two, large, many):
         iso.Iso_request_free(b[2])
 
 
