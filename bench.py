@@ -10,7 +10,8 @@ repeated runs of K steps; the same line carries the payload rate, the roofline f
 the dominant kernel with its DRAM traffic, the end-to-end rate with host buffers, the CPU
 oracle timed on the host cores, and a table (`detail.configs`) with every configuration
 under the combining, the direct and the hop-by-hop schedule, each checked against the
-oracle on sampled ranks after it was timed.
+oracle on sampled ranks after it was timed.  The table on that line is cut to its key figures, so that the
+line stays short (20 KB of it did not survive every reader); the whole table goes to the error output.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME] [--sweep paper]
     python bench.py --impl reference ...      # times the CPU oracle instead
@@ -770,12 +771,27 @@ def run_ours(args):
         del reps, b
         torch.cuda.empty_cache()
     line["clocks"] = clocks
-    line["detail"] = detail
+    line["detail"] = compact(detail)
     if rank == 0:
+        print(json.dumps({"detail": detail}), file=sys.stderr)
         print(json.dumps(line))
     if dist is not None:
         dist.destroy_process_group()
     return 0
+
+
+ROW_KEYS = ("ms", "rounds", "launches", "gbs_moved", "gbs_payload", "frac_of_measured", "parity_checked")
+
+
+def compact(x):
+    """`x` with the key figures of every row of a table, numbers to four digits."""
+    if isinstance(x, dict):
+        if "gbs_moved" in x and "launches" in x and "bytes_min" in x and "ms" in x:
+            x = {k: v for k, v in x.items() if k in ROW_KEYS}
+        return {k: compact(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [compact(v) for v in x]
+    return float("%.4g" % x) if isinstance(x, float) else x
 
 
 def sweep(torch, iso, wl, peak, args):

@@ -83,3 +83,16 @@ def test_traffic_entries_are_ignored_once_the_kernels_change(tmp_path, monkeypat
 def test_recorded_traffic_expires_with_any_source():
     csrc = os.path.join(ROOT, "paper_1606_07676_b200", "csrc")
     assert sorted(bench.KERNEL_SOURCES) == sorted(os.listdir(csrc))
+
+
+def test_the_line_stays_short():
+    """A run with the table of configurations prints a few kilobytes: key figures of every row, four digits."""
+    import json
+    times = [0.027204175, 0.027157741, 0.027248523]
+    st = dict(rounds=6, launches=1, bytes_moved=226492416, bytes_min=109051904)
+    full = dict(bench.row(st, times, 6448.4, True), steps_per_run=705, replicas=5, execution={"slabs": 1, "chains": 1, "graph": 0})
+    detail = {"headline": {"rounds": 6, "bytes_moved": 226492416}, "configs": {"c%d" % k: {key: full for key, *_ in bench.SCHEDULES} for k in range(9)}}
+    short = bench.compact(detail)
+    row = short["configs"]["c3"]["combining"]
+    assert row == {"ms": 0.0272, "rounds": 6, "launches": 1, "gbs_moved": 8326.0, "gbs_payload": 4009.0, "frac_of_measured": 1.291, "parity_checked": True}
+    assert short["headline"] == detail["headline"] and len(json.dumps(short)) < 6000 < len(json.dumps(detail))
