@@ -355,7 +355,8 @@ class Bound:
         """Selects the schedule; `execution` (slabs, chains, graph) copies another instance's
         tuned choice instead of tuning again."""
         iso = self.iso
-        iso.Iso_request_set_single_launch(self.req, Bound.single_launch)
+        # (a plan tuned to one launch per phase in one slab reads back like one in tiles: the number of launches tells)
+        iso.Iso_request_set_single_launch(self.req, Bound.single_launch if execution is None else execution["single"])
         iso.Iso_request_set_algorithm(self.req, alg, fusion)
         if Bound.bulk_threshold is not None:
             iso.Iso_request_set_bulk_threshold(self.req, Bound.bulk_threshold)
@@ -465,7 +466,7 @@ class Replicas:
 
     def set(self, alg, fusion):
         st = self.items[0].set(alg, fusion)
-        ex = self.items[0].execution() if Bound.tune else None
+        ex = dict(self.items[0].execution(), single=False if st["launches"] > 1 else Bound.single_launch) if Bound.tune else None
         for b in self.items[1:]:
             b.set(alg, fusion, ex)
         return st

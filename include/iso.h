@@ -336,7 +336,8 @@ int Iso_request_tune(Iso_request request, void *cuda_stream, int flags);
 
 /* What Iso_Start does at present: slabs (1: none), chains (1: none), graph replay (0/1).
  * Before the first Iso_Start after a change these are the values asked for (slabs 0:
- * automatic); any of the pointers may be NULL. */
+ * automatic); any of the pointers may be NULL.  All phases in tiles and one launch per phase
+ * in one slab read alike; Iso_request_get_stats's number of launches tells them apart. */
 int Iso_request_get_execution(Iso_request request, int *slabs, int *chains, int *graph);
 
 /*
